@@ -14,13 +14,16 @@
 // the storage dtype. DARE's mask of expert j is the library's Mask stream
 // with step = j.
 //
-// TIES trim threshold of each (tensor, expert): the r-th largest key of
+// TIES trim threshold of each (tensor, expert) slot: the r-th largest key of
 // |Delta_j| (key = the bits of the magnitude as uint32, r = ceil(retention
-// n)), found by a most-significant-digit radix select in three passes of 11,
-// 11 and 10 bits: each pass histograms the digit of the keys that match the
-// digits decided so far (shared-memory histograms per chunk, flushed into
-// 64-bit global bins), then one CTA per (tensor, expert) picks the digit
-// whose bin holds the r-th largest and the rank within it.
+// n)), selected exactly. A sample of the slot's keys gives an interval that
+// holds the threshold almost surely (small tensors are sampled whole, which
+// decides them); a pass over the inputs then counts the keys in 2046 equal
+// bins of that interval and in one bin below and one above it, and one CTA
+// per slot picks the bin that holds the r-th largest. A bin of one key, or
+// one all of whose keys are its first (bf16 differences lie on coarse grids),
+// is the threshold; any other bin, also the two outer ones when the sample
+// missed, is the next pass's interval. Passes skip decided slots.
 
 #include <cmath>
 #include <cstdarg>
@@ -37,10 +40,13 @@ namespace {
 
 constexpr int kMergeMaxExperts = SMAT_MERGE_MAX_EXPERTS;
 constexpr int64_t kMergeChunk = int64_t(1) << 16;
-constexpr int kHistBins = 2048;
-constexpr int kPasses = 3;
-constexpr int kPassShift[kPasses] = {21, 10, 0};
-constexpr int kPassWidth[kPasses] = {11, 11, 10};
+constexpr int kHistBins = 2048;  // an interval's 2046 bins, one below it and one above it
+constexpr int kInner = kHistBins - 2;
+// Passes over the inputs: one or two when the sample's interval holds the
+// threshold; a miss costs one pass and leaves fewer than 2046 2^20 keys, which
+// three more decide (bins of at most 2^20, 2^10 and 1 keys).
+constexpr int kPasses = 4;
+constexpr uint32_t kInfKey = 0x7F800000u;
 constexpr size_t kMergeAlign = 256;
 
 struct MTensor {
@@ -52,21 +58,28 @@ struct MTensor {
   int32_t dtype, pad;
 };
 
+// Threshold selection of one (tensor, expert) slot.
+struct TiesSlot {  // 16 bytes
+  uint32_t lo;     // first key of the interval, a multiple of 2^shift
+  int32_t shift;   // its bins hold 2^shift keys each
+  uint32_t done;   // the threshold is decided
+  uint32_t pad;
+};
+
 struct MArgs {
   const MTensor* tensors;
   const Chunk* chunks;
   const void* const* experts;  // [tensor * K + e]
   uint32_t* thr;               // [tensor * K + e] TIES threshold keys
-  uint32_t* prefix;            // radix select: the digits decided so far
-  int64_t* rank;               // radix select: rank among keys with that prefix (1 = largest)
-  unsigned long long* hist;    // [(tensor * K + e) * kHistBins]
+  TiesSlot* slots;             // [tensor * K + e]
+  int64_t* rank;               // r of each slot (1 = the largest key)
+  uint32_t* n_done;            // slots decided so far
+  unsigned long long* hist;    // [(tensor * K + e) * kHistBins]; bit 63: some key is not its bin's first
   int64_t n_chunks;
   RoundKeys key;
   int32_t K, method;
   float gamma, c;              // c: per-expert coefficient (WA 1/K, TA gamma, DARE gamma / p_keep)
-  int32_t shift, width;        // current radix pass
-  uint32_t decided;            // mask of the key bits decided before this pass
-  int32_t last_pass;
+  int32_t n_slots;
 };
 
 __device__ __forceinline__ uint32_t abs_key(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
@@ -343,7 +356,6 @@ __device__ __forceinline__ void merge_ties16(const MArgs& m, const MTensor& T, i
   uint32_t cnt[4] = {0u, 0u, 0u, 0u};  // four 8-bit counts per word (K <= 16)
 #pragma unroll
   for (int k = 0; k < 16; ++k) part[k] = 0.0f;
-  constexpr uint32_t kInfKey = 0x7F800000u;
   auto agree = [&](float d, uint32_t lo, int k) {
     const uint32_t key = abs_key(d);
     return key >= lo && key <= kInfKey && ((__float_as_uint(d) ^ __float_as_uint(sum[k])) & 0x80000000u) == 0u;
@@ -482,98 +494,35 @@ __global__ void __launch_bounds__(kBlock, 2) dare_kernel(const __grid_constant__
   }
 }
 
-// One radix pass of the TIES threshold selection. A work item is a chunk
-// and up to kHistExperts of its experts: theta0 is read once for them, and
-// each thread has theta0's and every expert's 32-byte load in flight at once;
-// one shared-memory histogram per expert, flushed into the 64-bit global bins.
-constexpr int kHistExperts = 4;
+// --------------------------------------------------- TIES threshold selection ---
+// Elements sampled per slot, as 16-element groups spread evenly over the
+// tensor; a tensor of at most this many elements is read whole.
+constexpr int kSampleElems = 1 << 16;
 
-// The key is abs(Delta)'s bits: its sign bit is 0, so the prefix test and
-// the digit are taken on Delta's raw bits with bit 31 masked out of both
-// (one operation per key fewer). FIRST: the first pass, where no digit is
-// decided yet and every key counts.
-template <int DT, bool FIRST>
-__global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 1) ties_hist_kernel(const __grid_constant__ MArgs m) {
-  __shared__ uint32_t h[kHistExperts * kHistBins];
-  const int nbat = (m.K + kHistExperts - 1) / kHistExperts;
-  const int64_t items = m.n_chunks * nbat;
-  const uint32_t digit = ((1u << m.width) - 1u) & (0x7FFFFFFFu >> m.shift);
-  const uint32_t dm = m.decided & 0x7FFFFFFFu;
-  for (int64_t w = blockIdx.x; w < items; w += gridDim.x) {
-    const int64_t ci = w / nbat;
-    const int e0 = (int)(w % nbat) * kHistExperts;
-    const int ne = m.K - e0 < kHistExperts ? m.K - e0 : kHistExperts;
-    const Chunk ch = m.chunks[ci];
-    const MTensor& T = m.tensors[ch.tensor];
-    const int slot0 = ch.tensor * m.K + e0;
-    for (int b = threadIdx.x; b < kHistExperts * kHistBins; b += kBlock) h[b] = 0u;
-    __syncthreads();
-    uint32_t P[kHistExperts];
-    const void* xp[kHistExperts];
-#pragma unroll
-    for (int b = 0; b < kHistExperts; ++b) {
-      P[b] = b < ne ? m.prefix[slot0 + b] : 0u;
-      xp[b] = b < ne ? m.experts[slot0 + b] : nullptr;
-    }
-    const bool vec = (T.flags & TF_VEC) != 0u;
-    for (int64_t i = ch.begin + 16 * (int64_t)threadIdx.x; i < ch.end; i += 16 * (int64_t)kBlock) {
-      if (vec && i + 16 <= ch.end) {
-        Raw16<DT> t0, x[kHistExperts];
-        load16<DT>(T.theta0, i, t0);
-#pragma unroll
-        for (int b = 0; b < kHistExperts; ++b)
-          if (b < ne) load16<DT>(xp[b], i, x[b]);
-#pragma unroll
-        for (int b = 0; b < kHistExperts; ++b) {
-          if (b < ne) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const float2 d = sub2_rn(x[b].pair(q), t0.pair(q));
-              const uint32_t k0 = __float_as_uint(d.x), k1 = __float_as_uint(d.y);
-              if (FIRST || (k0 & dm) == P[b]) atomicAdd(&h[b * kHistBins + ((k0 >> m.shift) & digit)], 1u);
-              if (FIRST || (k1 & dm) == P[b]) atomicAdd(&h[b * kHistBins + ((k1 >> m.shift) & digit)], 1u);
-            }
-          }
-        }
-      } else {
-        const int64_t e_end = (i + 16 < ch.end) ? i + 16 : ch.end;
-        for (int64_t k = i; k < e_end; ++k) {
-          const float t0 = load1<DT>(T.theta0, k);
-          for (int b = 0; b < ne; ++b) {
-            const uint32_t key = abs_key(__fsub_rn(load1<DT>(xp[b], k), t0));
-            if ((key & m.decided) == P[b]) atomicAdd(&h[b * kHistBins + ((key >> m.shift) & digit)], 1u);
-          }
-        }
-      }
-    }
-    __syncthreads();
-    // the ne histograms are consecutive slots' bins in the global array
-    unsigned long long* gh = m.hist + (size_t)slot0 * kHistBins;
-    for (int b = threadIdx.x; b < ne * kHistBins; b += kBlock)
-      if (h[b]) atomicAdd(gh + b, (unsigned long long)h[b]);
-    __syncthreads();
-  }
+// The interval [lo, lo + width) as the slot's next one: the smallest shift
+// whose 2046 bins cover it from a multiple of 2^shift.
+__device__ __forceinline__ void set_interval(TiesSlot& S, uint32_t lo, uint64_t width) {
+  int s = 0;
+  while ((uint64_t(kInner) << s) < width + (lo & ((1u << s) - 1u))) ++s;
+  S.lo = lo & ~((1u << s) - 1u);
+  S.shift = s;
 }
 
-// After a pass: one CTA per (tensor, expert) picks the digit whose bin holds
-// the rank-th largest key (bins scanned from the top), records it and the
-// rank within that bin, and clears the histogram for the next pass.
-__global__ void __launch_bounds__(kBlock) ties_select_kernel(const __grid_constant__ MArgs m) {
-  __shared__ unsigned long long s_sum[kBlock];
-  __shared__ int s_digit;
-  __shared__ long long s_above;
-  const int slot = blockIdx.x;
-  unsigned long long* gh = m.hist + (size_t)slot * kHistBins;
-  const long long r = m.rank[slot];
-  const int nb = 1 << m.width;
+// The bin that holds the r-th entry counted from the top of a histogram of nb
+// bins (counts: bits 0 to 62) and the entries above that bin, by all threads
+// of the CTA; digit -1 if there are fewer than r.
+template <typename Count>
+__device__ __forceinline__ void select_from_top(const Count* hist, int nb, long long r, unsigned long long* s_sum,
+                                                int* s_digit, long long* s_above) {
+  constexpr unsigned long long kCount = ~0ull >> 1;
   const int per = nb / kBlock;  // bins per thread, highest bins in thread 0
   unsigned long long local = 0;
   const int top = nb - 1 - threadIdx.x * per;
-  for (int k = 0; k < per; ++k) local += gh[top - k];
+  for (int k = 0; k < per; ++k) local += hist[top - k] & kCount;
   s_sum[threadIdx.x] = local;
   if (threadIdx.x == 0) {
-    s_digit = -1;
-    s_above = 0;
+    *s_digit = -1;
+    *s_above = 0;
   }
   __syncthreads();
   // inclusive scan from the top (Hillis-Steele; 8 steps over 256 entries)
@@ -588,22 +537,269 @@ __global__ void __launch_bounds__(kBlock) ties_select_kernel(const __grid_consta
   if (r > 0 && (long long)excl < r && r <= (long long)incl) {
     unsigned long long acc = excl;
     for (int k = 0; k < per; ++k) {
-      const unsigned long long c = gh[top - k];
+      const unsigned long long c = hist[top - k] & kCount;
       if ((long long)(acc + c) >= r) {
-        s_digit = top - k;
-        s_above = (long long)acc;
+        *s_digit = top - k;
+        *s_above = (long long)acc;
         break;
       }
       acc += c;
     }
   }
   __syncthreads();
-  if (threadIdx.x == 0 && r > 0 && s_digit >= 0) {
-    const uint32_t p = m.prefix[slot] | ((uint32_t)s_digit << m.shift);
-    m.prefix[slot] = p;
-    m.rank[slot] = r - s_above;
-    if (m.last_pass) m.thr[slot] = p;
+}
+
+// The first interval of each slot, one CTA per slot: two order statistics of
+// the sample, eight standard deviations of the sampled rank to either side of
+// r's share, each by a radix select of three digits (11, 11 and 10 bits). The
+// three readings of the sample (2 x 128 KB for bf16) come from L2 after the first.
+template <int DT>
+__global__ void __launch_bounds__(kBlock) ties_sample_kernel(const __grid_constant__ MArgs m) {
+  __shared__ uint32_t h[2][kHistBins];
+  __shared__ unsigned long long s_sum[kBlock];
+  __shared__ int s_digit;
+  __shared__ long long s_above;
+  const int slot = blockIdx.x;
+  const MTensor& T = m.tensors[slot / m.K];
+  const void* x = m.experts[slot];
+  const int64_t n = T.numel, r = m.rank[slot];
+  if (n <= 0) {
+    if (threadIdx.x == 0) {
+      m.slots[slot].done = 1u;
+      atomicAdd(m.n_done, 1u);
+    }
+    return;
   }
+  const bool all = n <= kSampleElems, vec = (T.flags & TF_VEC) != 0u;
+  const int groups = all ? (int)((n + 15) / 16) : kSampleElems / 16;
+  const int64_t seen = all ? n : kSampleElems;
+  // ranks in the sample, counted from the largest key: the upper end of the
+  // interval and the lower one
+  long long rank[2] = {r, r};
+  if (!all) {
+    const double p = (double)r / (double)n, at = p * (double)seen;
+    const double d = 8.0 * sqrt(at * (1.0 - p)) + 32.0;
+    rank[0] = (long long)ceil(at - d);
+    rank[1] = (long long)floor(at + d);
+  }
+  const bool open_top = rank[0] < 1, open_bottom = rank[1] > seen;
+  if (open_top) rank[0] = 1;
+  if (open_bottom) rank[1] = seen;
+  uint32_t prefix[2] = {0u, 0u};
+  const int shifts[3] = {21, 10, 0}, widths[3] = {11, 11, 10};
+#pragma unroll 1
+  for (int pass = 0; pass < 3; ++pass) {
+    const int shift = shifts[pass], nb = 1 << widths[pass];
+    const uint32_t decided = pass == 0 ? 0u : ~0u << shifts[pass - 1];
+    const bool same = prefix[0] == prefix[1];
+    for (int b = threadIdx.x; b < 2 * kHistBins; b += kBlock) (&h[0][0])[b] = 0u;
+    __syncthreads();
+    auto count = [&](uint32_t key) {
+      const uint32_t digit = (key >> shift) & (uint32_t)(nb - 1);
+      if ((key & decided) == prefix[0]) atomicAdd(&h[0][digit], 1u);
+      if (!same && (key & decided) == prefix[1]) atomicAdd(&h[1][digit], 1u);
+    };
+    for (int g = threadIdx.x; g < groups; g += kBlock) {
+      const int64_t i = 16 * (all ? (int64_t)g : (int64_t)g * (n / 16) / groups);
+      if (vec && i + 16 <= n) {
+        Raw16<DT> t0, y;
+        load16<DT>(T.theta0, i, t0);
+        load16<DT>(x, i, y);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const float2 d = sub2_rn(y.pair(q), t0.pair(q));
+          count(abs_key(d.x));
+          count(abs_key(d.y));
+        }
+      } else {
+        for (int64_t k = i; k < n && k < i + 16; ++k) count(abs_key(__fsub_rn(load1<DT>(x, k), load1<DT>(T.theta0, k))));
+      }
+    }
+    __syncthreads();
+    for (int q = 0; q < 2; ++q) {
+      select_from_top(h[same ? 0 : q], nb, rank[q], s_sum, &s_digit, &s_above);
+      prefix[q] |= (uint32_t)s_digit << shift;
+      rank[q] -= s_above;
+      __syncthreads();
+    }
+  }
+  if (threadIdx.x == 0) {
+    TiesSlot S;
+    S.done = all ? 1u : 0u;
+    S.pad = 0u;
+    const uint32_t lo = open_bottom ? 0u : prefix[1];
+    const uint32_t hi = open_top ? 0x7FFFFFFFu : prefix[0];
+    set_interval(S, lo, (uint64_t)hi - lo + 1);
+    m.slots[slot] = S;
+    if (all) {
+      m.thr[slot] = prefix[0];
+      atomicAdd(m.n_done, 1u);
+    }
+  }
+}
+
+// One pass of the selection. A work item is a chunk and up to kHistExperts of
+// its experts: theta0 is read once for them, and each thread has theta0's and
+// every expert's 32-byte load in flight at once; one shared-memory histogram
+// per expert, flushed into the 64-bit global bins.
+//
+// Every key counts (the outer bins take what lies outside the interval), so
+// that no branch surrounds the shared-memory atomic: a pass that tested each
+// key against the digits decided so far and branched around the atomic took
+// twice as long at the same traffic (5.7 against 2.9 ms for 8 experts of 1.07e9
+// bf16 elements), bound by issue slots instead of HBM.
+constexpr int kHistExperts = 4;
+constexpr uint32_t kOffFirst = 0x80000000u;  // shared bins: some key is not its bin's first
+
+template <int DT>
+__global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 1) ties_hist_kernel(const __grid_constant__ MArgs m) {
+  __shared__ uint32_t h[kHistExperts * kHistBins];
+  if (*m.n_done == (uint32_t)m.n_slots) return;
+  const int nbat = (m.K + kHistExperts - 1) / kHistExperts;
+  const int64_t items = m.n_chunks * nbat;
+  for (int64_t w = blockIdx.x; w < items; w += gridDim.x) {
+    const int64_t ci = w / nbat;
+    const int e0 = (int)(w % nbat) * kHistExperts;
+    const int ne = m.K - e0 < kHistExperts ? m.K - e0 : kHistExperts;
+    const Chunk ch = m.chunks[ci];
+    const MTensor& T = m.tensors[ch.tensor];
+    const int slot0 = ch.tensor * m.K + e0;
+    uint32_t lo[kHistExperts];
+    int sh[kHistExperts];
+    const void* xp[kHistExperts];
+    bool any = false;
+#pragma unroll
+    for (int b = 0; b < kHistExperts; ++b) {
+      xp[b] = nullptr;
+      lo[b] = 0u;
+      sh[b] = 0;
+      if (b < ne) {
+        const TiesSlot S = m.slots[slot0 + b];
+        if (!S.done) {  // a decided expert is not read again
+          any = true;
+          xp[b] = m.experts[slot0 + b];
+          lo[b] = S.lo;
+          sh[b] = S.shift;
+        }
+      }
+    }
+    if (!any) continue;  // the same slots in every thread
+    for (int b = threadIdx.x; b < kHistExperts * kHistBins; b += kBlock) h[b] = 0u;
+    __syncthreads();
+    // bin of a key: 1 + (key - lo) / 2^shift, clamped to [0, 2047]
+    auto bin = [&](uint32_t key, int b) {
+      return __viaddmin_s32_relu((int)(key - lo[b]) >> sh[b], 1, kHistBins - 1);
+    };
+    auto mark = [&](uint32_t key, int b) {  // bf16: a key that is not its bin's first
+      const int j = bin(key, b);
+      if ((key & ((1u << sh[b]) - 1u)) != 0u && j > 0 && j < kHistBins - 1) atomicOr(&h[b * kHistBins + j], kOffFirst);
+    };
+    const bool vec = (T.flags & TF_VEC) != 0u;
+    for (int64_t i = ch.begin + 16 * (int64_t)threadIdx.x; i < ch.end; i += 16 * (int64_t)kBlock) {
+      if (vec && i + 16 <= ch.end) {
+        Raw16<DT> t0, x[kHistExperts];
+        load16<DT>(T.theta0, i, t0);
+#pragma unroll
+        for (int b = 0; b < kHistExperts; ++b)
+          if (xp[b]) load16<DT>(xp[b], i, x[b]);
+        uint32_t off = 0u;  // bf16: experts with a key that is not a multiple of 2^shift
+#pragma unroll
+        for (int b = 0; b < kHistExperts; ++b) {
+          if (xp[b]) {
+            uint32_t bits = 0u;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              const float2 d = sub2_rn(x[b].pair(q), t0.pair(q));
+              const uint32_t k0 = abs_key(d.x), k1 = abs_key(d.y);
+              bits |= k0 | k1;
+              atomicAdd(&h[b * kHistBins + bin(k0, b)], 1u);
+              atomicAdd(&h[b * kHistBins + bin(k1, b)], 1u);
+            }
+            if (DT == DT_BF16 && (bits & ((1u << sh[b]) - 1u)) != 0u) off |= 1u << b;
+          }
+        }
+        if (DT == DT_BF16 && off) {  // rare: the group again for its experts with such a key
+#pragma unroll
+          for (int b = 0; b < kHistExperts; ++b) {
+            if ((off >> b) & 1u) {
+              Raw16<DT> u0, y;
+              load16<DT>(T.theta0, i, u0);
+              load16<DT>(xp[b], i, y);
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                const float2 d = sub2_rn(y.pair(q), u0.pair(q));
+                mark(abs_key(d.x), b);
+                mark(abs_key(d.y), b);
+              }
+            }
+          }
+        }
+      } else {
+        const int64_t e_end = (i + 16 < ch.end) ? i + 16 : ch.end;
+        for (int64_t k = i; k < e_end; ++k) {
+          const float t0 = load1<DT>(T.theta0, k);
+#pragma unroll
+          for (int b = 0; b < kHistExperts; ++b) {
+            if (xp[b]) {
+              const uint32_t key = abs_key(__fsub_rn(load1<DT>(xp[b], k), t0));
+              atomicAdd(&h[b * kHistBins + bin(key, b)], 1u);
+              if (DT == DT_BF16) mark(key, b);
+            }
+          }
+        }
+      }
+    }
+    __syncthreads();
+    // the ne histograms are consecutive slots' bins in the global array
+    unsigned long long* gh = m.hist + (size_t)slot0 * kHistBins;
+    for (int b = threadIdx.x; b < ne * kHistBins; b += kBlock) {
+      const uint32_t c = h[b];
+      if (c) {
+        atomicAdd(gh + b, (unsigned long long)(c & ~kOffFirst));
+        if (c & kOffFirst) atomicOr(gh + b, 1ull << 63);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// After a pass: one CTA per slot picks the bin that holds the r-th largest
+// key, and either decides the threshold or sets the next pass's interval and
+// clears the histogram.
+template <int DT>
+__global__ void __launch_bounds__(kBlock) ties_select_kernel(const __grid_constant__ MArgs m) {
+  __shared__ unsigned long long s_sum[kBlock];
+  __shared__ int s_digit;
+  __shared__ long long s_above;
+  const int slot = blockIdx.x;
+  TiesSlot S = m.slots[slot];
+  if (S.done) return;
+  unsigned long long* gh = m.hist + (size_t)slot * kHistBins;
+  select_from_top(gh, kHistBins, m.rank[slot], s_sum, &s_digit, &s_above);
+  if (threadIdx.x == 0) {
+    const int b = s_digit;
+    const uint64_t past = (uint64_t)S.lo + (uint64_t(kInner) << S.shift);  // first key above the interval
+    if (b <= 0) {
+      set_interval(S, 0u, S.lo);
+    } else if (b == kHistBins - 1 && past <= kInfKey) {
+      set_interval(S, (uint32_t)past, kInfKey + 1u - past);
+    } else if (b == kHistBins - 1) {  // NaN keys alone are left: the hardware's NaN
+      m.thr[slot] = 0x7FFFFFFFu;
+      S.done = 1u;
+      atomicAdd(m.n_done, 1u);
+    } else {
+      const uint32_t first = S.lo + ((uint32_t)(b - 1) << S.shift);
+      if (S.shift == 0 || (DT == DT_BF16 && (gh[b] >> 63) == 0ull)) {
+        m.thr[slot] = first;
+        S.done = 1u;
+        atomicAdd(m.n_done, 1u);
+      } else {
+        set_interval(S, first, uint64_t(1) << S.shift);
+      }
+    }
+    m.slots[slot] = S;
+  }
+  __syncthreads();  // gh[b] has been read
   for (int b = threadIdx.x; b < kHistBins; b += kBlock) gh[b] = 0ull;
 }
 
@@ -629,7 +825,7 @@ cudaError_t merge_method(const MArgs& m, int grid, cudaStream_t s) {
 
 // ------------------------------------------------------------------- host ---
 struct MLayout {
-  size_t tensors, chunks, experts, thr, prefix, rank, hist, total;
+  size_t tensors, chunks, experts, thr, slots, n_done, rank, hist, total;
 };
 
 size_t align_m(size_t x) { return (x + kMergeAlign - 1) / kMergeAlign * kMergeAlign; }
@@ -642,7 +838,8 @@ MLayout merge_layout(int32_t n, int64_t n_chunks, int K, bool ties) {
   L.chunks = off;  off = align_m(off + sizeof(Chunk) * (size_t)n_chunks);
   L.experts = off; off = align_m(off + sizeof(void*) * slots);
   L.thr = off;     off = align_m(off + sizeof(uint32_t) * slots);
-  L.prefix = off;  off = align_m(off + sizeof(uint32_t) * slots);
+  L.slots = off;   off = align_m(off + sizeof(TiesSlot) * slots);
+  L.n_done = off;  off = align_m(off + sizeof(uint32_t));
   L.rank = off;    off = align_m(off + sizeof(int64_t) * slots);
   L.hist = off;    off = align_m(off + (ties ? sizeof(unsigned long long) * kHistBins * slots : 0));
   L.total = off;
@@ -721,21 +918,16 @@ cudaError_t merge_launch(MArgs m, int64_t slots, bool ties, int sms, cudaStream_
   if (ties) {
     const int64_t items = m.n_chunks * ((m.K + kHistExperts - 1) / kHistExperts);
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ties_hist_kernel<DT, false>, kBlock, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ties_hist_kernel<DT>, kBlock, 0) != cudaSuccess ||
         occ < 1)
       occ = 1;
     const int64_t resident = (int64_t)occ * sms;
     const int hgrid = (int)(items < resident ? items : resident);
+    m.n_slots = (int32_t)slots;
+    ties_sample_kernel<DT><<<(int)slots, kBlock, 0, s>>>(m);
     for (int p = 0; p < kPasses; ++p) {
-      m.shift = kPassShift[p];
-      m.width = kPassWidth[p];
-      m.decided = (m.shift + m.width >= 32) ? 0u : ~((1u << (m.shift + m.width)) - 1u);
-      m.last_pass = p == kPasses - 1;
-      if (p == 0)
-        ties_hist_kernel<DT, true><<<hgrid, kBlock, 0, s>>>(m);
-      else
-        ties_hist_kernel<DT, false><<<hgrid, kBlock, 0, s>>>(m);
-      ties_select_kernel<<<(int)slots, kBlock, 0, s>>>(m);
+      ties_hist_kernel<DT><<<hgrid, kBlock, 0, s>>>(m);
+      ties_select_kernel<DT><<<(int)slots, kBlock, 0, s>>>(m);
     }
   }
   const int grid = (int)(m.n_chunks < 2 * (int64_t)sms ? m.n_chunks : 2 * (int64_t)sms);
@@ -825,7 +1017,8 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
   m.chunks = reinterpret_cast<const Chunk*>(ws + L.chunks);
   m.experts = reinterpret_cast<const void* const*>(ws + L.experts);
   m.thr = reinterpret_cast<uint32_t*>(ws + L.thr);
-  m.prefix = reinterpret_cast<uint32_t*>(ws + L.prefix);
+  m.slots = reinterpret_cast<TiesSlot*>(ws + L.slots);
+  m.n_done = reinterpret_cast<uint32_t*>(ws + L.n_done);
   m.rank = reinterpret_cast<int64_t*>(ws + L.rank);
   m.hist = ties ? reinterpret_cast<unsigned long long*>(ws + L.hist) : nullptr;
   m.n_chunks = nc;
@@ -846,7 +1039,7 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
     return mfail(SMAT_ERR_CUDA, "device query failed");
   const int rounds = cfg->philox_rounds == 7 ? 7 : 10;
   if (ties) {
-    e = cudaMemsetAsync(ws + L.prefix, 0, sizeof(uint32_t) * slots, stream);
+    e = cudaMemsetAsync(ws + L.n_done, 0, sizeof(uint32_t), stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws + L.thr, 0, sizeof(uint32_t) * slots, stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ws + L.hist, 0, sizeof(unsigned long long) * kHistBins * slots, stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.rank, hrank.data(), sizeof(int64_t) * slots, cudaMemcpyHostToDevice, stream);

@@ -182,3 +182,40 @@ def test_merge_special_values(method, dtype):
     nan_g, nan_r = np.isnan(gf), np.isnan(rf)
     assert np.array_equal(nan_g, nan_r)
     assert np.array_equal(got.view(view)[~nan_g], ref.view(view)[~nan_r])
+
+
+@pytest.mark.parametrize("dtype", [O.F32, O.BF16])
+@pytest.mark.parametrize("shape", ["normal", "mostly_zero", "sample_low", "sample_high", "infinities", "two_values"])
+@pytest.mark.parametrize("retention", [1e-4, 0.5, 1.0])
+def test_merge_ties_threshold_selection(dtype, shape, retention):
+    """Thresholds of tensors larger than the selection's sample (65,536
+    elements, in 16-element groups at 16 floor(g (n / 16) / 4096)) equal the
+    oracle's, also where the sample shows other magnitudes than the rest (its
+    interval misses, and the next passes start from the whole range), where
+    most keys are equal, and with infinities."""
+    n, K = 200_000 + 37, 2
+    g = torch.Generator().manual_seed(31)
+    t0 = torch.randn(n, generator=g) * 0.02
+    d = torch.randn(K, n, generator=g) * 1e-3
+    seen = torch.zeros(n, dtype=torch.bool)
+    first = 16 * (torch.arange(4096) * (n // 16) // 4096)
+    seen[(first[:, None] + torch.arange(16)).reshape(-1)] = True
+    if shape == "mostly_zero":
+        d[torch.rand(K, n, generator=g) < 0.8] = 0.0
+    elif shape == "sample_low":
+        d[:, seen] *= 1e-3
+    elif shape == "sample_high":
+        d[:, seen] *= 1e3
+    elif shape == "infinities":
+        d[torch.rand(K, n, generator=g) < 0.7] = float("inf")
+    elif shape == "two_values":
+        d = torch.where(d > 0, 0.25, 0.5)
+        t0 = torch.zeros(n)
+    tdt = torch.bfloat16 if dtype == O.BF16 else torch.float32
+    t0d = t0.to(tdt).cuda()
+    exd = [(t0 + d[e]).to(tdt).cuda() for e in range(K)]
+    out = torch.empty_like(t0d)
+    kw = dict(gamma=0.7, retention=retention)
+    thr = S.merge([t0d], [exd], [out], S.SMAT_MERGE_TIES, return_thresholds=True, **kw)
+    torch.cuda.synchronize()
+    _check([t0d], [exd], [out], dtype, S.SMAT_MERGE_TIES, kw, thr=thr)

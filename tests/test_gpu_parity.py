@@ -262,6 +262,31 @@ def test_inplace_gradient_map():
     assert np.array_equal(to_host(g), ref)
 
 
+@pytest.mark.parametrize("gdt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("alpha_mode", [S.SMAT_ALPHA_PER_TENSOR, S.SMAT_ALPHA_PER_ELEMENT])
+@pytest.mark.parametrize("keep", [0.3, 0.7, 0.002])
+def test_inplace_gradient_map_equals_out_of_place(gdt, alpha_mode, keep):
+    """In place, mask ties are written as kept and the dropped ones rewritten
+    at the end of the chunk (out of place the likelier outcome comes first):
+    the same bits either way, on whole chunks, remainders and chunks of 2^12
+    and 2^17 elements, with thresholds whose ties are mostly kept and mostly
+    dropped."""
+    n = 300_000 + 13
+    th = torch.randn(n, device="cuda") * 0.02
+    for flags in (S.SMAT_FLAG_CHUNK_LOG2(12), S.SMAT_FLAG_CHUNK_LOG2(17)):
+        sess = S.SmatSession([th], [th.clone()], [torch.empty_like(th)], [keep], [1e-3], seed=3, alpha_min=0.3,
+                             alpha_mode=alpha_mode, flags=flags)
+        sess.simulate_multi(2)
+        g = torch.randn(n, device="cuda").to(gdt)
+        out = torch.empty_like(g)
+        sess.grad_map_multi(2, [g], [out])
+        sess.grad_map_multi(2, [g])
+        torch.cuda.synchronize()
+        bits = torch.int32 if gdt == torch.float32 else torch.int16
+        assert torch.equal(g.view(bits), out.view(bits))
+        sess.close()
+
+
 def test_gradient_map_needs_the_forward_of_its_step():
     """The gradient map regenerates the mask of the forward that produced
     theta~ (Eq. smat-gradient; App. D): a map for a step that no forward on

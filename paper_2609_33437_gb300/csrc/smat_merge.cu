@@ -3,7 +3,7 @@
 // theta0, for weight averaging, Task Arithmetic, DARE followed by Task
 // Arithmetic and TIES (the merging methods of Sec. 5). Elementwise and bound
 // by HBM bandwidth: each element reads theta0 and the K experts once and
-// writes the result once (TIES first reads every expert three more times to
+// writes the result once (TIES first reads every expert once or twice more to
 // select its per-tensor trim thresholds exactly).
 //
 // Arithmetic, identical to the CPU oracle: Delta_j one fp32 subtraction;
@@ -20,15 +20,17 @@
 // holds the threshold almost surely (small tensors are sampled whole, which
 // decides them); a pass over the inputs then counts the keys in 2046 equal
 // bins of that interval and in one bin below and one above it, and one CTA
-// per slot picks the bin that holds the r-th largest. A bin of one key, or
-// one all of whose keys are its first (bf16 differences lie on coarse grids),
-// is the threshold; any other bin, also the two outer ones when the sample
-// missed, is the next pass's interval. Passes skip decided slots.
+// per slot picks the bin that holds the r-th largest. A bin of one key, or the
+// first key of a bin (bf16 differences lie on coarse grids) if that is
+// where the r-th lies, is the threshold; any other bin, also the two outer
+// ones when the sample missed, is the next pass's interval. Passes skip decided
+// slots.
 
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <type_traits>
 #include <unordered_set>
 #include <vector>
 
@@ -74,7 +76,7 @@ struct MArgs {
   TiesSlot* slots;             // [tensor * K + e]
   int64_t* rank;               // r of each slot (1 = the largest key)
   uint32_t* n_done;            // slots decided so far
-  unsigned long long* hist;    // [(tensor * K + e) * kHistBins]; bit 63: some key is not its bin's first
+  unsigned long long* hist;    // [(tensor * K + e) * kHistBins], see ties_hist_kernel
   int64_t n_chunks;
   RoundKeys key;
   int32_t K, method;
@@ -313,93 +315,109 @@ __device__ __forceinline__ void dare_linear16(const MArgs& m, const MTensor& T, 
   store_merged16<DT>(T, i, t0, acc);
 }
 
-// TIES on one 16-element group: elect, then the disjoint mean (the experts
-// are read twice; the second read is served by the L2). The oracle's
-// agreement test, abs(Delta) >= thr and (sum > 0 and Delta > 0 or sum < 0 and
-// Delta < 0), is taken as: key in [max(thr, 1), key(+inf)] (Delta nonzero,
-// not NaN) and equal sign bits of Delta and sum; elements whose sum is 0 or
-// NaN, where the oracle finds no agreeing expert, are set to 0 at the end.
+// ------------------------------------------------------------ TIES merge pass ---
+// Eight consecutive elements as loaded (bf16: 16 bytes, fp32: 32).
 template <int DT>
-__device__ __forceinline__ void merge_ties16(const MArgs& m, const MTensor& T, int t, int64_t i) {
-  Raw16<DT> t0;
-  load16<DT>(T.theta0, i, t0);
-  const void* const* xp = m.experts + t * m.K;
-  const uint32_t* tp = m.thr + t * m.K;
-  float sum[16];
+struct Raw8 {
+  uint32_t r[DT == DT_BF16 ? 4 : 8];
+  __device__ __forceinline__ float2 pair(int m) const {
+    if (DT == DT_BF16) return make_float2(__uint_as_float(r[m] << 16), __uint_as_float(r[m] & 0xFFFF0000u));
+    return make_float2(__uint_as_float(r[2 * m]), __uint_as_float(r[2 * m + 1]));
+  }
+};
+
+template <int DT>
+__device__ __forceinline__ void load8(const void* base, int64_t i, Raw8<DT>& v) {
+  if constexpr (DT == DT_BF16) {
+    asm("ld.global.L1::no_allocate.v4.b32 {%0,%1,%2,%3}, [%4];"
+        : "=r"(v.r[0]), "=r"(v.r[1]), "=r"(v.r[2]), "=r"(v.r[3])
+        : "l"(static_cast<const uint16_t*>(base) + i));
+  } else {
+    ld32B(static_cast<const float*>(base) + i, v.r);
+  }
+}
+
+// One expert's Delta of one element into the running sums: kept positive values
+// (Delta >= lo), kept negative ones (Delta <= -lo), both together, and the two
+// counts (positive in the low byte, negative in the next). Written out so that
+// the additions are predicated: as C++ conditions they became branches (three
+// times the merge pass's time), and as factors 1 and 0 of multiply-adds a
+// comparison and a select each.
+__device__ __forceinline__ void ties_add(float d, float lo, float& sum, float& pos, float& neg, uint32_t& cnt) {
+  asm("{\n\t.reg .pred p, n;\n\t"
+      "setp.ge.f32 p, %4, %5;\n\tsetp.le.f32 n, %4, %6;\n\t"
+      "@p add.rn.f32 %0, %0, %4;\n\t@p add.rn.f32 %1, %1, %4;\n\t@p add.u32 %3, %3, 1;\n\t"
+      "@n add.rn.f32 %0, %0, %4;\n\t@n add.rn.f32 %2, %2, %4;\n\t@n add.u32 %3, %3, 256;\n\t}"
+      : "+f"(sum), "+f"(pos), "+f"(neg), "+r"(cnt)
+      : "f"(d), "f"(lo), "f"(-lo));
+}
+
+// TIES on an 8-element group in one reading of the experts: beside the sum of
+// the kept values that elects the sign, the kept positive values and the kept
+// negative ones are summed and counted by themselves, each in expert order, so
+// that the elected one's sum is the disjoint mean's numerator whatever the
+// sign. Kept: key >= lo = max(thr, 1): a zero Delta changes no sum and agrees
+// with no sign. A NaN Delta passes neither test, where the oracle's sum
+// becomes NaN and elects nothing: false is returned (nothing is stored) if
+// some Delta of the group is NaN, or infinities of both signs meet, and the
+// caller takes the element path. BATCH: experts whose loads are in flight
+// together; FULL: it divides their number (a build of its own: with the
+// remainder's code beside it the loop spilled, and the pass took 7.2 ms
+// instead of 4.2 for 8 experts of 1.07e9 bf16 elements).
+template <int DT, int BATCH, bool FULL>
+__device__ __forceinline__ bool merge_ties8(const MArgs& m, const void* t0_p, void* out_p, const void* const* xp,
+                                            const float* lo, int64_t i) {
+  Raw8<DT> t0;
+  load8<DT>(t0_p, i, t0);
+  float sum[8], pos[8], neg[8];
+  uint32_t cnt[8];
+  float2 all = splat(0.0f);  // NaN if some Delta is
 #pragma unroll
-  for (int k = 0; k < 16; ++k) sum[k] = 0.0f;
-  auto elect = [&](const Raw16<DT>& x, uint32_t thr) {
+  for (int k = 0; k < 8; ++k) {
+    sum[k] = pos[k] = neg[k] = 0.0f;
+    cnt[k] = 0u;
+  }
+  auto add = [&](const Raw8<DT>& x, float l) {
 #pragma unroll
-    for (int h = 0; h < 8; ++h) {
-      const float2 b = t0.pair(h);
-      const float2 d = sub2_rn(x.pair(h), b);
-      if (abs_key(d.x) >= thr) sum[2 * h] = __fadd_rn(sum[2 * h], d.x);
-      if (abs_key(d.y) >= thr) sum[2 * h + 1] = __fadd_rn(sum[2 * h + 1], d.y);
+    for (int h = 0; h < 4; ++h) {
+      const float2 d = sub2_rn(x.pair(h), t0.pair(h));
+      all = add2_rn(all, d);
+      ties_add(d.x, l, sum[2 * h], pos[2 * h], neg[2 * h], cnt[2 * h]);
+      ties_add(d.y, l, sum[2 * h + 1], pos[2 * h + 1], neg[2 * h + 1], cnt[2 * h + 1]);
     }
   };
-  int e = 0;
 #pragma unroll 1
-  for (; e + kExpertBatch <= m.K; e += kExpertBatch) {
-    Raw16<DT> x[kExpertBatch];
+  for (int e = 0; e < m.K; e += BATCH) {
+    Raw8<DT> x[BATCH];
 #pragma unroll
-    for (int b = 0; b < kExpertBatch; ++b) load16<DT>(xp[e + b], i, x[b]);
+    for (int b = 0; b < BATCH; ++b)
+      if (FULL || e + b < m.K) load8<DT>(xp[e + b], i, x[b]);
 #pragma unroll
-    for (int b = 0; b < kExpertBatch; ++b) elect(x[b], tp[e + b]);
+    for (int b = 0; b < BATCH; ++b)
+      if (FULL || e + b < m.K) add(x[b], lo[e + b]);
   }
-#pragma unroll 1
-  for (; e < m.K; ++e) {
-    Raw16<DT> x;
-    load16<DT>(xp[e], i, x);
-    elect(x, tp[e]);
+  if (isnan(__fadd_rn(all.x, all.y))) return false;
+  float out[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float part = sum[k] > 0.0f ? pos[k] : neg[k];
+    const uint32_t n = sum[k] > 0.0f ? (cnt[k] & 0xFFu) : (cnt[k] >> 8);
+    const float mean = n && (sum[k] > 0.0f || sum[k] < 0.0f) ? __fdiv_rn(part, (float)n) : 0.0f;
+    const float b = (k & 1) ? t0.pair(k >> 1).y : t0.pair(k >> 1).x;
+    out[k] = __fadd_rn(b, __fmul_rn(m.gamma, mean));
   }
-  float part[16];
-  uint32_t cnt[4] = {0u, 0u, 0u, 0u};  // four 8-bit counts per word (K <= 16)
+  if constexpr (DT == DT_BF16) {
+    asm volatile("st.global.v4.b32 [%0], {%1,%2,%3,%4};" ::"l"(static_cast<uint16_t*>(out_p) + i),
+                 "r"(pack_bf16x2(out[0], out[1])), "r"(pack_bf16x2(out[2], out[3])),
+                 "r"(pack_bf16x2(out[4], out[5])), "r"(pack_bf16x2(out[6], out[7]))
+                 : "memory");
+  } else {
+    uint32_t r[8];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) part[k] = 0.0f;
-  auto agree = [&](float d, uint32_t lo, int k) {
-    const uint32_t key = abs_key(d);
-    return key >= lo && key <= kInfKey && ((__float_as_uint(d) ^ __float_as_uint(sum[k])) & 0x80000000u) == 0u;
-  };
-  auto gather = [&](const Raw16<DT>& x, uint32_t thr) {
-    const uint32_t lo = thr > 1u ? thr : 1u;
-#pragma unroll
-    for (int h = 0; h < 8; ++h) {
-      const float2 b = t0.pair(h);
-      const float2 d = sub2_rn(x.pair(h), b);
-      if (agree(d.x, lo, 2 * h)) {
-        part[2 * h] = __fadd_rn(part[2 * h], d.x);
-        cnt[h >> 1] += 1u << (16 * (h & 1));
-      }
-      if (agree(d.y, lo, 2 * h + 1)) {
-        part[2 * h + 1] = __fadd_rn(part[2 * h + 1], d.y);
-        cnt[h >> 1] += 1u << (16 * (h & 1) + 8);
-      }
-    }
-  };
-  e = 0;
-#pragma unroll 1
-  for (; e + kExpertBatch <= m.K; e += kExpertBatch) {
-    Raw16<DT> x[kExpertBatch];
-#pragma unroll
-    for (int b = 0; b < kExpertBatch; ++b) load16<DT>(xp[e + b], i, x[b]);
-#pragma unroll
-    for (int b = 0; b < kExpertBatch; ++b) gather(x[b], tp[e + b]);
+    for (int k = 0; k < 8; ++k) r[k] = __float_as_uint(out[k]);
+    st32B(static_cast<float*>(out_p) + i, r);
   }
-#pragma unroll 1
-  for (; e < m.K; ++e) {
-    Raw16<DT> x;
-    load16<DT>(xp[e], i, x);
-    gather(x, tp[e]);
-  }
-  float out[16];
-#pragma unroll
-  for (int k = 0; k < 16; ++k) {
-    const uint32_t n = (cnt[k >> 2] >> (8 * (k & 3))) & 0xFFu;
-    const bool elected = sum[k] > 0.0f || sum[k] < 0.0f;
-    const float merged = (n && elected) ? __fdiv_rn(part[k], (float)n) : 0.0f;
-    out[k] = __fadd_rn(t0.at(k), __fmul_rn(m.gamma, merged));
-  }
-  store16<DT>(T.out, i, out);
+  return true;
 }
 
 // Any method, one element (any alignment).
@@ -434,6 +452,33 @@ __device__ __forceinline__ void merge_elem(const MArgs& m, const MTensor& T, int
   store1<DT>(T.out, i, __fadd_rn(t0, acc));
 }
 
+// TIES merge pass (no draws: one build for all stream variants).
+template <int DT, int BATCH, bool FULL>
+__global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 3 : 2) ties_merge_kernel(const __grid_constant__ MArgs m) {
+  __shared__ const void* s_x[kMergeMaxExperts];
+  __shared__ float s_lo[kMergeMaxExperts];
+  for (int64_t ci = blockIdx.x; ci < m.n_chunks; ci += gridDim.x) {
+    const Chunk ch = m.chunks[ci];
+    const MTensor& T = m.tensors[ch.tensor];
+    const void* const t0_p = T.theta0;
+    void* const out_p = T.out;
+    const bool vec = (T.flags & TF_VEC) != 0u;
+    __syncthreads();
+    if (threadIdx.x < m.K) {
+      s_x[threadIdx.x] = m.experts[ch.tensor * m.K + threadIdx.x];
+      const uint32_t thr = m.thr[ch.tensor * m.K + threadIdx.x];
+      s_lo[threadIdx.x] = __uint_as_float(thr > 1u ? thr : 1u);
+    }
+    __syncthreads();
+    for (int64_t i = ch.begin + 8 * (int64_t)threadIdx.x; i < ch.end; i += 8 * (int64_t)kBlock) {
+      if (vec && i + 8 <= ch.end && merge_ties8<DT, BATCH, FULL>(m, t0_p, out_p, s_x, s_lo, i)) continue;
+      const int64_t e_end = (i + 8 < ch.end) ? i + 8 : ch.end;
+#pragma unroll 1
+      for (int64_t e = i; e < e_end; ++e) merge_elem<10, DT, SMAT_MERGE_TIES>(m, T, ch.tensor, e);
+    }
+  }
+}
+
 template <int R, int DT, int METHOD>
 __global__ void __launch_bounds__(kBlock, 2) merge_kernel(const __grid_constant__ MArgs m) {
   for (int64_t ci = blockIdx.x; ci < m.n_chunks; ci += gridDim.x) {
@@ -442,10 +487,7 @@ __global__ void __launch_bounds__(kBlock, 2) merge_kernel(const __grid_constant_
     const bool vec = (T.flags & TF_VEC) != 0u;
     for (int64_t i = ch.begin + 16 * (int64_t)threadIdx.x; i < ch.end; i += 16 * (int64_t)kBlock) {
       if (vec && i + 16 <= ch.end) {
-        if (METHOD == SMAT_MERGE_TIES)
-          merge_ties16<DT>(m, T, ch.tensor, i);
-        else
-          merge_linear16<DT>(m, T, ch.tensor, i);
+        merge_linear16<DT>(m, T, ch.tensor, i);
       } else {
         const int64_t e_end = (i + 16 < ch.end) ? i + 16 : ch.end;
         for (int64_t e = i; e < e_end; ++e) merge_elem<R, DT, METHOD>(m, T, ch.tensor, e);
@@ -508,39 +550,49 @@ __device__ __forceinline__ void set_interval(TiesSlot& S, uint32_t lo, uint64_t 
   S.shift = s;
 }
 
+__device__ __forceinline__ unsigned long long count_at(const uint32_t* p) { return *p; }  // shared memory
+__device__ __forceinline__ unsigned long long count_at(const unsigned long long* p) {     // global bin (numel < 2^40)
+  return __ldcg(p) & ((1ull << 41) - 1u);
+}
+
 // The bin that holds the r-th entry counted from the top of a histogram of nb
-// bins (counts: bits 0 to 62) and the entries above that bin, by all threads
-// of the CTA; digit -1 if there are fewer than r.
-template <typename Count>
-__device__ __forceinline__ void select_from_top(const Count* hist, int nb, long long r, unsigned long long* s_sum,
-                                                int* s_digit, long long* s_above) {
-  constexpr unsigned long long kCount = ~0ull >> 1;
-  const int per = nb / kBlock;  // bins per thread, highest bins in thread 0
+// bins and the entries above that bin, by all NT threads of the CTA; digit -1
+// if there are fewer than r.
+template <int NT>
+struct SelectShared {
+  unsigned long long sum[NT];
+  int digit;
+  long long above;
+};
+
+template <int NT, typename Count>
+__device__ __forceinline__ void select_from_top(const Count* hist, int nb, long long r, SelectShared<NT>& sh) {
+  const int per = nb / NT;  // bins per thread, highest bins in thread 0
   unsigned long long local = 0;
   const int top = nb - 1 - threadIdx.x * per;
-  for (int k = 0; k < per; ++k) local += hist[top - k] & kCount;
-  s_sum[threadIdx.x] = local;
+  for (int k = 0; k < per; ++k) local += count_at(hist + top - k);
+  sh.sum[threadIdx.x] = local;
   if (threadIdx.x == 0) {
-    *s_digit = -1;
-    *s_above = 0;
+    sh.digit = -1;
+    sh.above = 0;
   }
   __syncthreads();
-  // inclusive scan from the top (Hillis-Steele; 8 steps over 256 entries)
-  for (int o = 1; o < kBlock; o <<= 1) {
-    const unsigned long long v = threadIdx.x >= o ? s_sum[threadIdx.x - o] : 0ull;
+  // inclusive scan from the top (Hillis-Steele)
+  for (int o = 1; o < NT; o <<= 1) {
+    const unsigned long long v = threadIdx.x >= o ? sh.sum[threadIdx.x - o] : 0ull;
     __syncthreads();
-    s_sum[threadIdx.x] += v;
+    sh.sum[threadIdx.x] += v;
     __syncthreads();
   }
-  const unsigned long long incl = s_sum[threadIdx.x];
+  const unsigned long long incl = sh.sum[threadIdx.x];
   const unsigned long long excl = incl - local;
   if (r > 0 && (long long)excl < r && r <= (long long)incl) {
     unsigned long long acc = excl;
     for (int k = 0; k < per; ++k) {
-      const unsigned long long c = hist[top - k] & kCount;
+      const unsigned long long c = count_at(hist + top - k);
       if ((long long)(acc + c) >= r) {
-        *s_digit = top - k;
-        *s_above = (long long)acc;
+        sh.digit = top - k;
+        sh.above = (long long)acc;
         break;
       }
       acc += c;
@@ -553,12 +605,12 @@ __device__ __forceinline__ void select_from_top(const Count* hist, int nb, long 
 // the sample, eight standard deviations of the sampled rank to either side of
 // r's share, each by a radix select of three digits (11, 11 and 10 bits). The
 // three readings of the sample (2 x 128 KB for bf16) come from L2 after the first.
+constexpr int kSampleThreads = 1024;
+
 template <int DT>
-__global__ void __launch_bounds__(kBlock) ties_sample_kernel(const __grid_constant__ MArgs m) {
+__global__ void __launch_bounds__(kSampleThreads) ties_sample_kernel(const __grid_constant__ MArgs m) {
   __shared__ uint32_t h[2][kHistBins];
-  __shared__ unsigned long long s_sum[kBlock];
-  __shared__ int s_digit;
-  __shared__ long long s_above;
+  __shared__ SelectShared<kSampleThreads> sh;
   const int slot = blockIdx.x;
   const MTensor& T = m.tensors[slot / m.K];
   const void* x = m.experts[slot];
@@ -592,14 +644,14 @@ __global__ void __launch_bounds__(kBlock) ties_sample_kernel(const __grid_consta
     const int shift = shifts[pass], nb = 1 << widths[pass];
     const uint32_t decided = pass == 0 ? 0u : ~0u << shifts[pass - 1];
     const bool same = prefix[0] == prefix[1];
-    for (int b = threadIdx.x; b < 2 * kHistBins; b += kBlock) (&h[0][0])[b] = 0u;
+    for (int b = threadIdx.x; b < 2 * kHistBins; b += kSampleThreads) (&h[0][0])[b] = 0u;
     __syncthreads();
     auto count = [&](uint32_t key) {
       const uint32_t digit = (key >> shift) & (uint32_t)(nb - 1);
       if ((key & decided) == prefix[0]) atomicAdd(&h[0][digit], 1u);
       if (!same && (key & decided) == prefix[1]) atomicAdd(&h[1][digit], 1u);
     };
-    for (int g = threadIdx.x; g < groups; g += kBlock) {
+    for (int g = threadIdx.x; g < groups; g += kSampleThreads) {
       const int64_t i = 16 * (all ? (int64_t)g : (int64_t)g * (n / 16) / groups);
       if (vec && i + 16 <= n) {
         Raw16<DT> t0, y;
@@ -617,9 +669,9 @@ __global__ void __launch_bounds__(kBlock) ties_sample_kernel(const __grid_consta
     }
     __syncthreads();
     for (int q = 0; q < 2; ++q) {
-      select_from_top(h[same ? 0 : q], nb, rank[q], s_sum, &s_digit, &s_above);
-      prefix[q] |= (uint32_t)s_digit << shift;
-      rank[q] -= s_above;
+      select_from_top(h[same ? 0 : q], nb, rank[q], sh);
+      prefix[q] |= (uint32_t)sh.digit << shift;
+      rank[q] -= sh.above;
       __syncthreads();
     }
   }
@@ -646,14 +698,46 @@ __global__ void __launch_bounds__(kBlock) ties_sample_kernel(const __grid_consta
 // Every key counts (the outer bins take what lies outside the interval), so
 // that no branch surrounds the shared-memory atomic: a pass that tested each
 // key against the digits decided so far and branched around the atomic took
-// twice as long at the same traffic (5.7 against 2.9 ms for 8 experts of 1.07e9
-// bf16 elements), bound by issue slots instead of HBM.
+// 5.7 ms for 8 experts of 1.07e9 bf16 elements, bound by issue slots; this one
+// takes 3.4 (2.9 at HBM speed), bound by the shared-memory atomics (LSU data
+// pipe 72% busy).
+//
+// bf16: a key that is not its bin's first (differences of bf16 values near
+// each other are multiples of coarse powers of two, so few keys are) sends its
+// group and expert to a list; after the chunk the CTA counts such keys per
+// bin. In the loop this is one operation per two keys and a seldom taken
+// branch; flagging there took 0.6 of 4.0 ms, and a flag without a count sent most
+// bf16 thresholds to a second pass. A shared bin holds the count
+// (17 bits, a chunk has 2^16 elements) and the count of those keys (15 bits);
+// a global bin the sums in bits 0 to 40 and 41 to 62. Where such keys are too
+// many to count (the list is full, or kOffMost of them in one chunk's bin)
+// bit 63 says so.
 constexpr int kHistExperts = 4;
-constexpr uint32_t kOffFirst = 0x80000000u;  // shared bins: some key is not its bin's first
+constexpr uint32_t kOffOne = 1u << 17;
+constexpr uint32_t kOffMost = 256u;  // sums of 2^14 chunks stay below 2^22
+constexpr int64_t kOffChunks = 1 << 14;
+constexpr int kOffList = 512;
 
 template <int DT>
-__global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 1) ties_hist_kernel(const __grid_constant__ MArgs m) {
+__device__ __forceinline__ void load_lane(const void* base, int64_t i, Raw16<DT>& v) {
+  load16<DT>(base, i, v);
+}
+template <int DT>
+__device__ __forceinline__ void load_lane(const void* base, int64_t i, Raw8<DT>& v) {
+  load8<DT>(base, i, v);
+}
+
+// A thread's 32 bytes of one array: 16 bf16 or 8 fp32 elements. (16 fp32
+// elements of theta0 and four experts took 147 registers, one CTA per SM.)
+template <int DT>
+using RawLane = std::conditional_t<DT == DT_BF16, Raw16<DT>, Raw8<DT>>;
+
+template <int DT>
+__global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 3) ties_hist_kernel(const __grid_constant__ MArgs m) {
+  constexpr int kLane = DT == DT_BF16 ? 16 : 8;
   __shared__ uint32_t h[kHistExperts * kHistBins];
+  __shared__ uint16_t list[kOffList];  // (group << 2) | expert of the batch
+  __shared__ int n_list;
   if (*m.n_done == (uint32_t)m.n_slots) return;
   const int nbat = (m.K + kHistExperts - 1) / kHistExperts;
   const int64_t items = m.n_chunks * nbat;
@@ -685,121 +769,137 @@ __global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 1) ties_hist_kerne
     }
     if (!any) continue;  // the same slots in every thread
     for (int b = threadIdx.x; b < kHistExperts * kHistBins; b += kBlock) h[b] = 0u;
+    if (threadIdx.x == 0) n_list = 0;
     __syncthreads();
     // bin of a key: 1 + (key - lo) / 2^shift, clamped to [0, 2047]
-    auto bin = [&](uint32_t key, int b) {
-      return __viaddmin_s32_relu((int)(key - lo[b]) >> sh[b], 1, kHistBins - 1);
-    };
-    auto mark = [&](uint32_t key, int b) {  // bf16: a key that is not its bin's first
-      const int j = bin(key, b);
-      if ((key & ((1u << sh[b]) - 1u)) != 0u && j > 0 && j < kHistBins - 1) atomicOr(&h[b * kHistBins + j], kOffFirst);
+    auto bin_of = [&](uint32_t key, uint32_t low, int shift) {
+      return __viaddmin_s32_relu((int)(key - low) >> shift, 1, kHistBins - 1);
     };
     const bool vec = (T.flags & TF_VEC) != 0u;
-    for (int64_t i = ch.begin + 16 * (int64_t)threadIdx.x; i < ch.end; i += 16 * (int64_t)kBlock) {
-      if (vec && i + 16 <= ch.end) {
-        Raw16<DT> t0, x[kHistExperts];
-        load16<DT>(T.theta0, i, t0);
+    const void* t0p = T.theta0;
+    for (int64_t i = ch.begin + kLane * (int64_t)threadIdx.x; i < ch.end; i += kLane * (int64_t)kBlock) {
+      if (vec && i + kLane <= ch.end) {
+        RawLane<DT> t0, x[kHistExperts];
+        load_lane<DT>(t0p, i, t0);
 #pragma unroll
         for (int b = 0; b < kHistExperts; ++b)
-          if (xp[b]) load16<DT>(xp[b], i, x[b]);
-        uint32_t off = 0u;  // bf16: experts with a key that is not a multiple of 2^shift
+          if (xp[b]) load_lane<DT>(xp[b], i, x[b]);
 #pragma unroll
         for (int b = 0; b < kHistExperts; ++b) {
           if (xp[b]) {
             uint32_t bits = 0u;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
+            for (int q = 0; q < kLane / 2; ++q) {
               const float2 d = sub2_rn(x[b].pair(q), t0.pair(q));
               const uint32_t k0 = abs_key(d.x), k1 = abs_key(d.y);
               bits |= k0 | k1;
-              atomicAdd(&h[b * kHistBins + bin(k0, b)], 1u);
-              atomicAdd(&h[b * kHistBins + bin(k1, b)], 1u);
+              atomicAdd(&h[b * kHistBins + bin_of(k0, lo[b], sh[b])], 1u);
+              atomicAdd(&h[b * kHistBins + bin_of(k1, lo[b], sh[b])], 1u);
             }
-            if (DT == DT_BF16 && (bits & ((1u << sh[b]) - 1u)) != 0u) off |= 1u << b;
-          }
-        }
-        if (DT == DT_BF16 && off) {  // rare: the group again for its experts with such a key
-#pragma unroll
-          for (int b = 0; b < kHistExperts; ++b) {
-            if ((off >> b) & 1u) {
-              Raw16<DT> u0, y;
-              load16<DT>(T.theta0, i, u0);
-              load16<DT>(xp[b], i, y);
-#pragma unroll
-              for (int q = 0; q < 8; ++q) {
-                const float2 d = sub2_rn(y.pair(q), u0.pair(q));
-                mark(abs_key(d.x), b);
-                mark(abs_key(d.y), b);
-              }
+            if (DT == DT_BF16 && (bits & ((1u << sh[b]) - 1u)) != 0u) {
+              const int at = atomicAdd(&n_list, 1);
+              if (at < kOffList) list[at] = (uint16_t)(((uint32_t)(i - ch.begin) >> 4 << 2) | b);
             }
           }
         }
       } else {
-        const int64_t e_end = (i + 16 < ch.end) ? i + 16 : ch.end;
+        const int64_t e_end = (i + kLane < ch.end) ? i + kLane : ch.end;
         for (int64_t k = i; k < e_end; ++k) {
-          const float t0 = load1<DT>(T.theta0, k);
+          const float t0 = load1<DT>(t0p, k);
 #pragma unroll
           for (int b = 0; b < kHistExperts; ++b) {
             if (xp[b]) {
               const uint32_t key = abs_key(__fsub_rn(load1<DT>(xp[b], k), t0));
-              atomicAdd(&h[b * kHistBins + bin(key, b)], 1u);
-              if (DT == DT_BF16) mark(key, b);
+              atomicAdd(&h[b * kHistBins + bin_of(key, lo[b], sh[b])], 1u);
+              if (DT == DT_BF16 && (key & ((1u << sh[b]) - 1u)) != 0u) {
+                const int at = atomicAdd(&n_list, 1);  // the group may be listed more than once: it is counted too often
+                if (at < kOffList) list[at] = (uint16_t)(((uint32_t)(i - ch.begin) >> 4 << 2) | b);
+              }
             }
           }
         }
       }
     }
     __syncthreads();
+    const int listed = n_list;
+    if (DT == DT_BF16 && listed > 0 && listed <= kOffList) {
+      // sixteen threads per entry, an element each
+      for (int j = threadIdx.x >> 4; j < listed; j += kBlock / 16) {
+        const uint32_t it = list[j];
+        const int b = (int)(it & 3u);
+        const int64_t k = ch.begin + 16 * (int64_t)(it >> 2) + (threadIdx.x & 15);
+        if (k < ch.end) {
+          const TiesSlot S = m.slots[slot0 + b];
+          const uint32_t key = abs_key(__fsub_rn(load1<DT>(m.experts[slot0 + b], k), load1<DT>(t0p, k)));
+          const int bin = bin_of(key, S.lo, S.shift);
+          uint32_t* p = &h[b * kHistBins + bin];
+          // past kOffMost the exact count no longer matters (at most 256 threads add beyond it)
+          if ((key & ((1u << S.shift) - 1u)) != 0u && bin > 0 && bin < kHistBins - 1 &&
+              (*(volatile uint32_t*)p >> 17) < kOffMost)
+            atomicAdd(p, kOffOne);
+        }
+      }
+      __syncthreads();
+    }
     // the ne histograms are consecutive slots' bins in the global array
     unsigned long long* gh = m.hist + (size_t)slot0 * kHistBins;
+    const uint32_t most = T.numel <= kOffChunks * kMergeChunk ? kOffMost : 1u;
     for (int b = threadIdx.x; b < ne * kHistBins; b += kBlock) {
       const uint32_t c = h[b];
       if (c) {
-        atomicAdd(gh + b, (unsigned long long)(c & ~kOffFirst));
-        if (c & kOffFirst) atomicOr(gh + b, 1ull << 63);
+        const uint32_t off = c >> 17;
+        atomicAdd(gh + b, (unsigned long long)(c & (kOffOne - 1u)) | (off < most ? (unsigned long long)off << 41 : 0ull));
+        if (off >= most || listed > kOffList) atomicOr(gh + b, 1ull << 63);
       }
     }
     __syncthreads();
   }
 }
 
-// After a pass: one CTA per slot picks the bin that holds the r-th largest
-// key, and either decides the threshold or sets the next pass's interval and
-// clears the histogram.
+// After a pass, one CTA per slot: the bin that holds the r-th largest key either
+// decides the threshold or is the next pass's interval (and the histogram is
+// cleared). A launch of its own, about 6 us: done by the CTA that finishes a
+// tensor's last item it lengthened the pass by 0.75 of 3.4 ms (the call's
+// registers) and a small list's by 50 us (its slots one after the other).
 template <int DT>
 __global__ void __launch_bounds__(kBlock) ties_select_kernel(const __grid_constant__ MArgs m) {
-  __shared__ unsigned long long s_sum[kBlock];
-  __shared__ int s_digit;
-  __shared__ long long s_above;
+  __shared__ SelectShared<kBlock> sh;
   const int slot = blockIdx.x;
   TiesSlot S = m.slots[slot];
   if (S.done) return;
   unsigned long long* gh = m.hist + (size_t)slot * kHistBins;
-  select_from_top(gh, kHistBins, m.rank[slot], s_sum, &s_digit, &s_above);
+  const long long r = m.rank[slot];
+  select_from_top(gh, kHistBins, r, sh);
   if (threadIdx.x == 0) {
-    const int b = s_digit;
+    const int b = sh.digit;
     const uint64_t past = (uint64_t)S.lo + (uint64_t(kInner) << S.shift);  // first key above the interval
+    uint32_t thr = 0u;
     if (b <= 0) {
       set_interval(S, 0u, S.lo);
     } else if (b == kHistBins - 1 && past <= kInfKey) {
       set_interval(S, (uint32_t)past, kInfKey + 1u - past);
     } else if (b == kHistBins - 1) {  // NaN keys alone are left: the hardware's NaN
-      m.thr[slot] = 0x7FFFFFFFu;
+      thr = 0x7FFFFFFFu;
       S.done = 1u;
-      atomicAdd(m.n_done, 1u);
     } else {
       const uint32_t first = S.lo + ((uint32_t)(b - 1) << S.shift);
-      if (S.shift == 0 || (DT == DT_BF16 && (gh[b] >> 63) == 0ull)) {
-        m.thr[slot] = first;
+      // the bin's keys that are not its first are all larger: r - above is past them
+      const unsigned long long c = __ldcg(gh + b);
+      const bool counted = DT == DT_BF16 && (c >> 63) == 0ull;
+      if (S.shift == 0 || (counted && r - sh.above > (long long)(c >> 41))) {
+        thr = first;
         S.done = 1u;
-        atomicAdd(m.n_done, 1u);
       } else {
         set_interval(S, first, uint64_t(1) << S.shift);
       }
     }
     m.slots[slot] = S;
+    if (S.done) {
+      m.thr[slot] = thr;
+      atomicAdd(m.n_done, 1u);
+    }
   }
-  __syncthreads();  // gh[b] has been read
+  __syncthreads();  // the bins have been read
   for (int b = threadIdx.x; b < kHistBins; b += kBlock) gh[b] = 0ull;
 }
 
@@ -818,7 +918,7 @@ cudaError_t merge_method(const MArgs& m, int grid, cudaStream_t s) {
       dare_kernel<R, DT><<<grid, kBlock, smem, s>>>(m);
       break;
     }
-    default: merge_kernel<R, DT, SMAT_MERGE_TIES><<<grid, kBlock, 0, s>>>(m); break;
+    default: return cudaErrorInvalidValue;  // TIES: ties_merge_run
   }
   return cudaGetLastError();
 }
@@ -913,8 +1013,19 @@ smat_status merge_check(const smat_merge_tensor* t, int32_t n, const smat_merge_
   return SMAT_OK;
 }
 
+template <int DT, int BATCH, bool FULL>
+cudaError_t ties_merge_run(const MArgs& m, int sms, cudaStream_t s) {
+  int per_sm = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ties_merge_kernel<DT, BATCH, FULL>, kBlock, 0) != cudaSuccess ||
+      per_sm < 1)
+    per_sm = 1;
+  const int64_t resident = per_sm * (int64_t)sms;
+  ties_merge_kernel<DT, BATCH, FULL><<<(int)(m.n_chunks < resident ? m.n_chunks : resident), kBlock, 0, s>>>(m);
+  return cudaGetLastError();
+}
+
 template <int R, int DT>
-cudaError_t merge_launch(MArgs m, int64_t slots, bool ties, int sms, cudaStream_t s) {
+cudaError_t merge_launch(MArgs m, int64_t slots, int64_t largest, bool ties, int sms, cudaStream_t s) {
   if (ties) {
     const int64_t items = m.n_chunks * ((m.K + kHistExperts - 1) / kHistExperts);
     int occ = 0;
@@ -924,11 +1035,18 @@ cudaError_t merge_launch(MArgs m, int64_t slots, bool ties, int sms, cudaStream_
     const int64_t resident = (int64_t)occ * sms;
     const int hgrid = (int)(items < resident ? items : resident);
     m.n_slots = (int32_t)slots;
-    ties_sample_kernel<DT><<<(int)slots, kBlock, 0, s>>>(m);
-    for (int p = 0; p < kPasses; ++p) {
+    ties_sample_kernel<DT><<<(int)slots, kSampleThreads, 0, s>>>(m);
+    // no pass where every tensor is small enough for the sample to decide
+    for (int p = 0; p < (largest > kSampleElems ? kPasses : 0); ++p) {
       ties_hist_kernel<DT><<<hgrid, kBlock, 0, s>>>(m);
       ties_select_kernel<DT><<<(int)slots, kBlock, 0, s>>>(m);
     }
+  }
+  if (ties) {
+    if constexpr (DT == DT_BF16)
+      if (m.K % 8 == 0) return ties_merge_run<DT, 8, true>(m, sms, s);
+    if (m.K % 4 == 0) return ties_merge_run<DT, 4, true>(m, sms, s);
+    return ties_merge_run<DT, 4, false>(m, sms, s);
   }
   const int grid = (int)(m.n_chunks < 2 * (int64_t)sms ? m.n_chunks : 2 * (int64_t)sms);
   return merge_method<R, DT>(m, grid, s);
@@ -1046,12 +1164,14 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
     if (e != cudaSuccess) return mfail(SMAT_ERR_CUDA, "TIES state initialisation failed");
   }
   const int64_t slots64 = (int64_t)slots;
+  int64_t largest = 0;
+  for (int32_t k = 0; k < n_tensors; ++k) largest = tensors[k].numel > largest ? tensors[k].numel : largest;
   if (dtype == SMAT_BF16)
-    e = rounds == 7 ? merge_launch<7, DT_BF16>(m, slots64, ties, sms, stream)
-                    : merge_launch<10, DT_BF16>(m, slots64, ties, sms, stream);
+    e = rounds == 7 ? merge_launch<7, DT_BF16>(m, slots64, largest, ties, sms, stream)
+                    : merge_launch<10, DT_BF16>(m, slots64, largest, ties, sms, stream);
   else
-    e = rounds == 7 ? merge_launch<7, DT_F32>(m, slots64, ties, sms, stream)
-                    : merge_launch<10, DT_F32>(m, slots64, ties, sms, stream);
+    e = rounds == 7 ? merge_launch<7, DT_F32>(m, slots64, largest, ties, sms, stream)
+                    : merge_launch<10, DT_F32>(m, slots64, largest, ties, sms, stream);
   if (e != cudaSuccess) return mfail(SMAT_ERR_CUDA, "merge launch failed");
   return SMAT_OK;
 }

@@ -219,3 +219,30 @@ def test_merge_ties_threshold_selection(dtype, shape, retention):
     thr = S.merge([t0d], [exd], [out], S.SMAT_MERGE_TIES, return_thresholds=True, **kw)
     torch.cuda.synchronize()
     _check([t0d], [exd], [out], dtype, S.SMAT_MERGE_TIES, kw, thr=thr)
+
+
+@pytest.mark.parametrize("K", [1, 3, 4, 8, 12, 16])
+@pytest.mark.parametrize("dtype", [O.F32, O.BF16])
+def test_merge_ties_expert_counts(K, dtype):
+    """TIES over one to sixteen experts (the merge pass has builds for batches
+    of eight and four and for a remainder; the threshold passes take four at a
+    time) equals the oracle, with groups of eight that hold a NaN, infinities of
+    one sign and of both."""
+    t0s, exs = _experts([17, 4096, 65_536 + 41, 140_000], K, dtype, seed=60 + K)
+    for k in (1, 3):
+        n = t0s[k].numel()
+        exs[k][0][n // 3] = float("nan")
+        exs[k][K - 1][n // 5] = float("inf")
+        exs[k][0][n // 7] = float("-inf")
+        exs[k][K - 1][n // 7] = float("inf")
+    outs = [torch.empty_like(t) for t in t0s]
+    kw = dict(gamma=0.6, retention=0.4)
+    S.merge(t0s, exs, outs, S.SMAT_MERGE_TIES, **kw)
+    torch.cuda.synchronize()
+    for k, (t0, ex, out) in enumerate(zip(t0s, exs, outs)):
+        ref, _ = O.merge(O.MERGE_TIES, to_host(t0), [to_host(x) for x in ex], dtype=dtype, tensor_id=k, **kw)
+        got = to_host(out)
+        view = np.uint16 if dtype == O.BF16 else np.uint32
+        nan_g, nan_r = np.isnan(f32_of(got)), np.isnan(f32_of(ref))
+        assert np.array_equal(nan_g, nan_r)
+        assert np.array_equal(got.view(view)[~nan_g], ref.view(view)[~nan_r]), k

@@ -26,6 +26,7 @@
 // ones when the sample missed, is the next pass's interval. Passes skip decided
 // slots.
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -41,7 +42,17 @@ namespace smat {
 namespace {
 
 constexpr int kMergeMaxExperts = SMAT_MERGE_MAX_EXPERTS;
-constexpr int64_t kMergeChunk = int64_t(1) << 16;
+// Elements per chunk of a merge: 2^16, or for lists of fewer than 2432 such
+// chunks (16 per SM) a smaller power of two down to 2^13, so that a small
+// merge is spread over the chip (61 chunks of 2^16 left most SMs idle: TIES of 4
+// experts of 4e6 fp32 elements spent 55 us in the merge pass, 14 at HBM speed).
+constexpr int64_t kMergeChunkMax = int64_t(1) << 16;
+constexpr int64_t kMergeChunkMin = int64_t(1) << 13;
+int64_t merge_chunk_for(int64_t total) {
+  int64_t c = kMergeChunkMax;
+  while (c > kMergeChunkMin && total / c < 2432) c /= 2;
+  return c;
+}
 constexpr int kHistBins = 2048;  // an interval's 2046 bins, one below it and one above it
 constexpr int kInner = kHistBins - 2;
 // Passes over the inputs: one or two when the sample's interval holds the
@@ -82,6 +93,7 @@ struct MArgs {
   int32_t K, method;
   float gamma, c;              // c: per-expert coefficient (WA 1/K, TA gamma, DARE gamma / p_keep)
   int32_t n_slots;
+  int64_t chunk;               // elements per chunk
 };
 
 __device__ __forceinline__ uint32_t abs_key(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
@@ -708,7 +720,7 @@ __global__ void __launch_bounds__(kSampleThreads) ties_sample_kernel(const __gri
 // bin. In the loop this is one operation per two keys and a seldom taken
 // branch; flagging there took 0.6 of 4.0 ms, and a flag without a count sent most
 // bf16 thresholds to a second pass. A shared bin holds the count
-// (17 bits, a chunk has 2^16 elements) and the count of those keys (15 bits);
+// (17 bits, a chunk has at most 2^16 elements) and the count of those keys (15 bits);
 // a global bin the sums in bits 0 to 40 and 41 to 62. Where such keys are too
 // many to count (the list is full, or kOffMost of them in one chunk's bin)
 // bit 63 says so.
@@ -843,7 +855,7 @@ __global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 3) ties_hist_kerne
     }
     // the ne histograms are consecutive slots' bins in the global array
     unsigned long long* gh = m.hist + (size_t)slot0 * kHistBins;
-    const uint32_t most = T.numel <= kOffChunks * kMergeChunk ? kOffMost : 1u;
+    const uint32_t most = T.numel <= kOffChunks * m.chunk ? kOffMost : 1u;
     for (int b = threadIdx.x; b < ne * kHistBins; b += kBlock) {
       const uint32_t c = h[b];
       if (c) {
@@ -978,7 +990,7 @@ smat_status merge_check(const smat_merge_tensor* t, int32_t n, const smat_merge_
   if (cfg->flags != 0) return mfail(SMAT_ERR_UNSUPPORTED, "unknown flags 0x%x", cfg->flags);
   if (n < 0 || (n > 0 && !t)) return mfail(SMAT_ERR_INVALID_ARG, "bad tensor list");
   std::unordered_set<uint32_t> ids;
-  int64_t nc = 0;
+  int64_t nc = 0, total = 0;
   for (int32_t k = 0; k < n; ++k) {
     const smat_merge_tensor& d = t[k];
     if (d.numel < 0 || d.numel >= (int64_t(1) << 40))
@@ -1005,8 +1017,10 @@ smat_status merge_check(const smat_merge_tensor* t, int32_t n, const smat_merge_
           return mfail(SMAT_ERR_INVALID_ARG, "tensor %d: out overlaps expert %d", k, e);
       }
     }
-    nc += (d.numel + kMergeChunk - 1) / kMergeChunk;
+    total = std::min(total + d.numel, int64_t(1) << 62);
   }
+  const int64_t chunk = merge_chunk_for(total);
+  for (int32_t k = 0; k < n; ++k) nc += (t[k].numel + chunk - 1) / chunk;
   if (nc >= (int64_t(1) << 31)) return mfail(SMAT_ERR_INVALID_ARG, "too many chunks");
   *n_chunks = nc;
   *dtype_out = n > 0 ? t[0].dtype : SMAT_F32;
@@ -1073,6 +1087,9 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
   if (st != SMAT_OK) return st;
   const int K = cfg->n_experts;
   const bool ties = cfg->method == SMAT_MERGE_TIES;
+  int64_t total = 0;
+  for (int32_t k = 0; k < n_tensors; ++k) total = std::min(total + tensors[k].numel, int64_t(1) << 62);
+  const int64_t chunk = merge_chunk_for(total);
   const MLayout L = merge_layout(n_tensors, nc, K, ties);
   if (!d_workspace || (uintptr_t)d_workspace % kMergeAlign)
     return mfail(SMAT_ERR_WORKSPACE, "workspace NULL or not 256-byte aligned");
@@ -1119,12 +1136,12 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
       r = r < 1 ? 1 : (r > d.numel ? d.numel : r);
       for (int e = 0; e < K; ++e) hrank[(size_t)k * K + e] = r;
     }
-    for (int64_t j = 0; j * kMergeChunk < d.numel; ++j) {
+    for (int64_t j = 0; j * chunk < d.numel; ++j) {
       Chunk ch;
       ch.tensor = k;
       ch.pad = 0;
-      ch.begin = j * kMergeChunk;
-      ch.end = (j + 1) * kMergeChunk < d.numel ? (j + 1) * kMergeChunk : d.numel;
+      ch.begin = j * chunk;
+      ch.end = (j + 1) * chunk < d.numel ? (j + 1) * chunk : d.numel;
       hc.push_back(ch);
     }
   }
@@ -1140,6 +1157,7 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
   m.rank = reinterpret_cast<int64_t*>(ws + L.rank);
   m.hist = ties ? reinterpret_cast<unsigned long long*>(ws + L.hist) : nullptr;
   m.n_chunks = nc;
+  m.chunk = chunk;
   m.key = make_round_keys(cfg->seed);
   m.K = K;
   m.method = cfg->method;

@@ -158,89 +158,77 @@ __device__ __forceinline__ void merge_linear16(const MArgs& m, const MTensor& T,
 }
 
 // DARE keep masks. A warp first draws the masks of its 32 groups for all K
-// experts (expert e's mask is the Mask stream at step e) into shared memory,
-// as byte masks: byte b of word q of (expert e, thread t) is 0xFF iff element
-// 4q + b of t's group is kept. An element whose mask byte equals the
-// threshold's high byte (probability 1/256 per element and expert) is decided
-// by its low 24 bits (MASK_LO stream): these ties are queued per warp across
-// all experts and then drawn by the whole warp, one MASK_LO block per lane, so
-// a warp spends about one Philox pass per group on them instead of one mostly
-// idle pass per expert. A queue that fills up (about K/16 ties per thread are
-// expected, the capacity is 4 per thread) makes the owner draw the rest itself.
-constexpr int kDareQueue = 128;
-struct DareQueue {
-  uint16_t q[kBlock / 32][kDareQueue];  // (lane << 8) | (expert << 4) | element
-  int n[kBlock / 32];
-};
-// Dynamic shared memory of the DARE kernel: the queue, then uint4 keep masks
-// [K][kBlock] (16 bytes per expert and thread).
-constexpr size_t kDareQueueBytes = (sizeof(DareQueue) + 15) / 16 * 16;
-size_t dare_smem_bytes(int K) { return kDareQueueBytes + (size_t)K * kBlock * sizeof(uint4); }
+// experts (expert e's mask is the Mask stream at step e) into shared memory:
+// bit 8b + 7 of word q of (expert e, thread t) is element 4q + b of t's group.
+// A group with an element whose mask byte equals the threshold's high byte
+// (probability 1/256 per element and expert; its low 24 bits, MASK_LO stream,
+// decide) goes to the warp's queue: a ballot gives every such lane its slot,
+// so the main loop has no branch for it. The whole warp then draws the queued
+// groups together, about K / 16 per lane; most warps meet such a group for
+// every expert, and resolving it where it was met took as many instructions
+// as the expert's Philox block.
+// Dynamic shared memory: uint4 keep flags [K][kBlock], then the queues,
+// 32 K entries (lane << 4 | expert) per warp.
+size_t dare_smem_bytes(int K) {
+  return (size_t)K * kBlock * sizeof(uint4) + (size_t)K * kBlock * sizeof(uint16_t);
+}
 
 struct DareShared {
-  DareQueue* qs;
-  uint4* keep;  // keep[e * kBlock + thread]
+  uint4* keep;      // keep[e * kBlock + thread]
+  uint16_t* queue;  // this warp's
 };
-
-// Byte masks of expert e from its Mask block w; ties go to the warp's queue,
-// or are drawn here once the queue is full.
-template <int R>
-__device__ __forceinline__ uint4 dare_keep_masks(const MArgs& m, const MTensor& T, const uint4& w, int e,
-                                                 uint64_t g0, DareShared& s) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t kw[4];
-  if (keep_bytes16(w, T.t_hi, kw) && T.t_lo != 0u) {
-    uint32_t tb = tie_bits16(w, T.t_hi);
-    int slot = atomicAdd(&s.qs->n[warp], __popc(tb));
-    while (tb) {
-      const int k = __ffs(tb) - 1;
-      tb &= tb - 1u;
-      if (slot < kDareQueue) {
-        s.qs->q[warp][slot] = (uint16_t)((lane << 8) | (e << 4) | k);
-      } else {
-        const uint64_t g = g0 + (uint64_t)k;
-        const uint4 l = stream_block_at<R>(m.key, (uint32_t)e, S_MASK_LO, T.tid, g >> 2);
-        if ((pick(l, (unsigned)(g & 3)) >> 8) < T.t_lo) set_kept(kw, k);
-      }
-      ++slot;
-    }
-  }
-  // flag bit 7 of each byte -> 0x00 / 0xFF
-  return make_uint4((kw[0] >> 7) * 0xFFu, (kw[1] >> 7) * 0xFFu, (kw[2] >> 7) * 0xFFu, (kw[3] >> 7) * 0xFFu);
-}
 
 // Called by all 32 lanes of the warp (full: this lane has a vector group at
 // element index g0; gw0: lane 0's group). Two experts' Mask blocks are drawn
-// together (two independent Philox chains per thread). On return the lane's
-// keep masks are complete.
+// together (two independent Philox chains per thread). On return the warp's
+// keep flags are complete.
 template <int R>
 __device__ __forceinline__ void dare_masks(const MArgs& m, const MTensor& T, bool full, uint64_t g0, uint64_t gw0,
-                                           DareShared& s) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0) s.qs->n[warp] = 0;
-  __syncwarp();
-  if (full) {
+                                           const DareShared& s) {
+  const int lane = threadIdx.x & 31, wbase = threadIdx.x & ~31;
+  const bool low = full && T.t_lo != 0u;
+  const uint32_t below = (1u << lane) - 1u;
+  int n = 0;
+  auto draw = [&](const uint4& w, int e) {
+    uint32_t kw[4];
+    const bool tie = keep_bytes16(w, T.t_hi, kw) && low;
+    s.keep[e * kBlock + threadIdx.x] = make_uint4(kw[0], kw[1], kw[2], kw[3]);
+    const uint32_t b = __ballot_sync(0xFFFFFFFFu, tie);
+    if (tie) s.queue[n + __popc(b & below)] = (uint16_t)((lane << 4) | e);
+    n += __popc(b);
+  };
 #pragma unroll 1
-    for (int e = 0; e < m.K; e += 2) {
-      const uint4 w0 = stream_block_at<R>(m.key, (uint32_t)e, S_MASK, T.tid, g0 >> 4);
-      const uint4 w1 = stream_block_at<R>(m.key, (uint32_t)e + 1u, S_MASK, T.tid, g0 >> 4);
-      s.keep[e * kBlock + threadIdx.x] = dare_keep_masks<R>(m, T, w0, e, g0, s);
-      if (e + 1 < m.K) s.keep[(e + 1) * kBlock + threadIdx.x] = dare_keep_masks<R>(m, T, w1, e + 1, g0, s);
-    }
+  for (int e = 0; e < m.K; e += 2) {
+    const uint4 w0 = stream_block_at<R>(m.key, (uint32_t)e, S_MASK, T.tid, g0 >> 4);
+    const uint4 w1 = stream_block_at<R>(m.key, (uint32_t)e + 1u, S_MASK, T.tid, g0 >> 4);
+    draw(w0, e);
+    if (e + 1 < m.K) draw(w1, e + 1);
   }
   __syncwarp();
-  const int n = min(s.qs->n[warp], kDareQueue);
+#pragma unroll 1
   for (int j = lane; j < n; j += 32) {
-    const uint32_t it = s.qs->q[warp][j];
-    const int owner = (int)(it >> 8), e = (int)((it >> 4) & 15u), k = (int)(it & 15u);
-    const uint64_t g = gw0 + 16 * (uint64_t)owner + (uint64_t)k;
-    const uint4 l = stream_block_at<R>(m.key, (uint32_t)e, S_MASK_LO, T.tid, g >> 2);
-    if ((pick(l, (unsigned)(g & 3)) >> 8) < T.t_lo) {
-      uint32_t* kwp = reinterpret_cast<uint32_t*>(&s.keep[e * kBlock + (warp << 5) + owner]);
-      atomicOr(kwp + (k >> 2), 0xFFu << (8 * (k & 3)));
+    const uint32_t it = s.queue[j];
+    const int owner = (int)(it >> 4), e = (int)(it & 15u);
+    const uint64_t g = gw0 + 16 * (uint64_t)owner;
+    uint32_t tb = tie_bits16(stream_block_at<R>(m.key, (uint32_t)e, S_MASK, T.tid, g >> 4), T.t_hi);
+    uint32_t* kwp = reinterpret_cast<uint32_t*>(&s.keep[e * kBlock + wbase + owner]);
+    while (tb) {
+      const int k = __ffs(tb) - 1;
+      tb &= tb - 1u;
+      const uint4 l = stream_block_at<R>(m.key, (uint32_t)e, S_MASK_LO, T.tid, (g + (uint64_t)k) >> 2);
+      if ((pick(l, (unsigned)(k & 3)) >> 8) < T.t_lo) kwp[k >> 2] |= 0x80u << (8 * (k & 3));  // one lane per group
     }
   }
   __syncwarp();
+}
+
+// prmt.b32 with sign-replicating selectors (nibble bit 3): two keep flags of
+// a word spread over the 16-bit lanes of a mask.
+template <int SEL>
+__device__ __forceinline__ uint32_t spread_flags(uint32_t kw) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(kw), "n"(SEL));
+  return r;
 }
 
 // Expert e's DARE contribution to a bf16 group: the expert's bf16 words are
@@ -251,16 +239,15 @@ __device__ __forceinline__ void dare_masks(const MArgs& m, const MTensor& T, boo
 // the caller takes the select path below for a group with an infinite or NaN
 // theta0 (whose Delta would be NaN instead of unused).
 __device__ __forceinline__ void dare_acc16_blend(float c, const uint4& km, const Raw16<DT_BF16>& x,
-                                                 const Raw16<DT_BF16>& t0, float2 (&acc)[8]) {
+                                                 const Raw16<DT_BF16>& t0, const float2 (&b0)[8], float2 (&acc)[8]) {
   const float2 c2 = splat(c);
   const uint32_t kmw[4] = {km.x, km.y, km.z, km.w};
 #pragma unroll
   for (int h = 0; h < 8; ++h) {
-    // 16-bit lanes of the word's two elements: bytes 0, 1 (even h) or 2, 3 (odd h) of mask word h / 2
-    const uint32_t lm = __byte_perm(kmw[h >> 1], 0u, (h & 1) ? 0x3322u : 0x1100u);
+    // 16-bit lanes of the word's two elements: flags 0, 1 (even h) or 2, 3 (odd h) of flag word h / 2
+    const uint32_t lm = (h & 1) ? spread_flags<0xBBAA>(kmw[h >> 1]) : spread_flags<0x9988>(kmw[h >> 1]);
     const uint32_t xw = (x.r[h] & lm) | (t0.r[h] & ~lm);
-    const float2 b = t0.pair(h);
-    const float2 d = sub2_rn(make_float2(__uint_as_float(xw << 16), __uint_as_float(xw & 0xFFFF0000u)), b);
+    const float2 d = sub2_rn(make_float2(__uint_as_float(xw << 16), __uint_as_float(xw & 0xFFFF0000u)), b0[h]);
     acc[h] = fma2_rn(c2, d, acc[h]);
   }
 }
@@ -289,36 +276,41 @@ __device__ __forceinline__ bool nonfinite16(const Raw16<DT_BF16>& v) {
   return (nf & 0x80008000u) != 0u;
 }
 
-// Experts loaded before the keep masks are drawn (fp32 groups are twice the
-// registers: two, so that nothing spills).
+// Experts loaded together, the first of them before the keep masks are drawn.
 template <int DT>
-constexpr int kDarePrefetch = DT == DT_BF16 ? kExpertBatch : 2;
+constexpr int kDareBatch = DT == DT_BF16 ? 4 : 2;
 
-// DARE + TA on one 16-element group whose t0 and first kDarePrefetch experts
-// are already loaded; keep masks from shared memory (masked) or all kept.
+// DARE + TA on one 16-element group whose t0 and first kDareBatch experts are
+// already loaded; keep flags from shared memory (masked) or all kept.
 template <int DT>
 __device__ __forceinline__ void dare_linear16(const MArgs& m, const MTensor& T, int t, int64_t i, bool masked,
-                                              const Raw16<DT>& t0, Raw16<DT> (&x)[kExpertBatch],
+                                              const Raw16<DT>& t0, Raw16<DT> (&x)[kDareBatch<DT>],
                                               const DareShared& s) {
-  float2 acc[8];
+  float2 acc[8], b0[8];
 #pragma unroll
-  for (int h = 0; h < 8; ++h) acc[h] = splat(0.0f);
+  for (int h = 0; h < 8; ++h) {
+    acc[h] = splat(0.0f);
+    b0[h] = t0.pair(h);
+    asm volatile("" : "+f"(b0[h].x), "+f"(b0[h].y));  // kept unpacked, not unpacked again for every expert
+  }
   const void* const* xp = m.experts + t * m.K;
   bool blend = false;
   if (DT == DT_BF16) blend = !nonfinite16(*reinterpret_cast<const Raw16<DT_BF16>*>(&t0));
 #pragma unroll 1
-  for (int e = 0; e < m.K; e += kExpertBatch) {
+  for (int e = 0; e < m.K; e += kDareBatch<DT>) {
+    if (e > 0) {
 #pragma unroll
-    for (int b = 0; b < kExpertBatch; ++b)
-      if ((e > 0 || b >= kDarePrefetch<DT>) && e + b < m.K) load16<DT>(xp[e + b], i, x[b]);
+      for (int b = 0; b < kDareBatch<DT>; ++b)
+        if (e + b < m.K) load16<DT>(xp[e + b], i, x[b]);
+    }
 #pragma unroll
-    for (int b = 0; b < kExpertBatch; ++b) {
+    for (int b = 0; b < kDareBatch<DT>; ++b) {
       if (e + b < m.K) {
         const uint4 km = masked ? s.keep[(e + b) * kBlock + threadIdx.x]
-                                : make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
+                                : make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
         if (DT == DT_BF16 && blend)
           dare_acc16_blend(m.c, km, *reinterpret_cast<const Raw16<DT_BF16>*>(&x[b]),
-                           *reinterpret_cast<const Raw16<DT_BF16>*>(&t0), acc);
+                           *reinterpret_cast<const Raw16<DT_BF16>*>(&t0), b0, acc);
         else
           dare_acc16_select<DT>(m.c, km, x[b], t0, acc);
       }
@@ -515,10 +507,10 @@ __global__ void __launch_bounds__(kBlock, 2) merge_kernel(const __grid_constant_
 template <int R, int DT>
 __global__ void __launch_bounds__(kBlock, 2) dare_kernel(const __grid_constant__ MArgs m) {
   extern __shared__ __align__(16) unsigned char dare_smem[];
-  DareShared s;
-  s.qs = reinterpret_cast<DareQueue*>(dare_smem);
-  s.keep = reinterpret_cast<uint4*>(dare_smem + kDareQueueBytes);
   const int warp = threadIdx.x >> 5;
+  DareShared s;
+  s.keep = reinterpret_cast<uint4*>(dare_smem);
+  s.queue = reinterpret_cast<uint16_t*>(s.keep + m.K * kBlock) + 32 * m.K * warp;
   for (int64_t ci = blockIdx.x; ci < m.n_chunks; ci += gridDim.x) {
     const Chunk ch = m.chunks[ci];
     const MTensor& T = m.tensors[ch.tensor];
@@ -528,11 +520,11 @@ __global__ void __launch_bounds__(kBlock, 2) dare_kernel(const __grid_constant__
     for (int64_t base = ch.begin; base < ch.end; base += 16 * (int64_t)kBlock) {
       const int64_t i = base + 16 * (int64_t)threadIdx.x;
       const bool full = vec && i + 16 <= ch.end;
-      Raw16<DT> t0, x[kExpertBatch];
+      Raw16<DT> t0, x[kDareBatch<DT>];
       if (full) {
         load16<DT>(T.theta0, i, t0);
 #pragma unroll
-        for (int b = 0; b < kDarePrefetch<DT>; ++b)
+        for (int b = 0; b < kDareBatch<DT>; ++b)
           if (b < m.K) load16<DT>(xp[b], i, x[b]);
       }
       if (masked)

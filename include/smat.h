@@ -282,9 +282,11 @@ smat_status smat_debug_philox(const uint32_t* d_ctr, int64_t n, uint64_t seed, i
 
 /* Test hook: the unit noise transform of n raw noise words d_words (device):
  * d_out[i] = sym(w) = (2 (w >> 8) + 1 - 2^24) 2^-24 for SMAT_NOISE_UNIFORM,
- * erfinv(sym(w)) as the forward evaluates it for SMAT_NOISE_GAUSSIAN, or
- * -sign(v) ln(1 - |v|), v = sym(w), for SMAT_NOISE_LAPLACE (the forward scales
- * these by fl(sqrt3 sigma), fl(sqrt2 sigma) and fl(sigma / sqrt2)). */
+ * erfinv(sym(w)) for SMAT_NOISE_GAUSSIAN, or -sign(v) ln(1 - |v|), v = sym(w),
+ * for SMAT_NOISE_LAPLACE. The forward scales these by fl(sqrt3 sigma),
+ * fl(sqrt2 sigma) and fl(sigma / sqrt2); for the Gaussian law it scales the
+ * same ratio erfinv(v) / v and takes the product with v and the sum with the
+ * element in one multiply-add. */
 smat_status smat_debug_noise_unit(const uint32_t* d_words, int64_t n, int32_t noise, float* d_out,
                                   smat_stream_t stream);
 

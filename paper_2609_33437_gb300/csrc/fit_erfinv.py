@@ -1,5 +1,6 @@
 """Fit the polynomial coefficients of the device erfinv used by the Gaussian
-Perturb transform (smat_device.cuh: erfinv_poly, erfinv_poly2, erfinv_central2).
+Perturb transform (smat_device.cuh: coef_p, coef_q, used by erfinv_ratio and
+erfinv_central2).
 
 Method (structure of M. Giles, "Approximating the erfinv function", GPU
 Computing Gems Jade Edition, 2011; coefficients fitted here): for
@@ -20,11 +21,11 @@ import mpmath as mp
 import numpy as np
 
 mp.mp.dps = 40
-L0 = -8.0          # central / tail boundary in log2(1 - x^2)
-DEG_P = 9
-DEG_Q = 9
+L0 = -10.0         # central / tail boundary in log2(1 - x^2)
+DEG_P = 10
+DEG_Q = 7
 S_MAX = float(mp.sqrt(23.0)) + 1e-3
-S_MID = 3.8125     # tail Horner variable s - S_MID (exact in fp32), |s - S_MID| <= 1
+S_MID = 4.0        # tail Horner variable s - S_MID (exact in fp32), |s - S_MID| <= 1
 
 
 def f_central(L):
@@ -46,17 +47,19 @@ def fit(func, lo, hi, deg, shift=0.0, n=400):
     k = np.arange(n)
     nodes = 0.5 * (lo + hi) + 0.5 * (hi - lo) * np.cos(np.pi * (k + 0.5) / n)
     y = np.array([float(func(v)) for v in nodes])
-    # relative-error least squares in the monomial basis of (variable - shift)
-    V = np.vander(nodes - shift, deg + 1, increasing=True) / y[:, None]
+    # relative-error least squares in the monomial basis of the variable scaled
+    # to magnitude 1 (unscaled, the high powers spoil the fit's conditioning)
+    scale = max(abs(lo - shift), abs(hi - shift))
+    V = np.vander((nodes - shift) / scale, deg + 1, increasing=True) / y[:, None]
     c, *_ = np.linalg.lstsq(V, np.ones_like(y), rcond=None)
     # a few Lawson-style reweightings toward minimax
     w = np.ones_like(y)
-    for _ in range(30):
+    for _ in range(40):
         r = V @ c - 1.0
         w = w * (np.abs(r) + 1e-30) ** 0.5
         w /= w.max()
         c, *_ = np.linalg.lstsq(V * w[:, None], w, rcond=None)
-    return c  # increasing powers
+    return c / scale ** np.arange(deg + 1)  # increasing powers
 
 
 def horner_f32(c, v):
@@ -92,8 +95,8 @@ def main():
     v = (s - np.float32(S_MID)).astype(np.float32)
     y[~central] = (x[~central].astype(np.float64) * horner_f32(cQ, v).astype(np.float64)).astype(np.float32)
     rel = np.abs(y.astype(np.float64) - ref) / ref
-    print("max rel error: central %.3g, tail %.3g (fp32 ulp 5.96e-8); tail fraction %.4g"
-          % (rel[central].max(), rel[~central].max(), (~central).mean()))
+    print("max rel error: central %.3g, tail %.3g, root mean square %.3g (fp32 ulp 5.96e-8); tail fraction %.4g"
+          % (rel[central].max(), rel[~central].max(), np.sqrt(np.mean(rel**2)), (~central).mean()))
     # sensitivity to the hardware log2 (absolute error up to ~2^-22)
     for dL in (2.0**-22, -2.0**-22):
         Lp = (L.astype(np.float64) + dL).astype(np.float32)

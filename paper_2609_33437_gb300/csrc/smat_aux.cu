@@ -123,7 +123,7 @@ __global__ void debug_noise_unit_kernel(const uint32_t* words, int64_t n, int no
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const float x = sym24(words[i] >> 8);
-    out[i] = (noise == NOISE_GAUSSIAN) ? erfinv_poly(x) : (noise == NOISE_LAPLACE) ? laplace_unit(x) : x;
+    out[i] = (noise == NOISE_GAUSSIAN) ? __fmul_rn(x, erfinv_ratio(x)) : (noise == NOISE_LAPLACE) ? laplace_unit(x) : x;
   }
 }
 
@@ -147,7 +147,7 @@ cudaError_t launch_simulate(const KArgs& a, int grid, int dtype, int noise, bool
 }
 
 cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise, bool per_elem_alpha,
-                                  int rounds, bool inplace, bool wide, cudaStream_t s) {
+                                  int rounds, bool inplace, cudaStream_t s) {
   if (noise == NOISE_LAPLACE)
     return dtype == DT_BF16 ? SMAT_BY_FAMILY(launch_laplace_bf16)(a, grid, true, per_elem_alpha, inplace, s)
                             : SMAT_BY_FAMILY(launch_laplace_f32)(a, grid, true, per_elem_alpha, inplace, s);
@@ -155,7 +155,7 @@ cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise
     return dtype == DT_BF16
                ? SMAT_BY_FAMILY(launch_stats_simulate_inplace_bf16)(a, grid, noise, per_elem_alpha, rounds, s)
                : SMAT_BY_FAMILY(launch_stats_simulate_inplace_f32)(a, grid, noise, per_elem_alpha, rounds, s);
-  return dtype == DT_BF16 ? SMAT_BY_FAMILY(launch_stats_simulate_bf16)(a, grid, noise, per_elem_alpha, rounds, wide, s)
+  return dtype == DT_BF16 ? SMAT_BY_FAMILY(launch_stats_simulate_bf16)(a, grid, noise, per_elem_alpha, rounds, s)
                           : SMAT_BY_FAMILY(launch_stats_simulate_f32)(a, grid, noise, per_elem_alpha, rounds, s);
 }
 

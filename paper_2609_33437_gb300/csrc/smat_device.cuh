@@ -114,45 +114,49 @@ __device__ __forceinline__ float sym24(uint32_t u) {
   return __fmaf_rn(__uint2float_rn(u), kSymScale, kSymShift);
 }
 
-// erfinv(x) for |x| <= 1 - 2^-24 (every value sym24() produces), after the
-// structure of M. Giles, "Approximating the erfinv function" (GPU Computing
-// Gems Jade Edition, 2011), with coefficients fitted for this form by
-// csrc/fit_erfinv.py: with L = log2(1 - x^2) (one fused multiply-add and the
-// hardware log2),
-//   L >= -8:  erfinv(x) = x * P(L)                 (degree 9, 99.8% of inputs)
-//   L <  -8:  erfinv(x) = x * Q(sqrt(-L) - 3.8125)  (degree 9)
-// Both ratios erfinv(x) / x are even in x, so the result is exactly odd.
-// Relative error about 2e-7 (a few fp32 ulps); the tests bound it.
-__device__ __forceinline__ float erfinv_poly(float x) {
-  const float t = __fmaf_rn(-x, x, 1.0f);
+// erfinv(x) / x for |x| <= 1 - 2^-24 (every value sym24() produces), after
+// the structure of M. Giles, "Approximating the erfinv function" (GPU
+// Computing Gems Jade Edition, 2011), with coefficients fitted for this form
+// by csrc/fit_erfinv.py: with L = log2(1 - x^2) (one fused multiply-add and
+// the hardware log2),
+//   L >= -10:  P(L)             (degree 10, 99.95% of inputs)
+//   L <  -10:  Q(sqrt(-L) - 4)  (degree 7)
+// Both are even in x, so x times the ratio is exactly odd. Relative error at
+// most 1.3e-7 (central) and 1.4e-7 (tail), 3.4e-8 in the mean square; the tests
+// bound it. A 16-element group with a tail element is done again by the element
+// path: 0.8% of the groups, where -8 with degree 9 left 3.1% and the forward
+// took 1 to 2% longer for the shorter polynomial (vision-language list).
+constexpr float kCentralL = -10.0f;
+__device__ __forceinline__ float coef_p(int k) {  // increasing powers; k is a constant after unrolling
+  constexpr float c[11] = {8.862268925e-01f, -1.608197540e-01f, 5.548856221e-03f, 7.783531910e-04f,
+                           -2.820832924e-05f, -6.361147825e-06f, 7.189328244e-07f, 2.113999500e-07f,
+                           1.929385540e-08f, 8.415084740e-10f, 1.491148871e-11f};
+  return c[k];
+}
+__device__ __forceinline__ float coef_q(int k) {
+  constexpr float c[8] = {3.164558649e+00f, 8.375940323e-01f, 3.158505773e-03f, -1.759567996e-03f,
+                          9.093442350e-04f, -5.168370553e-04f, 2.645634813e-04f, -7.838992315e-05f};
+  return c[k];
+}
+__device__ __forceinline__ float lg2_approx(float t) {
   float L;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(L) : "f"(t));
+  return L;
+}
+__device__ __forceinline__ float erfinv_ratio(float x) {
+  const float L = lg2_approx(-__fmaf_rn(x, x, -1.0f));
   float p;
-  if (L >= -8.0f) {
-    p = 2.676246447e-10f;
-    p = __fmaf_rn(p, L, 9.962457526e-09f);
-    p = __fmaf_rn(p, L, 1.280022701e-07f);
-    p = __fmaf_rn(p, L, 2.725655577e-07f);
-    p = __fmaf_rn(p, L, -7.822631233e-06f);
-    p = __fmaf_rn(p, L, -3.107573502e-05f);
-    p = __fmaf_rn(p, L, 7.751958910e-04f);
-    p = __fmaf_rn(p, L, 5.547157954e-03f);
-    p = __fmaf_rn(p, L, -1.608200818e-01f);
-    p = __fmaf_rn(p, L, 8.862268925e-01f);
+  if (L >= kCentralL) {
+    p = coef_p(10);
+#pragma unroll
+    for (int k = 9; k >= 0; --k) p = __fmaf_rn(p, L, coef_p(k));
   } else {
-    const float v = __fsub_rn(sqrtf(-L), 3.8125f);
-    p = 2.205743658e-05f;
-    p = __fmaf_rn(p, v, -2.623226646e-05f);
-    p = __fmaf_rn(p, v, -9.935771232e-05f);
-    p = __fmaf_rn(p, v, 3.947049263e-04f);
-    p = __fmaf_rn(p, v, -8.652319084e-04f);
-    p = __fmaf_rn(p, v, 1.542331069e-03f);
-    p = __fmaf_rn(p, v, -2.662600018e-03f);
-    p = __fmaf_rn(p, v, 4.380439408e-03f);
-    p = __fmaf_rn(p, v, 8.361965418e-01f);
-    p = __fmaf_rn(p, v, 3.007633686e+00f);
+    const float v = __fsub_rn(sqrtf(-L), 4.0f);
+    p = coef_q(7);
+#pragma unroll
+    for (int k = 6; k >= 0; --k) p = __fmaf_rn(p, v, coef_q(k));
   }
-  return __fmul_rn(x, p);
+  return p;
 }
 
 // Packed fp32 pairs (sm_100 and later): two independent IEEE operations with
@@ -202,17 +206,9 @@ __device__ __forceinline__ float2 fma2_rn(float2 a, float2 b, float2 c) {
   return d;
 }
 
-// sym24 of two 24-bit noise fields: (2u + 1 - 2^24) 2^-24, exact. Two
-// equivalent forms (identical values): an integer multiply-add, conversion
-// and multiply, or a conversion and one fused multiply-add (see sym24). The
-// Gaussian path measures faster with the second, the uniform path with the
-// first.
-template <bool FMA_FORM>
+// sym24 of two 24-bit noise fields.
 __device__ __forceinline__ float2 sym2(uint32_t u0, uint32_t u1) {
-  if (FMA_FORM)
-    return fma2_rn(make_float2(__uint2float_rn(u0), __uint2float_rn(u1)), splat(kSymScale), splat(kSymShift));
-  const float2 m = make_float2(__int2float_rn(2 * (int)u0 + 1 - (1 << 24)), __int2float_rn(2 * (int)u1 + 1 - (1 << 24)));
-  return mul2_rn(m, splat(5.9604644775390625e-08f));
+  return fma2_rn(make_float2(__uint2float_rn(u0), __uint2float_rn(u1)), splat(kSymScale), splat(kSymShift));
 }
 
 // 16-bit option: (2u + 1 - 2^16) 2^-16 of two 16-bit draws as one conversion
@@ -227,10 +223,10 @@ __device__ __forceinline__ float sym16(uint32_t u) {
   return __fmaf_rn(__uint2float_rn(u), kSym16Scale, kSym16Shift);
 }
 // The symmetric uniform of two draws of the variant (sym24 or sym16).
-template <bool D16, bool FMA_FORM>
+template <bool D16>
 __device__ __forceinline__ float2 sym2v(uint32_t u0, uint32_t u1) {
   if constexpr (D16) return sym2_16(u0, u1);
-  else return sym2<FMA_FORM>(u0, u1);
+  else return sym2(u0, u1);
 }
 
 // The four 24-bit noise fields of a quad from its three noise words A, B, C:
@@ -254,34 +250,6 @@ __device__ __forceinline__ void halves_of(const uint4& b, int hi, uint32_t (&u)[
   u[3] = w1 >> 16;
 }
 
-__device__ __forceinline__ float lg2_approx(float t) {
-  float L;
-  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(L) : "f"(t));
-  return L;
-}
-
-// erfinv_poly on a pair: the central polynomial with packed multiply-adds
-// when both lanes are central (99.6% of pairs), else lane by lane.
-__device__ __forceinline__ float2 erfinv_poly2(float2 x) {
-  const float2 t = fma2_rn(make_float2(-x.x, -x.y), x, splat(1.0f));
-  const float2 L = make_float2(lg2_approx(t.x), lg2_approx(t.y));
-  float2 p;
-  if (fminf(L.x, L.y) >= -8.0f) {
-    p = splat(2.676246447e-10f);
-    p = fma2_rn(p, L, splat(9.962457526e-09f));
-    p = fma2_rn(p, L, splat(1.280022701e-07f));
-    p = fma2_rn(p, L, splat(2.725655577e-07f));
-    p = fma2_rn(p, L, splat(-7.822631233e-06f));
-    p = fma2_rn(p, L, splat(-3.107573502e-05f));
-    p = fma2_rn(p, L, splat(7.751958910e-04f));
-    p = fma2_rn(p, L, splat(5.547157954e-03f));
-    p = fma2_rn(p, L, splat(-1.608200818e-01f));
-    p = fma2_rn(p, L, splat(8.862268925e-01f));
-    return mul2_rn(x, p);
-  }
-  return make_float2(erfinv_poly(x.x), erfinv_poly(x.y));
-}
-
 // Laplace(0, 1) variate of v in (-1, 1) by the inverse CDF, -sign(v) ln(1 -
 // |v|): 1 - |v| is exact in fp32 for every noise-grid v, and log1pf of -|v|
 // keeps full relative accuracy for small |v|.
@@ -289,64 +257,53 @@ __device__ __forceinline__ float laplace_unit(float v) {
   return copysignf(-log1pf(-fabsf(v)), v);
 }
 
-// The group path's erfinv of a pair: the central polynomial only (packed,
-// branch free). minL collects the smallest L = log2(1 - x^2) seen, computed
-// exactly as erfinv_poly computes it; an element with L < -8 belongs to the
-// tail and its value here is wrong: the caller queues its group and rewrites
-// it through the element path (erfinv_poly).
+// The group path's erfinv(x) / x of a pair: the central polynomial only
+// (packed, branch free). minL collects the smallest L = log2(1 - x^2) seen,
+// computed exactly as erfinv_ratio computes it; an element with L < kCentralL
+// belongs to the tail and its value here is wrong: the caller queues its group
+// and rewrites it through the element path.
 __device__ __forceinline__ float2 erfinv_central2(float2 x, float& minL) {
-  const float2 t = fma2_rn(make_float2(-x.x, -x.y), x, splat(1.0f));
-  const float2 L = make_float2(lg2_approx(t.x), lg2_approx(t.y));
+  const float2 t = fma2_rn(x, x, splat(-1.0f));
+  const float2 L = make_float2(lg2_approx(-t.x), lg2_approx(-t.y));
   minL = fminf(minL, fminf(L.x, L.y));
-  float2 p = splat(2.676246447e-10f);
-  p = fma2_rn(p, L, splat(9.962457526e-09f));
-  p = fma2_rn(p, L, splat(1.280022701e-07f));
-  p = fma2_rn(p, L, splat(2.725655577e-07f));
-  p = fma2_rn(p, L, splat(-7.822631233e-06f));
-  p = fma2_rn(p, L, splat(-3.107573502e-05f));
-  p = fma2_rn(p, L, splat(7.751958910e-04f));
-  p = fma2_rn(p, L, splat(5.547157954e-03f));
-  p = fma2_rn(p, L, splat(-1.608200818e-01f));
-  p = fma2_rn(p, L, splat(8.862268925e-01f));
-  return mul2_rn(x, p);
+  float2 p = splat(coef_p(10));
+#pragma unroll
+  for (int k = 9; k >= 0; --k) p = fma2_rn(p, L, splat(coef_p(k)));
+  return p;
 }
 
-// Group-path noise of a pair (see erfinv_central2 for minL); D16: the two
-// draws are 16-bit.
-template <int NOISE, bool D16 = false>
-__device__ __forceinline__ float2 noise_group2(uint32_t n0, uint32_t n1, float2 scale, float& minL) {
-  if (NOISE == NOISE_UNIFORM) return mul2_rn(scale, sym2v<D16, false>(n0, n1));
-  if (NOISE == NOISE_GAUSSIAN) return mul2_rn(scale, erfinv_central2(sym2v<D16, true>(n0, n1), minL));
-  if (NOISE == NOISE_LAPLACE) {
-    const float2 v = sym2v<D16, true>(n0, n1);
-    return mul2_rn(scale, make_float2(laplace_unit(v.x), laplace_unit(v.y)));
+// x plus the Perturb of a pair whose draws are n0, n1 (24-bit fields, or
+// 16-bit draws with D16), given the law's factor at RMS sigma: uniform
+// scale sym(u), each operation rounded, with scale = fl(sqrt3 sigma);
+// Gaussian scale erfinv(sym(u)) with scale = fl(sqrt2 sigma) (inverse-CDF
+// transform: sqrt2 erfinv(v) is N(0, 1) for v uniform on (-1, 1)), taken as
+// one multiply-add (scale ratio) v + x, which rounds twice less than product,
+// scaling and sum and is two instructions shorter; Laplace scale z(v), one
+// multiply-add too. CENTRAL: the group path's central polynomial (minL as in
+// erfinv_central2).
+template <int NOISE, bool D16, bool CENTRAL>
+__device__ __forceinline__ float2 perturb2(float2 x, uint32_t n0, uint32_t n1, float2 scale, float& minL) {
+  if (NOISE == NOISE_UNIFORM) {
+    const float2 eps = mul2_rn(scale, sym2v<D16>(n0, n1));
+    return make_float2(__fadd_rn(x.x, eps.x), __fadd_rn(x.y, eps.y));
   }
-  return splat(0.0f);
-}
-
-// Perturb of one element from its 24-bit noise field u: uniform
-// scale * sym24(u) with scale = fl(sqrt3 sigma), or Gaussian
-// scale * erfinv(sym24(u)) with
-// scale = fl(sqrt2 sigma) (inverse-CDF transform: sqrt2 erfinv(v) is
-// N(0, 1) for v uniform on (-1, 1)).
-template <int NOISE, bool D16 = false>
-__device__ __forceinline__ float2 noise_of2(uint32_t n0, uint32_t n1, float2 scale) {
-  if (NOISE == NOISE_UNIFORM) return mul2_rn(scale, sym2v<D16, false>(n0, n1));
-  if (NOISE == NOISE_GAUSSIAN) return mul2_rn(scale, erfinv_poly2(sym2v<D16, true>(n0, n1)));
-  if (NOISE == NOISE_LAPLACE) {
-    const float2 v = sym2v<D16, true>(n0, n1);
-    return mul2_rn(scale, make_float2(laplace_unit(v.x), laplace_unit(v.y)));
+  const float2 v = sym2v<D16>(n0, n1);
+  if (NOISE == NOISE_GAUSSIAN) {
+    const float2 p = CENTRAL ? erfinv_central2(v, minL) : make_float2(erfinv_ratio(v.x), erfinv_ratio(v.y));
+    return fma2_rn(mul2_rn(scale, p), v, x);
   }
-  return splat(0.0f);
+  if (NOISE == NOISE_LAPLACE) return fma2_rn(scale, make_float2(laplace_unit(v.x), laplace_unit(v.y)), x);
+  return x;
 }
 
-template <int NOISE, bool D16 = false>
-__device__ __forceinline__ float noise_of(uint32_t u, float scale) {
+// The same for one element.
+template <int NOISE, bool D16>
+__device__ __forceinline__ float perturb1(float x, uint32_t u, float scale) {
   const float v = D16 ? sym16(u) : sym24(u);
-  if (NOISE == NOISE_UNIFORM) return __fmul_rn(scale, v);
-  if (NOISE == NOISE_GAUSSIAN) return __fmul_rn(scale, erfinv_poly(v));
-  if (NOISE == NOISE_LAPLACE) return __fmul_rn(scale, laplace_unit(v));
-  return 0.0f;
+  if (NOISE == NOISE_UNIFORM) return __fadd_rn(x, __fmul_rn(scale, v));
+  if (NOISE == NOISE_GAUSSIAN) return __fmaf_rn(__fmul_rn(scale, erfinv_ratio(v)), v, x);
+  if (NOISE == NOISE_LAPLACE) return __fmaf_rn(scale, laplace_unit(v), x);
+  return x;
 }
 
 // The draw of one element (any alignment) in the NOISE or ALPHA_E stream: its
@@ -396,11 +353,12 @@ __device__ __forceinline__ bool kept_of(const uint32_t (&kw)[4], int e) {
 // high byte of each element's 32-bit mask uniform comes from one MASK block
 // (byte b of word q serves element 4q + b); it is compared with the
 // threshold's high byte four bytes at a time (SWAR, no carries between
-// bytes). Bit 8b + 7 of kw[q] is element 4q + b's flag. Returns whether some
-// byte equals the threshold's high byte (probability 1/256 per element): such
-// a tie is decided by the low 24 bits of the uniform (MASK_LO stream), which
-// the caller resolves (group_ties16 / resolve_group_ties); its flag is left
-// clear here.
+// bytes), six operations per word. Bit 8b + 7 of kw[q] is element 4q + b's
+// flag, its other bits are not defined (the readers look at no other). Returns
+// whether some byte equals the threshold's high byte (probability 1/256 per
+// element): such a tie is decided by the low 24 bits of the uniform (MASK_LO
+// stream), which the caller resolves (group_ties16 / resolve_group_ties); its
+// flag is left clear here.
 __device__ __forceinline__ bool keep_bytes16(const uint4& w, uint32_t t_hi, uint32_t (&kw)[4]) {
   const uint32_t words[4] = {w.x, w.y, w.z, w.w};
   const uint32_t tt = t_hi * 0x01010101u;
@@ -408,14 +366,11 @@ __device__ __forceinline__ bool keep_bytes16(const uint4& w, uint32_t t_hi, uint
   uint32_t anytie = 0u;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const uint32_t x = words[q];
-    // bit 7 of each byte of d: low 7 bits of x >= low 7 bits of t
-    const uint32_t d = (x | 0x80808080u) - tl;
-    kw[q] = ((~x & tt) | (~(x ^ tt) & ~d)) & 0x80808080u;  // x < t per byte
-    const uint32_t e = x ^ tt;
-    anytie |= (e - 0x01010101u) & ~e & 0x80808080u;  // nonzero iff some byte equals t
+    const uint32_t x = words[q], d = (x | 0x80808080u) - tl, e = x ^ tt, s = e - 0x01010101u;
+    asm("lop3.b32 %0, %1, %2, %3, 0x4D;" : "=r"(kw[q]) : "r"(x), "r"(tt), "r"(d));        // (~x & tt) | (~(x ^ tt) & ~d)
+    asm("lop3.b32 %0, %1, %2, %3, 0xBA;" : "=r"(anytie) : "r"(s), "r"(e), "r"(anytie));  // (s & ~e) | anytie
   }
-  return anytie != 0u;
+  return (anytie & 0x80808080u) != 0u;
 }
 // 16-bit option: keep flags of the 16 elements gidx0 .. gidx0 + 15 (gidx0 %
 // 16 == 0) from the two MASK blocks gidx0 / 8 and gidx0 / 8 + 1 (half h of

@@ -8,15 +8,18 @@
 namespace smat {
 
 cudaError_t SMAT_FAMILY(launch_stats_simulate_bf16)(const KArgs& a, int grid, int noise, bool per_elem_alpha,
-                                                    int rounds, bool wide, cudaStream_t s) {
+                                                    int rounds, cudaStream_t s) {
   if (a.n_items <= 0) return cudaSuccess;
-  return (rounds & 0xFF) == 7 ? fused_run<7 | kFamily, DT_BF16, false>(a, grid, noise, per_elem_alpha, wide, s)
-                              : fused_run<10 | kFamily, DT_BF16, false>(a, grid, noise, per_elem_alpha, wide, s);
+  return (rounds & 0xFF) == 7 ? fused_run<7 | kFamily, DT_BF16, false>(a, grid, noise, per_elem_alpha, s)
+                              : fused_run<10 | kFamily, DT_BF16, false>(a, grid, noise, per_elem_alpha, s);
 }
 
 int SMAT_FAMILY(fused_wide_ctas_per_sm)(int noise, int rounds) {
-  return (rounds & 0xFF) == 7 ? fused_occ<7 | kFamily, DT_BF16, false>(noise, false, true)
-                              : fused_occ<10 | kFamily, DT_BF16, false>(noise, false, true);
+#define SMAT_WIDE_OCC(R) \
+  (noise == NOISE_GAUSSIAN ? FusedVariant<R, DT_BF16, NOISE_GAUSSIAN, false, false>::occ() \
+                           : FusedVariant<R, DT_BF16, NOISE_UNIFORM, false, false>::occ())
+  return (rounds & 0xFF) == 7 ? SMAT_WIDE_OCC(7 | kFamily) : SMAT_WIDE_OCC(10 | kFamily);
+#undef SMAT_WIDE_OCC
 }
 
 }  // namespace smat

@@ -250,7 +250,7 @@ struct smat_ctx {
   bool adams_uploaded = false;
   // work-list forward launch (with the statistics of sigma_rel tensors)
   bool fused = false;
-  bool wide = false;  // the bf16 fused launch carries statistics items: its four-CTA build
+  bool wide = false;  // the bf16 work-list launch is the four-CTA build
   std::vector<int32_t> h_items;
   int32_t item_begin[kMaxRanges] = {0, 0};
   int32_t item_count[kMaxRanges] = {0, 0};
@@ -355,6 +355,13 @@ int grid_for(const smat_ctx* c, int64_t chunks, int dtype) {
   const int64_t resident = (int64_t)c->sm_count *
                            streaming_ctas_per_sm(dtype, c->cfg.noise, c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT, c->rounds);
   return (int)(chunks < resident ? chunks : resident);
+}
+
+// Grid of the work-list launch of one dtype range.
+int fused_grid(const smat_ctx* c, int dt) {
+  const int64_t chunks = c->range_end[dt] - c->range_begin[dt];
+  if (!(c->wide && dt == SMAT_BF16)) return grid_for(c, chunks, dt);
+  return (int)std::min(chunks, (int64_t)c->sm_count * fused_wide_occ(c->cfg.noise, c->rounds));
 }
 
 // Rows a2 + a1: delta statistics (if needed) then the per-call scalars.
@@ -505,7 +512,7 @@ smat_status smat_init(smat_ctx** out, const smat_tensor_desc* tensors, int32_t n
     e = cudaMemcpyAsync(c->d_chunks, c->h_chunks.data(), sizeof(Chunk) * (size_t)nc,
                         cudaMemcpyHostToDevice, stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_sync, 0, sizeof(int32_t) * sync_words(n_tensors), stream);
-  c->wide = rel && cfg->alpha_mode != SMAT_ALPHA_PER_ELEMENT && cfg->noise != SMAT_NOISE_LAPLACE && !c->any_inplace;
+  c->wide = cfg->alpha_mode != SMAT_ALPHA_PER_ELEMENT && cfg->noise != SMAT_NOISE_LAPLACE && !c->any_inplace;
   if (e == cudaSuccess && c->fused) {
     // lead of about one grid width of the bf16 forward (one, two and four
     // measured on the 7B list: one is fastest)
@@ -551,16 +558,10 @@ smat_status smat_simulate_multi(smat_ctx* c, uint32_t step, smat_stream_t stream
       a.items = c->d_items + c->item_begin[dt];
       a.n_items = c->item_count[dt];
       a.work_counter = c->d_sync + dt;
-      const bool wide = c->wide && dt == SMAT_BF16;
-      int grid = grid_for(c, c->range_end[dt] - c->range_begin[dt], dt);
-      if (wide) {
-        const int64_t chunks = c->range_end[dt] - c->range_begin[dt];
-        const int64_t resident = (int64_t)c->sm_count * fused_wide_occ(c->cfg.noise, c->rounds);
-        grid = (int)(chunks < resident ? chunks : resident);
-      }
+      const int grid = fused_grid(c, dt);
       Timed t(c, 2, stream);
       const cudaError_t e = launch_stats_simulate(a, grid, dt, c->cfg.noise, c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT,
-                                                  c->rounds, c->any_inplace, wide, stream);
+                                                  c->rounds, c->any_inplace, stream);
       t.done();
       if (e != cudaSuccess) return cuda_fail(e, "fused statistics + forward launch");
     }
@@ -848,8 +849,8 @@ smat_status smat_debug_fused(smat_ctx* c, uint32_t step, const int32_t* d_items,
   a.items = d_items;
   a.n_items = n_items;
   a.work_counter = c->d_sync + SMAT_BF16;
-  e = launch_stats_simulate_bf16(a, grid_for(c, c->range_end[SMAT_BF16] - c->range_begin[SMAT_BF16], SMAT_BF16),
-                                 c->cfg.noise, c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT, c->rounds, false, stream);
+  e = launch_stats_simulate_bf16(a, fused_grid(c, SMAT_BF16), c->cfg.noise,
+                                 c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT, c->rounds, stream);
   if (e != cudaSuccess) return cuda_fail(e, "fused launch");
   c->scalars_step = -1;  // sigma_t of this call may be incomplete
   c->sim_step = -1;      // and its forward too

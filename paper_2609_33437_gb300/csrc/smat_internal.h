@@ -150,10 +150,8 @@ cudaError_t launch_delta_stats(const KArgs& a, int grid, int dtype, cudaStream_t
 cudaError_t launch_scalars(const KArgs& a, int noise, int rounds, cudaStream_t s);
 cudaError_t launch_simulate(const KArgs& a, int grid, int dtype, int noise, bool per_elem_alpha,
                             int rounds, bool inplace, cudaStream_t s);
-// wide: the list has statistics items (bf16 without per-element alpha, not
-// in place, uniform or Gaussian noise: the four-CTA-per-SM build).
 cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise, bool per_elem_alpha,
-                                  int rounds, bool inplace, bool wide, cudaStream_t s);
+                                  int rounds, bool inplace, cudaStream_t s);
 // The forward launchers below exist twice: as declared (the packed draw
 // layout) and with the suffix _d16 (the 16-bit draw option). Each forward
 // translation unit is compiled once per family (SMAT_DRAW16 defined for the
@@ -169,8 +167,8 @@ cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise
   cudaError_t launch_stats_simulate_f32##sfx(const KArgs& a, int grid, int noise, bool per_elem_alpha,        \
                                              int rounds, cudaStream_t s);                                     \
   cudaError_t launch_stats_simulate_bf16##sfx(const KArgs& a, int grid, int noise, bool per_elem_alpha,       \
-                                              int rounds, bool wide, cudaStream_t s);                         \
-  /* Resident CTAs per SM of the four-CTA build (bf16, uniform or Gaussian). */                              \
+                                              int rounds, cudaStream_t s);                                    \
+  /* Resident CTAs per SM of launch_stats_simulate_bf16 (uniform or Gaussian, no per-element alpha). */       \
   int fused_wide_ctas_per_sm##sfx(int noise, int rounds);                                                     \
   /* Laplace noise (10 rounds; smat_laplace_*.cu): the work-list launch when `fused`, else the grid-stride    \
      one; in-place instantiations when `inplace`. */                                                          \
@@ -197,7 +195,7 @@ SMAT_FORWARD_LAUNCHERS()
 SMAT_FORWARD_LAUNCHERS(_d16)
 #undef SMAT_FORWARD_LAUNCHERS
 
-// Family dispatch (smat_aux.cu): the four-CTA build's occupancy and the
+// Family dispatch (smat_aux.cu): the bf16 work-list launch's occupancy and the
 // gradient map for the variant code `rounds`.
 int fused_wide_occ(int noise, int rounds);
 cudaError_t launch_grad_map(const KArgs& a, int grid, int gdtype, bool per_elem_alpha, bool accumulate, int rounds,

@@ -92,25 +92,19 @@ __device__ __forceinline__ uint32_t sim_group16(const KArgs& a, const TView& v, 
       } else {
         kv = fma2_rn(c2, sub2_rn(th2, t02), t02);
       }
-      float x0 = kept_of(kw, e0) ? kv.x : t02.x;
-      float x1 = kept_of(kw, e0 + 1) ? kv.y : t02.y;
-      if (NOISE != NOISE_NONE) {
-        const float2 eps = EXACT ? noise_of2<NOISE, D16>(u[2 * h], u[2 * h + 1], scale2)
-                                 : noise_group2<NOISE, D16>(u[2 * h], u[2 * h + 1], scale2, minL);
-        x0 = __fadd_rn(x0, eps.x);
-        x1 = __fadd_rn(x1, eps.y);
-      }
-      out[e0] = x0;
-      out[e0 + 1] = x1;
+      const float2 x = make_float2(kept_of(kw, e0) ? kv.x : t02.x, kept_of(kw, e0 + 1) ? kv.y : t02.y);
+      const float2 o = perturb2<NOISE, D16, !EXACT>(x, u[2 * h], u[2 * h + 1], scale2, minL);
+      out[e0] = o.x;
+      out[e0 + 1] = o.y;
     }
   }
-  if (!EXACT && NOISE == NOISE_GAUSSIAN && minL < -8.0f) flags |= kQueueTail;
+  if (!EXACT && NOISE == NOISE_GAUSSIAN && minL < kCentralL) flags |= kQueueTail;
   if (!(IP && flags && (v.flags & TF_INPLACE))) store16<DT>(sim_p, i, out);
   return flags;
 }
 
 // Tail elements of the 16-element group at gidx0 (bit e set iff element e's
-// L = log2(1 - x^2) < -8), computed exactly as erfinv_central2 computes L.
+// L = log2(1 - x^2) < kCentralL), computed exactly as erfinv_central2 computes L.
 template <int R, bool J0>
 __device__ __forceinline__ uint32_t group_tails16(const KArgs& a, uint32_t tid, uint64_t gidx0) {
   constexpr bool D16 = draws16<R>();
@@ -133,7 +127,7 @@ __device__ __forceinline__ uint32_t group_tails16(const KArgs& a, uint32_t tid, 
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const float x = D16 ? sym16(u[r]) : sym24(u[r]);
-      if (lg2_approx(__fmaf_rn(-x, x, 1.0f)) < -8.0f) bits |= 1u << (4 * q + r);
+      if (lg2_approx(-__fmaf_rn(x, x, -1.0f)) < kCentralL) bits |= 1u << (4 * q + r);
     }
   }
   return bits;
@@ -150,7 +144,7 @@ __device__ __forceinline__ void sim_elem_as(const KArgs& a, const TView& v, cons
   const float x_th = load1<DT>(th_p, e), x_t0 = load1<DT>(t0_p, e);
   float x = x_t0;
   if (kept) x = (c == 1.0f) ? x_th : __fmaf_rn(c, __fsub_rn(x_th, x_t0), x_t0);
-  if (NOISE != NOISE_NONE) x = __fadd_rn(x, noise_of<NOISE, D16>(field1<R>(a, S_NOISE, v.tid, g), v.noise_scale));
+  if (NOISE != NOISE_NONE) x = perturb1<NOISE, D16>(x, field1<R>(a, S_NOISE, v.tid, g), v.noise_scale);
   store1<DT>(sim_p, e, x);
 }
 
@@ -276,12 +270,18 @@ __device__ __forceinline__ void forward_chunk(const KArgs& a, const TView& v, co
   }
 }
 
-// MINB: CTAs per SM the launch is built for. Lists with statistics items run
-// the bf16 launch at four CTAs per SM (64 registers): the extra warps hide
-// the statistics' memory latency (7B list: 11.98 -> 11.73 ms); forward-only
-// lists keep three (80 registers, no spills in the group path).
-template <int R, int DT, int NOISE, bool PE, bool IP, int MINB = ((DT == DT_BF16 && !PE) ? 3 : 2)>
-__global__ void __launch_bounds__(kBlock, MINB)
+// CTAs per SM the work-list launch is built for. bf16 without per-element alpha
+// runs at four (64 registers): the warps hide the Philox and multiply-add
+// latencies of the forward and the memory latency of the statistics better than
+// three CTAs with 80 registers do (a vision tower with uniform noise 660 -> 628
+// us for the step, 0.5B decoder 663 -> 651 us, vision-language list 3089 -> 3067
+// us, 7B list with statistics 11.98 -> 11.73 ms when it was introduced). In-place
+// and Laplace launches keep three.
+template <int DT, int NOISE, bool PE, bool IP>
+constexpr int kFusedCtas = DT != DT_BF16 || PE ? 2 : (IP || NOISE == NOISE_LAPLACE ? 3 : 4);
+
+template <int R, int DT, int NOISE, bool PE, bool IP>
+__global__ void __launch_bounds__(kBlock, kFusedCtas<DT, NOISE, PE, IP>)
     stats_simulate_kernel(const __grid_constant__ KArgs a) {
   __shared__ double sh_s[kBlock / 32];
   __shared__ double sh_q[kBlock / 32];
@@ -385,43 +385,23 @@ int occupancy_of(Kernel k) {
   return v;
 }
 
-template <int R, int DT, int NOISE, bool PE, bool IP, int MINB = ((DT == DT_BF16 && !PE) ? 3 : 2)>
+template <int R, int DT, int NOISE, bool PE, bool IP>
 struct FusedVariant {
   static int occ() {
-    static int v = occupancy_of(stats_simulate_kernel<R, DT, NOISE, PE, IP, MINB>);
+    static int v = occupancy_of(stats_simulate_kernel<R, DT, NOISE, PE, IP>);
     return v;
   }
   static cudaError_t run(const KArgs& a, int grid, cudaStream_t s) {
-    stats_simulate_kernel<R, DT, NOISE, PE, IP, MINB><<<grid, kBlock, 0, s>>>(a);
+    stats_simulate_kernel<R, DT, NOISE, PE, IP><<<grid, kBlock, 0, s>>>(a);
     return cudaGetLastError();
   }
 };
 
-// wide: the list has statistics items (the four-CTA build for bf16 without
-// per-element alpha and not in place; the other cases have one build).
 template <int R, int DT, bool IP>
-cudaError_t fused_run(const KArgs& a, int grid, int noise, bool pe, bool wide, cudaStream_t s) {
-  if constexpr (DT == DT_BF16 && !IP) {
-    if (wide && !pe)
-      return noise == NOISE_GAUSSIAN ? FusedVariant<R, DT, NOISE_GAUSSIAN, false, IP, 4>::run(a, grid, s)
-                                     : FusedVariant<R, DT, NOISE_UNIFORM, false, IP, 4>::run(a, grid, s);
-  }
+cudaError_t fused_run(const KArgs& a, int grid, int noise, bool pe, cudaStream_t s) {
   if (noise == NOISE_GAUSSIAN)
     return pe ? FusedVariant<R, DT, NOISE_GAUSSIAN, true, IP>::run(a, grid, s) : FusedVariant<R, DT, NOISE_GAUSSIAN, false, IP>::run(a, grid, s);
   return pe ? FusedVariant<R, DT, NOISE_UNIFORM, true, IP>::run(a, grid, s) : FusedVariant<R, DT, NOISE_UNIFORM, false, IP>::run(a, grid, s);
-}
-
-// Resident CTAs per SM of the launch fused_run makes.
-template <int R, int DT, bool IP>
-int fused_occ(int noise, bool pe, bool wide) {
-  if constexpr (DT == DT_BF16 && !IP) {
-    if (wide && !pe)
-      return noise == NOISE_GAUSSIAN ? FusedVariant<R, DT, NOISE_GAUSSIAN, false, IP, 4>::occ()
-                                     : FusedVariant<R, DT, NOISE_UNIFORM, false, IP, 4>::occ();
-  }
-  if (noise == NOISE_GAUSSIAN)
-    return pe ? FusedVariant<R, DT, NOISE_GAUSSIAN, true, IP>::occ() : FusedVariant<R, DT, NOISE_GAUSSIAN, false, IP>::occ();
-  return pe ? FusedVariant<R, DT, NOISE_UNIFORM, true, IP>::occ() : FusedVariant<R, DT, NOISE_UNIFORM, false, IP>::occ();
 }
 
 template <int R, int DT, int NOISE, bool PE, bool IP>

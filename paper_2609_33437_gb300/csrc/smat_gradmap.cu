@@ -77,16 +77,23 @@ __device__ __forceinline__ void grad_elem_as(const KArgs& a, const TView& v, con
   store1<GDT>(G.g_out, e, r);
 }
 
-// Four groups per iteration (strides apart) so each thread keeps four loads
-// of g~ in flight before the mask work (two: 4.39 ms, four: 4.32 ms on the
-// 7B list).
+// Groups per iteration (strides apart). Four keep four loads of g~ in flight per
+// thread before the mask work (7B list: two 4.39 ms, four 4.32 ms). With
+// per-element alpha (three more Philox blocks per group), and with an fp32 sum to
+// read beside g~, four groups' words spill at two or three CTAs per SM: one group
+// at four CTAs is faster (1e8 elements: per-element alpha bf16 150 -> 136 us, fp32
+// 150 -> 141 us; accumulation fp32 207 -> 190 us, with per-element alpha 222 ->
+// 205 us, bf16 159 -> 146 us).
+template <int GDT, bool PE, bool ACC>
+constexpr bool kGradLean = PE || (ACC && GDT == DT_F32);
+
 template <int R, int GDT, bool PE, bool ACC, bool J0>
 __device__ __forceinline__ void grad_chunk(const KArgs& a, const TView& v, const GradPtr& G, const Chunk& ch) {
   constexpr int64_t kStride = 16 * (int64_t)kBlock;
   const bool masked = (v.flags & TF_MASK) != 0u;
   const bool major = G.g_sim == G.g_out || tie_mostly_kept(v.t_lo);
   TieList tl;
-  constexpr int NG = 4;
+  constexpr int NG = kGradLean<GDT, PE, ACC> ? 1 : 4;
   for (int64_t i = ch.begin + 16 * (int64_t)threadIdx.x; i < ch.end; i += NG * kStride) {
     if (G.vec && i + (NG - 1) * kStride + 16 <= ch.end) {
       Raw16<GDT> gs[NG], go[NG];
@@ -164,7 +171,7 @@ __device__ __forceinline__ void grad_chunk(const KArgs& a, const TView& v, const
 }
 
 template <int R, int GDT, bool PE, bool ACC>
-__global__ void __launch_bounds__(kBlock, (GDT == DT_BF16 && !ACC) ? 3 : 2) gradmap_kernel(const __grid_constant__ KArgs a) {
+__global__ void __launch_bounds__(kBlock, kGradLean<GDT, PE, ACC> ? 4 : (GDT == DT_BF16 && !ACC) ? 3 : 2) gradmap_kernel(const __grid_constant__ KArgs a) {
   const int64_t units = a.grad_units;
   for (int64_t u = units * a.chunk_begin + blockIdx.x; u < units * a.chunk_end; u += gridDim.x) {
     Chunk ch = a.chunks[u / units];

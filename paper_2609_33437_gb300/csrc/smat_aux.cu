@@ -164,7 +164,10 @@ int streaming_ctas_per_sm(int dtype, int noise, bool pe, int rounds) {
                           : SMAT_BY_FAMILY(simulate_ctas_per_sm_f32)(noise, pe, rounds);
 }
 
-int fused_wide_occ(int noise, int rounds) { return SMAT_BY_FAMILY(fused_wide_ctas_per_sm)(noise, rounds); }
+int fused_wide_occ(int noise, bool per_elem_alpha, int rounds) {
+  if (noise == NOISE_LAPLACE) return SMAT_BY_FAMILY(laplace_ctas_per_sm_bf16)(per_elem_alpha);
+  return SMAT_BY_FAMILY(fused_wide_ctas_per_sm)(noise, per_elem_alpha, rounds);
+}
 
 cudaError_t launch_grad_map(const KArgs& a, int grid, int gdtype, bool per_elem_alpha, bool accumulate, int rounds,
                             cudaStream_t s) {

@@ -251,10 +251,11 @@ __device__ __forceinline__ void halves_of(const uint4& b, int hi, uint32_t (&u)[
 }
 
 // Laplace(0, 1) variate of v in (-1, 1) by the inverse CDF, -sign(v) ln(1 -
-// |v|): 1 - |v| is exact in fp32 for every noise-grid v, and log1pf of -|v|
-// keeps full relative accuracy for small |v|.
+// |v|): 1 - |v| is exact in fp32 for every noise-grid v, so the logarithm's own
+// rounding (relative, also near 1) is the only one. (log1pf of -|v| is the same
+// value by a longer sequence: 1e8 fp32 elements 247 -> 236 us.)
 __device__ __forceinline__ float laplace_unit(float v) {
-  return copysignf(-log1pf(-fabsf(v)), v);
+  return copysignf(-logf(1.0f - fabsf(v)), v);
 }
 
 // The group path's erfinv(x) / x of a pair: the central polynomial only

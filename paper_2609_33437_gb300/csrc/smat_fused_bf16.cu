@@ -14,11 +14,12 @@ cudaError_t SMAT_FAMILY(launch_stats_simulate_bf16)(const KArgs& a, int grid, in
                               : fused_run<10 | kFamily, DT_BF16, false>(a, grid, noise, per_elem_alpha, s);
 }
 
-int SMAT_FAMILY(fused_wide_ctas_per_sm)(int noise, int rounds) {
-#define SMAT_WIDE_OCC(R) \
-  (noise == NOISE_GAUSSIAN ? FusedVariant<R, DT_BF16, NOISE_GAUSSIAN, false, false>::occ() \
-                           : FusedVariant<R, DT_BF16, NOISE_UNIFORM, false, false>::occ())
-  return (rounds & 0xFF) == 7 ? SMAT_WIDE_OCC(7 | kFamily) : SMAT_WIDE_OCC(10 | kFamily);
+int SMAT_FAMILY(fused_wide_ctas_per_sm)(int noise, bool per_elem_alpha, int rounds) {
+#define SMAT_WIDE_OCC(R, PE) \
+  (noise == NOISE_GAUSSIAN ? FusedVariant<R, DT_BF16, NOISE_GAUSSIAN, PE, false>::occ() \
+                           : FusedVariant<R, DT_BF16, NOISE_UNIFORM, PE, false>::occ())
+  if (per_elem_alpha) return (rounds & 0xFF) == 7 ? SMAT_WIDE_OCC(7 | kFamily, true) : SMAT_WIDE_OCC(10 | kFamily, true);
+  return (rounds & 0xFF) == 7 ? SMAT_WIDE_OCC(7 | kFamily, false) : SMAT_WIDE_OCC(10 | kFamily, false);
 #undef SMAT_WIDE_OCC
 }
 

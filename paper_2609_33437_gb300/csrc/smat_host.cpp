@@ -250,7 +250,6 @@ struct smat_ctx {
   bool adams_uploaded = false;
   // work-list forward launch (with the statistics of sigma_rel tensors)
   bool fused = false;
-  bool wide = false;  // the bf16 work-list launch is the four-CTA build
   std::vector<int32_t> h_items;
   int32_t item_begin[kMaxRanges] = {0, 0};
   int32_t item_count[kMaxRanges] = {0, 0};
@@ -360,8 +359,9 @@ int grid_for(const smat_ctx* c, int64_t chunks, int dtype) {
 // Grid of the work-list launch of one dtype range.
 int fused_grid(const smat_ctx* c, int dt) {
   const int64_t chunks = c->range_end[dt] - c->range_begin[dt];
-  if (!(c->wide && dt == SMAT_BF16)) return grid_for(c, chunks, dt);
-  return (int)std::min(chunks, (int64_t)c->sm_count * fused_wide_occ(c->cfg.noise, c->rounds));
+  if (c->any_inplace || dt != SMAT_BF16) return grid_for(c, chunks, dt);
+  const int per_sm = fused_wide_occ(c->cfg.noise, c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT, c->rounds);
+  return (int)std::min(chunks, (int64_t)c->sm_count * per_sm);
 }
 
 // Rows a2 + a1: delta statistics (if needed) then the per-call scalars.
@@ -512,12 +512,11 @@ smat_status smat_init(smat_ctx** out, const smat_tensor_desc* tensors, int32_t n
     e = cudaMemcpyAsync(c->d_chunks, c->h_chunks.data(), sizeof(Chunk) * (size_t)nc,
                         cudaMemcpyHostToDevice, stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_sync, 0, sizeof(int32_t) * sync_words(n_tensors), stream);
-  c->wide = cfg->alpha_mode != SMAT_ALPHA_PER_ELEMENT && cfg->noise != SMAT_NOISE_LAPLACE && !c->any_inplace;
   if (e == cudaSuccess && c->fused) {
     // lead of about one grid width of the bf16 forward (one, two and four
     // measured on the 7B list: one is fastest)
     const int64_t lead = (int64_t)c->sm_count *
-                         (c->wide ? fused_wide_occ(cfg->noise, c->rounds)
+                         (!c->any_inplace ? fused_wide_occ(cfg->noise, cfg->alpha_mode == SMAT_ALPHA_PER_ELEMENT, c->rounds)
                                   : streaming_ctas_per_sm(SMAT_BF16, cfg->noise,
                                                           cfg->alpha_mode == SMAT_ALPHA_PER_ELEMENT, c->rounds));
     for (int dt = 0; dt < 2; ++dt) build_items(c, dt, lead);

@@ -168,14 +168,16 @@ cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise
                                              int rounds, cudaStream_t s);                                     \
   cudaError_t launch_stats_simulate_bf16##sfx(const KArgs& a, int grid, int noise, bool per_elem_alpha,       \
                                               int rounds, cudaStream_t s);                                    \
-  /* Resident CTAs per SM of launch_stats_simulate_bf16 (uniform or Gaussian, no per-element alpha). */       \
-  int fused_wide_ctas_per_sm##sfx(int noise, int rounds);                                                     \
+  /* Resident CTAs per SM of launch_stats_simulate_bf16 (uniform or Gaussian). */                             \
+  int fused_wide_ctas_per_sm##sfx(int noise, bool per_elem_alpha, int rounds);                                \
   /* Laplace noise (10 rounds; smat_laplace_*.cu): the work-list launch when `fused`, else the grid-stride    \
      one; in-place instantiations when `inplace`. */                                                          \
   cudaError_t launch_laplace_f32##sfx(const KArgs& a, int grid, bool fused, bool per_elem_alpha, bool inplace, \
                                       cudaStream_t s);                                                        \
   cudaError_t launch_laplace_bf16##sfx(const KArgs& a, int grid, bool fused, bool per_elem_alpha,             \
                                        bool inplace, cudaStream_t s);                                         \
+  /* Resident CTAs per SM of launch_laplace_bf16's work-list launch without in-place tensors. */               \
+  int laplace_ctas_per_sm_bf16##sfx(bool per_elem_alpha);                                                      \
   /* the same launches for lists with in-place tensors (smat_inplace_*.cu) */                                \
   cudaError_t launch_stats_simulate_inplace_f32##sfx(const KArgs& a, int grid, int noise, bool per_elem_alpha, \
                                                      int rounds, cudaStream_t s);                             \
@@ -197,7 +199,7 @@ SMAT_FORWARD_LAUNCHERS(_d16)
 
 // Family dispatch (smat_aux.cu): the bf16 work-list launch's occupancy and the
 // gradient map for the variant code `rounds`.
-int fused_wide_occ(int noise, int rounds);
+int fused_wide_occ(int noise, bool per_elem_alpha, int rounds);
 cudaError_t launch_grad_map(const KArgs& a, int grid, int gdtype, bool per_elem_alpha, bool accumulate, int rounds,
                             cudaStream_t s);
 int grad_map_occ(int gdtype, bool per_elem_alpha, bool accumulate, int rounds);

@@ -27,4 +27,9 @@ cudaError_t SMAT_FAMILY(launch_laplace_bf16)(const KArgs& a, int grid, bool fuse
   return inplace ? laplace_run<false, true>(a, grid, fused, s) : laplace_run<false, false>(a, grid, fused, s);
 }
 
+int SMAT_FAMILY(laplace_ctas_per_sm_bf16)(bool per_elem_alpha) {
+  return per_elem_alpha ? FusedVariant<10 | kFamily, DT_BF16, NOISE_LAPLACE, true, false>::occ()
+                        : FusedVariant<10 | kFamily, DT_BF16, NOISE_LAPLACE, false, false>::occ();
+}
+
 }  // namespace smat

@@ -275,10 +275,12 @@ __device__ __forceinline__ void forward_chunk(const KArgs& a, const TView& v, co
 // latencies of the forward and the memory latency of the statistics better than
 // three CTAs with 80 registers do (a vision tower with uniform noise 660 -> 628
 // us for the step, 0.5B decoder 663 -> 651 us, vision-language list 3089 -> 3067
-// us, 7B list with statistics 11.98 -> 11.73 ms when it was introduced). In-place
-// and Laplace launches keep three.
+// us, 7B list with statistics 11.98 -> 11.73 ms when it was introduced), and with
+// per-element alpha at three instead of two (1e8 elements: Gaussian 265 -> 239
+// us, Laplace 307 -> 270 us with the logarithm's change). In-place launches keep
+// three and two, Laplace without per-element alpha three (four: 207 -> 215 us).
 template <int DT, int NOISE, bool PE, bool IP>
-constexpr int kFusedCtas = DT != DT_BF16 || PE ? 2 : (IP || NOISE == NOISE_LAPLACE ? 3 : 4);
+constexpr int kFusedCtas = DT != DT_BF16 ? 2 : IP ? (PE ? 2 : 3) : (PE || NOISE == NOISE_LAPLACE ? 3 : 4);
 
 template <int R, int DT, int NOISE, bool PE, bool IP>
 __global__ void __launch_bounds__(kBlock, kFusedCtas<DT, NOISE, PE, IP>)

@@ -364,6 +364,17 @@ int fused_grid(const smat_ctx* c, int dt) {
   return (int)std::min(chunks, (int64_t)c->sm_count * per_sm);
 }
 
+// Grid of the fused AdamW launch over a's chunk range, and the split of its last
+// units (KArgs): up to eight pieces of at least 2^13 elements.
+int split_units(KArgs& a, int64_t resident) {
+  const int64_t units = (a.chunk_end - a.chunk_begin) * (int64_t)a.grad_units;
+  a.grad_split = 0;
+  while (a.grad_split < 3 && (a.grad_unit >> (a.grad_split + 1)) >= 2 * kMinChunkElems) a.grad_split += 1;
+  a.grad_whole = units / resident * resident;
+  const int64_t claims = a.grad_whole + ((units - a.grad_whole) << a.grad_split);
+  return (int)std::min(claims, resident);
+}
+
 // Rows a2 + a1: delta statistics (if needed) then the per-call scalars.
 smat_status run_scalars(smat_ctx* c, uint32_t step, bool with_sigma, cudaStream_t s) {
   KArgs a = base_args(c, step);
@@ -736,9 +747,7 @@ smat_status smat_grad_map_adamw_multi(smat_ctx* c, uint32_t step, const void* co
     a.chunk_end = c->range_end[dt];
     if (a.chunk_end <= a.chunk_begin) continue;
     const int pdt = dt == 0 ? SMAT_F32 : SMAT_BF16;
-    const int64_t units = (a.chunk_end - a.chunk_begin) * (int64_t)a.grad_units;
-    const int64_t resident = (int64_t)c->sm_count * grad_map_adamw_occ(gdtype, pdt, pe, c->rounds);
-    const int grid = (int)(units < resident ? units : resident);
+    const int grid = split_units(a, (int64_t)c->sm_count * grad_map_adamw_occ(gdtype, pdt, pe, c->rounds));
     Timed tm(c, 3, stream);
     const cudaError_t e = launch_grad_map_adamw(a, grid, gdtype, pdt, pe, c->rounds, stream);
     tm.done();

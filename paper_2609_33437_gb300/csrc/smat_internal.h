@@ -120,6 +120,8 @@ struct KArgs {
   int64_t chunk_end;
   int64_t grad_unit;     // gradient map: elements per unit (divides the chunk size)
   int32_t grad_units;    // gradient map: units per chunk
+  int64_t grad_whole;    // fused AdamW: units taken whole, a multiple of the grid; the rest in 2^grad_split pieces each
+  int32_t grad_split;
   RoundKeys key;
   uint32_t step;
   int32_t n_tensors;

@@ -264,3 +264,29 @@ def test_fused_adamw_special_moments(dtype):
             ga, ra = O.bf16_to_f32(got), O.bf16_to_f32(hth)
             assert np.all((got == hth) | (np.isnan(ga) & np.isnan(ra))), f"step {step} theta"
     sess.close()
+
+
+@pytest.mark.parametrize("pdt,gdt", [(torch.float32, torch.float32), (torch.bfloat16, torch.bfloat16)])
+def test_adamw_units_and_pieces_equal(pdt, gdt):
+    """The launch takes whole units and, past the last full round of the grid,
+    pieces of units: theta and the moments do not depend on the chunk size,
+    with fewer units than CTAs, a remainder of one unit, units too small to cut
+    and tensors that end inside a piece."""
+    sizes = [305 * (1 << 14) - 5, 4096, 70_001, 16]
+    t0 = [(torch.randn(n, device="cuda") * 0.02).to(pdt) for n in sizes]
+    gs = [torch.randn(n, device="cuda").to(gdt) for n in sizes]
+    ref = None
+    for log2 in (12, 14, 15, 18):
+        th = [t.clone() for t in t0]
+        m1 = [torch.full((n,), 0.01, device="cuda") for n in sizes]
+        m2 = [torch.full((n,), 0.02, device="cuda") for n in sizes]
+        sess = S.SmatSession(th, t0, [torch.empty_like(t) for t in t0], [0.7, 1.0, 0.3, 0.5], [1e-3] * 4, seed=5,
+                             alpha_min=0.3, flags=S.SMAT_FLAG_CHUNK_LOG2(log2))
+        sess.simulate_multi(3)
+        sess.grad_map_adamw_multi(3, gs, m1, m2, lr=1e-3, weight_decay=0.01, adam_step=4)
+        torch.cuda.synchronize()
+        got = [x.view(torch.int16 if x.dtype == torch.bfloat16 else torch.int32) for x in th + m1 + m2]
+        ref = got if ref is None else ref
+        for k, (a, b) in enumerate(zip(ref, got)):
+            assert torch.equal(a, b), (log2, k)
+        sess.close()

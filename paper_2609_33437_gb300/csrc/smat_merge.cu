@@ -483,8 +483,14 @@ __global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 3 : 2) ties_merge_kern
   }
 }
 
+// WA and TA. bf16 at three CTAs per SM (76 registers): two left 7% of the copy
+// bandwidth unused, four spill (8 experts of 1e8 elements: 332, 309 and 357 us,
+// 16 experts 572, 541 and 636 us).
+template <int DT>
+constexpr int kLinearCtas = DT == DT_BF16 ? 3 : 2;
+
 template <int R, int DT, int METHOD>
-__global__ void __launch_bounds__(kBlock, 2) merge_kernel(const __grid_constant__ MArgs m) {
+__global__ void __launch_bounds__(kBlock, kLinearCtas<DT>) merge_kernel(const __grid_constant__ MArgs m) {
   for (int64_t ci = blockIdx.x; ci < m.n_chunks; ci += gridDim.x) {
     const Chunk ch = m.chunks[ci];
     const MTensor& T = m.tensors[ch.tensor];
@@ -1054,8 +1060,8 @@ cudaError_t merge_launch(MArgs m, int64_t slots, int64_t largest, bool ties, int
     if (m.K % 4 == 0) return ties_merge_run<DT, 4, true>(m, sms, s);
     return ties_merge_run<DT, 4, false>(m, sms, s);
   }
-  const int grid = (int)(m.n_chunks < 2 * (int64_t)sms ? m.n_chunks : 2 * (int64_t)sms);
-  return merge_method<R, DT>(m, grid, s);
+  const int64_t resident = (m.method == SMAT_MERGE_DARE_TA ? 2 : kLinearCtas<DT>) * (int64_t)sms;
+  return merge_method<R, DT>(m, (int)(m.n_chunks < resident ? m.n_chunks : resident), s);
 }
 
 }  // namespace

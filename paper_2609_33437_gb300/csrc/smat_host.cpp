@@ -160,11 +160,12 @@ smat_status check_tensors(const smat_tensor_desc* t, int32_t n, const smat_confi
 // addressing its device address is the host address), or any host memory
 // when the device reads pageable memory directly (coherent CPU-GPU systems).
 smat_status check_gpu_access(const smat_tensor_desc* t, int32_t n) {
+  GpuAccess access;
   for (int32_t k = 0; k < n; ++k) {
     if (t[k].numel <= 0) continue;
     const void* ptrs[3] = {t[k].theta, t[k].theta0, t[k].sim};
     for (const void* p : ptrs) {
-      const int ok = gpu_can_access(p);
+      const int ok = access.check(p);
       if (ok < 0) return fail(SMAT_ERR_CUDA, "no current CUDA device or pointer attributes unavailable");
       if (!ok) return fail(SMAT_ERR_INVALID_ARG, "tensor %d: a data pointer is not accessible from the GPU", k);
     }
@@ -176,23 +177,52 @@ RoundKeys make_keys(uint64_t seed) { return make_round_keys(seed); }
 
 }  // namespace
 
-// 1 if the kernels can dereference p as it is: device or managed memory, host
-// memory registered with CUDA (pinned; under unified addressing its device
-// address is the host address), or any host memory when the device reads
-// pageable memory directly (coherent CPU-GPU systems); 0 if not; -1 on a
-// CUDA error.
-int smat::gpu_can_access(const void* p) {
-  int dev = 0, pageable = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return -1;
-  if (cudaDeviceGetAttribute(&pageable, cudaDevAttrPageableMemoryAccess, dev) != cudaSuccess) pageable = 0;
+// Device or managed memory, host memory registered with CUDA (pinned; under
+// unified addressing its device address is the host address), or any host
+// memory when the device reads pageable memory directly (coherent CPU-GPU
+// systems).
+GpuAccess::GpuAccess() {
+  int dev = 0;
+  ok_ = cudaGetDevice(&dev) == cudaSuccess;
+  if (ok_ && cudaDeviceGetAttribute(&pageable_, cudaDevAttrPageableMemoryAccess, dev) != cudaSuccess) pageable_ = 0;
+}
+
+int GpuAccess::check(const void* p) {
+  if (!ok_) return -1;
+  const uintptr_t x = (uintptr_t)p;
+  if (last_ < ranges_.size() && x >= ranges_[last_].first && x < ranges_[last_].second) return 1;
+  for (size_t k = 0; k < ranges_.size(); ++k)
+    if (x >= ranges_[k].first && x < ranges_[k].second) {
+      last_ = k;
+      return 1;
+    }
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
     return -1;
   }
+  if (at.type == cudaMemoryTypeDevice && ranges_.size() < 64) {
+    // the allocation that holds p (the driver call has no runtime equivalent)
+    using RangeFn = int (*)(unsigned long long*, size_t*, unsigned long long);
+    static const RangeFn range_of = [] {
+      void* fn = nullptr;
+      cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+      if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess) {
+        cudaGetLastError();
+        fn = nullptr;
+      }
+      return found == cudaDriverEntryPointSuccess ? (RangeFn)fn : nullptr;
+    }();
+    unsigned long long base = 0;
+    size_t size = 0;
+    if (range_of && range_of(&base, &size, (unsigned long long)x) == 0 && size > 0) {
+      last_ = ranges_.size();
+      ranges_.push_back({(uintptr_t)base, (uintptr_t)base + size});
+    }
+  }
   return (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged ||
           (at.type == cudaMemoryTypeHost && at.devicePointer == p) ||
-          (at.type == cudaMemoryTypeUnregistered && pageable))
+          (at.type == cudaMemoryTypeUnregistered && pageable_))
              ? 1
              : 0;
 }

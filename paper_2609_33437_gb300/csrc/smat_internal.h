@@ -4,6 +4,8 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <utility>
+#include <vector>
 
 #include <cuda_runtime.h>
 
@@ -229,8 +231,20 @@ constexpr int kBlock = 256;
 
 // Record `msg` as this thread's smat_last_error() text; returns `status`.
 int record_error_code(int status, const char* msg);
-// 1 if kernels can dereference p as it is, 0 if not, -1 on a CUDA error.
-int gpu_can_access(const void* p);
+// Which pointers of one call the kernels can dereference as they are. Keeps
+// the device allocations met so far, for this call alone, so that a list of
+// hundreds of views costs a few runtime queries instead of one per pointer.
+class GpuAccess {
+ public:
+  GpuAccess();
+  int check(const void* p);  // 1 if they can, 0 if not, -1 on a CUDA error
+
+ private:
+  bool ok_ = false;
+  int pageable_ = 0;
+  size_t last_ = 0;
+  std::vector<std::pair<uintptr_t, uintptr_t>> ranges_;
+};
 // Philox round keys of a seed (smat_host.cpp).
 RoundKeys make_round_keys(uint64_t seed);
 

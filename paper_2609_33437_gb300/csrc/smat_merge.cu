@@ -1092,10 +1092,11 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
   if (!d_workspace || (uintptr_t)d_workspace % kMergeAlign)
     return mfail(SMAT_ERR_WORKSPACE, "workspace NULL or not 256-byte aligned");
   if (workspace_bytes < L.total) return mfail(SMAT_ERR_WORKSPACE, "workspace %zu < %zu bytes", workspace_bytes, L.total);
+  GpuAccess access;
   for (int32_t k = 0; k < n_tensors; ++k) {
     if (tensors[k].numel <= 0) continue;
-    int ok = gpu_can_access(tensors[k].theta0) == 1 && gpu_can_access(tensors[k].out) == 1;
-    for (int e = 0; ok && e < K; ++e) ok = gpu_can_access(tensors[k].experts[e]) == 1;
+    int ok = access.check(tensors[k].theta0) == 1 && access.check(tensors[k].out) == 1;
+    for (int e = 0; ok && e < K; ++e) ok = access.check(tensors[k].experts[e]) == 1;
     if (!ok) return mfail(SMAT_ERR_INVALID_ARG, "tensor %d: a pointer is not accessible from the GPU", k);
   }
   if (n_tensors == 0 || nc == 0) return SMAT_OK;

@@ -12,7 +12,9 @@ smat_tensor_scalars -> SmatSession.tensor_scalars.
 """
 
 import ctypes
+import itertools
 import os
+import struct
 from typing import List, Optional, Sequence
 
 import torch
@@ -139,6 +141,27 @@ def dtype_code(dt: torch.dtype) -> int:
     raise TypeError(f"unsupported dtype {dt} (float32 or bfloat16)")
 
 
+# Per-tensor checks as whole-list passes: a call over a model's tensors
+# (hundreds, ten times as many pointers in a merge) is otherwise bound by the
+# interpreter, about 0.25 us for each attribute of each tensor.
+_numel, _contiguous = torch.Tensor.numel, torch.Tensor.is_contiguous
+_pointer = torch.Tensor.data_ptr
+
+
+def _all_cuda_contiguous(ts) -> bool:
+    return all(map(_contiguous, ts)) and all([t.is_cuda for t in ts])
+
+
+def _one_dtype(ts) -> Optional[torch.dtype]:
+    """The dtype of all of ts, or None if they differ."""
+    dt = ts[0].dtype
+    return dt if all([t.dtype is dt for t in ts]) else None
+
+
+def _pointers(ts):
+    return (ctypes.c_void_p * max(len(ts), 1))(*map(_pointer, ts))
+
+
 def _stream_handle(stream: Optional[torch.cuda.Stream]):
     s = stream if stream is not None else torch.cuda.current_stream()
     return ctypes.c_void_p(s.cuda_stream)
@@ -213,28 +236,35 @@ class SmatSession:
 
     def grad_map_multi(self, step: int, g_sims: Sequence[torch.Tensor], g_outs: Optional[Sequence[torch.Tensor]] = None,
                        accumulate: bool = False, stream: Optional[torch.cuda.Stream] = None):
+        in_place = g_outs is None or g_outs is g_sims
         g_outs = g_sims if g_outs is None else g_outs
         if len(g_sims) != self.n or len(g_outs) != self.n:
             raise ValueError("one gradient per tensor expected")
+        every = list(g_sims) if in_place else [*g_sims, *g_outs]
         gd = None
-        ins = (ctypes.c_void_p * max(self.n, 1))()
-        outs = (ctypes.c_void_p * max(self.n, 1))()
+        if every:
+            dt = _one_dtype(every)
+            if (dt is None or list(map(_numel, every)) != (self.numels if in_place else self.numels * 2)
+                    or not _all_cuda_contiguous(every)):
+                self._refuse_gradients(g_sims, g_outs)
+            gd = dtype_code(dt)
+        ins = _pointers(g_sims)
+        outs = ins if in_place else _pointers(g_outs)
+        self._gkeep = (list(g_sims), list(g_outs))
+        check("smat_grad_map_multi",
+              self._L.smat_grad_map_multi(self._ctx, int(step), ins, outs, SMAT_F32 if gd is None else gd,
+                                          int(bool(accumulate)), _stream_handle(stream)))
+
+    def _refuse_gradients(self, g_sims, g_outs):
+        """Raise what is wrong with the first gradient that cannot be taken."""
         for k in range(self.n):
             a, b = g_sims[k], g_outs[k]
             if a.numel() != self.numels[k] or b.numel() != self.numels[k] or a.dtype != b.dtype:
                 raise ValueError(f"gradient {k}: numel or dtype mismatch")
             if not (a.is_cuda and b.is_cuda and a.is_contiguous() and b.is_contiguous()):
                 raise ValueError(f"gradient {k}: must be contiguous CUDA tensors")
-            code = dtype_code(a.dtype)
-            if gd is None:
-                gd = code
-            elif gd != code:
-                raise ValueError("all gradients must share one dtype")
-            ins[k], outs[k] = a.data_ptr(), b.data_ptr()
-        self._gkeep = (list(g_sims), list(g_outs))
-        check("smat_grad_map_multi",
-              self._L.smat_grad_map_multi(self._ctx, int(step), ins, outs, SMAT_F32 if gd is None else gd,
-                                          int(bool(accumulate)), _stream_handle(stream)))
+            dtype_code(a.dtype)
+        raise ValueError("all gradients must share one dtype")
 
     def grad_map_adamw_multi(self, step: int, g_sims: Sequence[torch.Tensor], m1s: Sequence[torch.Tensor],
                              m2s: Sequence[torch.Tensor], lr: float, beta1: float = 0.9, beta2: float = 0.999,
@@ -245,9 +275,22 @@ class SmatSession:
         if len(g_sims) != self.n or len(m1s) != self.n or len(m2s) != self.n:
             raise ValueError("one gradient and two moment buffers per tensor expected")
         gd = None
-        gp = (ctypes.c_void_p * max(self.n, 1))()
-        p1 = (ctypes.c_void_p * max(self.n, 1))()
-        p2 = (ctypes.c_void_p * max(self.n, 1))()
+        if self.n:
+            dt = _one_dtype(g_sims)
+            every = [*g_sims, *m1s, *m2s]
+            if (dt is None or list(map(_numel, every)) != self.numels * 3 or _one_dtype(m1s) != torch.float32
+                    or _one_dtype(m2s) != torch.float32 or not _all_cuda_contiguous(every)):
+                self._refuse_adamw(g_sims, m1s, m2s)
+            gd = dtype_code(dt)
+        gp, p1, p2 = _pointers(g_sims), _pointers(m1s), _pointers(m2s)
+        self._gkeep = (list(g_sims), list(m1s), list(m2s))
+        opt = AdamW(float(lr), float(beta1), float(beta2), float(eps), float(weight_decay), int(adam_step))
+        check("smat_grad_map_adamw_multi",
+              self._L.smat_grad_map_adamw_multi(self._ctx, int(step), gp, p1, p2, SMAT_F32 if gd is None else gd,
+                                                ctypes.byref(opt), _stream_handle(stream)))
+
+    def _refuse_adamw(self, g_sims, m1s, m2s):
+        """Raise what is wrong with the first tensor that cannot be taken."""
         for k in range(self.n):
             g, a, b = g_sims[k], m1s[k], m2s[k]
             if g.numel() != self.numels[k] or a.numel() != self.numels[k] or b.numel() != self.numels[k]:
@@ -256,17 +299,8 @@ class SmatSession:
                 raise ValueError(f"tensor {k}: moments must be float32")
             if not all(x.is_cuda and x.is_contiguous() for x in (g, a, b)):
                 raise ValueError(f"tensor {k}: must be contiguous CUDA tensors")
-            code = dtype_code(g.dtype)
-            if gd is None:
-                gd = code
-            elif gd != code:
-                raise ValueError("all gradients must share one dtype")
-            gp[k], p1[k], p2[k] = g.data_ptr(), a.data_ptr(), b.data_ptr()
-        self._gkeep = (list(g_sims), list(m1s), list(m2s))
-        opt = AdamW(float(lr), float(beta1), float(beta2), float(eps), float(weight_decay), int(adam_step))
-        check("smat_grad_map_adamw_multi",
-              self._L.smat_grad_map_adamw_multi(self._ctx, int(step), gp, p1, p2, SMAT_F32 if gd is None else gd,
-                                                ctypes.byref(opt), _stream_handle(stream)))
+            dtype_code(g.dtype)
+        raise ValueError("all gradients must share one dtype")
 
     def swap(self) -> int:
         a = ctypes.c_int32()
@@ -460,23 +494,26 @@ def merge(theta0s: Sequence[torch.Tensor], experts: Sequence[Sequence[torch.Tens
     K = len(experts[0]) if n else 0
     tensor_ids = tensor_ids if tensor_ids is not None else list(range(n))
     elem_offsets = elem_offsets if elem_offsets is not None else [0] * n
-    descs = (MergeTensor * max(n, 1))()
-    keep = []
-    for k in range(n):
-        if len(experts[k]) != K:
-            raise ValueError("every tensor needs the same number of experts")
-        for t in [theta0s[k], outs[k], *experts[k]]:
-            if not t.is_contiguous() or t.numel() != theta0s[k].numel() or t.dtype != theta0s[k].dtype:
+    if any([len(e) != K for e in experts]):
+        raise ValueError("every tensor needs the same number of experts")
+    rows = [(t0, out, *ex) for t0, out, ex in zip(theta0s, outs, experts)]
+    every = list(itertools.chain.from_iterable(rows))
+    numels = list(map(_numel, theta0s))
+    wanted = list(itertools.chain.from_iterable([(x,) * (K + 2) for x in numels]))
+    if (list(map(_numel, every)) != wanted or not all(map(_contiguous, every))
+            or any([_one_dtype(r) is None for r in rows])):
+        for k, row in enumerate(rows):
+            if _one_dtype(row) is None or not all(t.is_contiguous() and t.numel() == numels[k] for t in row):
                 raise ValueError(f"tensor {k}: contiguous tensors of one shape and dtype")
-        ptrs = (ctypes.c_void_p * max(K, 1))(*[x.data_ptr() for x in experts[k]])
-        keep.append(ptrs)
-        d = descs[k]
-        d.theta0, d.out = theta0s[k].data_ptr(), outs[k].data_ptr()
-        d.experts = ctypes.cast(ptrs, ctypes.c_void_p)
-        d.numel = theta0s[k].numel()
-        d.elem_offset = int(elem_offsets[k])
-        d.tensor_id = int(tensor_ids[k])
-        d.dtype = dtype_code(theta0s[k].dtype)
+    codes = [dtype_code(t.dtype) for t in theta0s]
+    # smat_merge_tensor records (MergeTensor's layout) beside one array of all expert pointers
+    ex_ptrs = _pointers(list(itertools.chain.from_iterable(experts)))
+    row = max(K, 1) * ctypes.sizeof(ctypes.c_void_p)
+    ex0 = ctypes.addressof(ex_ptrs)
+    descs = (MergeTensor * max(n, 1))()
+    struct.pack_into("PPPqqIi" * n, descs, 0, *itertools.chain.from_iterable(
+        zip(map(_pointer, theta0s), range(ex0, ex0 + n * row, row), map(_pointer, outs), numels,
+            [ctypes.c_int64(int(x)).value for x in elem_offsets], [int(x) & 0xFFFFFFFF for x in tensor_ids], codes)))
     cfg = MergeConfig(int(method), K, float(gamma), float(p_drop), float(retention), int(seed) & (2**64 - 1),
                       int(philox_rounds), 0)
     nbytes = L.smat_merge_workspace_bytes(ctypes.byref(descs), n, ctypes.byref(cfg))

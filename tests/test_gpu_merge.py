@@ -246,3 +246,49 @@ def test_merge_ties_expert_counts(K, dtype):
         nan_g, nan_r = np.isnan(f32_of(got)), np.isnan(f32_of(ref))
         assert np.array_equal(nan_g, nan_r)
         assert np.array_equal(got.view(view)[~nan_g], ref.view(view)[~nan_r]), k
+
+
+def test_merge_refuses_mismatched_tensors():
+    """The binding's list checks refuse what a tensor-by-tensor check would,
+    naming the tensor, and take views, in-place outputs and empty tensors."""
+    t0s, exs = _experts([1000, 64, 0, 4096], 3, O.F32, seed=2)
+    outs = [torch.empty_like(t) for t in t0s]
+
+    def refused(k, t0=None, ex=None, out=None, error=ValueError):
+        a, b, c = list(t0s), [list(e) for e in exs], list(outs)
+        a[k] = t0 if t0 is not None else a[k]
+        c[k] = out if out is not None else c[k]
+        if ex is not None:
+            b[k][1] = ex
+        with pytest.raises(error) as e:
+            S.merge(a, b, c, S.SMAT_MERGE_TA)
+        return str(e.value)
+
+    for k in (0, 3):
+        n = t0s[k].numel()
+        wrong = torch.empty(n + 1, device="cuda")
+        other = torch.empty(n, device="cuda", dtype=torch.bfloat16)
+        strided = torch.empty(2 * n, device="cuda")[::2]
+        for kind in ("t0", "ex", "out"):
+            for bad in (wrong, other, strided):
+                assert f"tensor {k}" in refused(k, **{kind: bad})
+    with pytest.raises(ValueError):
+        S.merge(t0s, [exs[0], exs[1][:2], exs[2], exs[3]], outs, S.SMAT_MERGE_TA)
+    with pytest.raises(ValueError):
+        S.merge(t0s[:3], exs, outs, S.SMAT_MERGE_TA)
+    half = [t.half() for t in t0s]
+    with pytest.raises(TypeError):
+        S.merge(half, [[x.half() for x in e] for e in exs], [t.half() for t in outs], S.SMAT_MERGE_TA)
+    with pytest.raises(S.SmatError):
+        S.merge(t0s, [[] for _ in exs], outs, S.SMAT_MERGE_TA)
+    with pytest.raises(S.SmatError):
+        S.merge([], [], [], S.SMAT_MERGE_TA)  # no tensor, so no expert either
+    S.merge(t0s, exs, outs, S.SMAT_MERGE_TA, gamma=0.5, tensor_ids=[7, 5, 3, 1], elem_offsets=[0, 16, 0, 1 << 40])
+    flat = torch.cat([t.reshape(-1) for t in t0s])
+    at, views = 0, []
+    for t in t0s:
+        views.append(flat[at:at + t.numel()])
+        at += t.numel()
+    S.merge(views, exs, views, S.SMAT_MERGE_TA, gamma=0.5)
+    for a, b in zip(outs, views):
+        assert torch.equal(a, b)

@@ -287,6 +287,46 @@ def test_inplace_gradient_map_equals_out_of_place(gdt, alpha_mode, keep):
         sess.close()
 
 
+def test_gradient_lists_refused_by_the_binding():
+    """Gradients and moments that do not fit the list are refused, whichever
+    tensor they belong to; separate output lists and the in-place forms (no
+    outputs, the same list, the same tensors) are taken."""
+    sizes = [1000, 33, 4096]
+    th = [torch.randn(n, device="cuda") for n in sizes]
+    sess = S.SmatSession(th, [t.clone() for t in th], [torch.empty_like(t) for t in th], [0.5] * 3, [1e-3] * 3)
+    sess.simulate_multi(0)
+    gs = [torch.randn(n, device="cuda") for n in sizes]
+    out = [torch.empty_like(g) for g in gs]
+    m = [torch.zeros(n, device="cuda") for n in sizes]
+    for k, n in enumerate(sizes):
+        for bad, error in ((torch.empty(n + 1, device="cuda"), ValueError), (torch.empty(n), ValueError),
+                           (torch.empty(2 * n, device="cuda")[::2], ValueError),
+                           (torch.empty(n, device="cuda", dtype=torch.bfloat16), ValueError)):
+            lists = [list(gs), list(out), list(m)]
+            for which in range(3):
+                lists[which][k] = bad
+                if which < 2:
+                    with pytest.raises(error):
+                        sess.grad_map_multi(0, lists[0], lists[1])
+                else:
+                    with pytest.raises(error):
+                        sess.grad_map_adamw_multi(0, gs, lists[2], m, lr=1e-3)
+                    with pytest.raises(error):
+                        sess.grad_map_adamw_multi(0, gs, m, lists[2], lr=1e-3)
+                lists[which] = [list(gs), list(out), list(m)][which]
+    with pytest.raises(TypeError):
+        sess.grad_map_multi(0, [g.half() for g in gs])
+    with pytest.raises(ValueError):
+        sess.grad_map_multi(0, gs[:2])
+    sess.grad_map_multi(0, gs, out)
+    for form in (lambda g: sess.grad_map_multi(0, g), lambda g: sess.grad_map_multi(0, g, g),
+                 lambda g: sess.grad_map_multi(0, g, list(g))):
+        g = [x.clone() for x in gs]
+        form(g)
+        assert all(torch.equal(a, b) for a, b in zip(g, out))
+    sess.close()
+
+
 def test_gradient_map_needs_the_forward_of_its_step():
     """The gradient map regenerates the mask of the forward that produced
     theta~ (Eq. smat-gradient; App. D): a map for a step that no forward on

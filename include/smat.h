@@ -164,10 +164,10 @@ smat_status smat_init(smat_ctx** out, const smat_tensor_desc* tensors, int32_t n
  * active (SMAT_ERR_STATE otherwise): the simulated state is rebuilt only
  * while the model reads theta; with in-place tensors it also requires theta0
  * to be resident in their sim buffers (SMAT_ERR_STATE otherwise) and leaves
- * theta~ there. By default the forward is one persistent
- * launch whose CTAs take chunks of 2^18 elements from a work list in order;
- * with sigma_rel tensors the statistics run in the same launch (statistics
- * of later tensors beside the forward of earlier ones).
+ * theta~ there. By default the forward of a list without sigma_rel tensors is
+ * one launch per dtype that computes the per-call scalars too; with sigma_rel
+ * tensors the scalars come first, and the statistics run in the forward's launch
+ * (statistics of later tensors beside the forward of earlier ones).
  * SMAT_FLAG_UNFUSED_STATS runs the statistics as a separate pass and the
  * forward as a grid-stride launch. Results are identical either way. */
 smat_status smat_simulate_multi(smat_ctx* ctx, uint32_t step, smat_stream_t stream);
@@ -308,9 +308,9 @@ smat_status smat_debug_fused(smat_ctx* ctx, uint32_t step, const int32_t* d_item
 
 /* Per-kernel timing (for measurement): while enabled, every kernel this
  * context launches is bracketed by two CUDA events recorded on the launching
- * stream. Kinds: 0 delta statistics (a2, unfused), 1 per-call scalars (a1),
- * 2 forward (a3; with fused statistics when they are fused), 3 gradient map
- * (a5). Enabling clears the totals. Host-side
+ * stream. Kinds: 0 delta statistics (a2, unfused), 1 per-call scalars (a1, where
+ * they are a launch of their own), 2 forward (a3; with the scalars or the fused
+ * statistics where they are part of it), 3 gradient map (a5). Enabling clears the totals. Host-side
  * events only; no device memory is allocated. */
 smat_status smat_timing_enable(smat_ctx* ctx, int32_t enable);
 

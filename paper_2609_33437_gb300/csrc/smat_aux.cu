@@ -50,15 +50,7 @@ __global__ void scalars_kernel(const __grid_constant__ KArgs a) {
   }
   if (lane == 0) {
     DevScalars S;
-    if (a.alpha_mode == 2) {
-      S.alpha = 0.0f;
-      S.c = 0.0f;
-    } else {
-      const uint32_t ta = (a.alpha_mode == 0) ? kGlobalAlphaTensor : T.tid;
-      const uint4 w = stream_block<R>(a, S_ALPHA_T, ta, 0);
-      S.alpha = alpha_elem(a, w.x);
-      S.c = __fmul_rn(S.alpha, T.inv_keep);
-    }
+    scale_scalars<R>(a, T, S);
     S.sigma = sigma;
     S.noise_scale = noise_scale_of<NOISE>(sigma);
     a.scal[t] = S;
@@ -144,6 +136,18 @@ cudaError_t launch_simulate(const KArgs& a, int grid, int dtype, int noise, bool
                             : SMAT_BY_FAMILY(launch_simulate_inplace_f32)(a, grid, noise, per_elem_alpha, rounds, s);
   return dtype == DT_BF16 ? SMAT_BY_FAMILY(launch_simulate_bf16)(a, grid, noise, per_elem_alpha, rounds, s)
                           : SMAT_BY_FAMILY(launch_simulate_f32)(a, grid, noise, per_elem_alpha, rounds, s);
+}
+
+cudaError_t launch_direct(const KArgs& a, int dtype, int noise, bool per_elem_alpha, int rounds, bool inplace,
+                          cudaStream_t s) {
+  if (noise == NOISE_LAPLACE)
+    return dtype == DT_BF16 ? SMAT_BY_FAMILY(launch_direct_laplace_bf16)(a, per_elem_alpha, inplace, s)
+                            : SMAT_BY_FAMILY(launch_direct_laplace_f32)(a, per_elem_alpha, inplace, s);
+  if (inplace)
+    return dtype == DT_BF16 ? SMAT_BY_FAMILY(launch_direct_inplace_bf16)(a, noise, per_elem_alpha, rounds, s)
+                            : SMAT_BY_FAMILY(launch_direct_inplace_f32)(a, noise, per_elem_alpha, rounds, s);
+  return dtype == DT_BF16 ? SMAT_BY_FAMILY(launch_direct_bf16)(a, noise, per_elem_alpha, rounds, s)
+                          : SMAT_BY_FAMILY(launch_direct_f32)(a, noise, per_elem_alpha, rounds, s);
 }
 
 cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise, bool per_elem_alpha,

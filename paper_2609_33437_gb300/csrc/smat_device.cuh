@@ -11,10 +11,11 @@
 //   a6 mask_bits_kernel    packed keep bits (test hook)
 //
 // All of them are multi-tensor launches over a chunk table (chunks of one
-// tensor, 2^12 to 2^18 elements, the size chosen per list). The forward, with
-// the statistics fused for sigma_rel tensors, is a persistent launch whose
-// CTAs take whole chunks from an ordered work list; the unfused statistics,
-// the grid-stride forward and the gradient map walk the table in grid-stride
+// tensor, 2^12 to 2^18 elements, the size chosen per list). The forward of a
+// list without statistics has one CTA per chunk, which draws the chunk's scalars
+// itself; with statistics fused for sigma_rel tensors it is a persistent launch
+// whose CTAs take whole chunks from an ordered work list; the unfused statistics,
+// the forward beside them and the gradient map walk the table in grid-stride
 // order. Each thread owns 16 consecutive elements at a time (one 256-bit load
 // per bf16 input, two per fp32 input), which is exactly one Philox block of
 // the mask stream (16 high bytes) and three blocks of the noise stream (24
@@ -117,20 +118,20 @@ __device__ __forceinline__ float sym24(uint32_t u) {
 // erfinv(x) / x for |x| <= 1 - 2^-24 (every value sym24() produces), after
 // the structure of M. Giles, "Approximating the erfinv function" (GPU
 // Computing Gems Jade Edition, 2011), with coefficients fitted for this form
-// by csrc/fit_erfinv.py: with L = log2(1 - x^2) (one fused multiply-add and
-// the hardware log2),
+// by csrc/fit_erfinv.py to the hardware's own log2: with L = log2(1 - x^2) (one
+// fused multiply-add and the hardware log2),
 //   L >= -10:  P(L)             (degree 10, 99.95% of inputs)
 //   L <  -10:  Q(sqrt(-L) - 4)  (degree 7)
-// Both are even in x, so x times the ratio is exactly odd. Relative error at
-// most 1.3e-7 (central) and 1.4e-7 (tail), 3.4e-8 in the mean square; the tests
-// bound it. A 16-element group with a tail element is done again by the element
-// path: 0.8% of the groups, where -8 with degree 9 left 3.1% and the forward
-// took 1 to 2% longer for the shorter polynomial (vision-language list).
+// Both are even in x, so x times the ratio is exactly odd. Over every input: the
+// ratio within 1.41e-7 (3.0e-8 in the root mean square), x times it within 1.70e-7
+// (3.9e-8). A 16-element group with a tail element is done again by the element
+// path: 0.8% of the groups, where -8 with degree 9 left 3.1% and the forward took 1
+// to 2% longer for the shorter polynomial (vision-language list).
 constexpr float kCentralL = -10.0f;
 __device__ __forceinline__ float coef_p(int k) {  // increasing powers; k is a constant after unrolling
-  constexpr float c[11] = {8.862268925e-01f, -1.608197540e-01f, 5.548856221e-03f, 7.783531910e-04f,
-                           -2.820832924e-05f, -6.361147825e-06f, 7.189328244e-07f, 2.113999500e-07f,
-                           1.929385540e-08f, 8.415084740e-10f, 1.491148871e-11f};
+  constexpr float c[11] = {8.862269521e-01f, -1.608195305e-01f, 5.549574737e-03f, 7.792675169e-04f,
+                           -2.760529605e-05f, -6.129674603e-06f, 7.734802239e-07f, 2.193963837e-07f,
+                           2.000419030e-08f, 8.764800552e-10f, 1.564317426e-11f};
   return c[k];
 }
 __device__ __forceinline__ float coef_q(int k) {
@@ -625,6 +626,21 @@ struct TView {
   float inv_keep, c, noise_scale;
   bool has_noise;
 };
+
+// Scale of tensor T at this call (row a1) into S: alpha_t and c_t = alpha_t /
+// p_keep (0 in the per-element mode).
+template <int R>
+__device__ __forceinline__ void scale_scalars(const KArgs& a, const DevTensor& T, DevScalars& S) {
+  if (a.alpha_mode == 2) {
+    S.alpha = 0.0f;
+    S.c = 0.0f;
+  } else {
+    const uint32_t ta = (a.alpha_mode == 0) ? kGlobalAlphaTensor : T.tid;
+    const uint4 w = stream_block<R>(a, S_ALPHA_T, ta, 0);
+    S.alpha = alpha_elem(a, w.x);
+    S.c = __fmul_rn(S.alpha, T.inv_keep);
+  }
+}
 
 // Flags published by one CTA and waited for by another (work-list launches):
 // a release store after the data, an acquire load before reading it. Every

@@ -553,7 +553,7 @@ smat_status smat_init(smat_ctx** out, const smat_tensor_desc* tensors, int32_t n
     e = cudaMemcpyAsync(c->d_chunks, c->h_chunks.data(), sizeof(Chunk) * (size_t)nc,
                         cudaMemcpyHostToDevice, stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->d_sync, 0, sizeof(int32_t) * sync_words(n_tensors), stream);
-  if (e == cudaSuccess && c->fused) {
+  if (e == cudaSuccess && c->fused && rel) {
     // lead of about one grid width of the bf16 forward (one, two and four
     // measured on the 7B list: one is fastest)
     const int64_t lead = (int64_t)c->sm_count *
@@ -583,9 +583,28 @@ smat_status smat_simulate_multi(smat_ctx* c, uint32_t step, smat_stream_t stream
     return fail(SMAT_ERR_STATE, "in-place tensors: theta0 has not been refilled since the last forward");
   c->theta0_resident = false;  // the forward below overwrites it
   c->sim_step = -1;            // set again once every launch of this forward is enqueued
+  if (c->fused && !c->any_sigma_rel) {
+    // a1 and a3 in one launch per dtype, one CTA per chunk
+    c->scalars_step = -1;
+    KArgs a = base_args(c, step);
+    for (int dt = 0; dt < 2; ++dt) {
+      a.chunk_begin = c->range_begin[dt];
+      a.chunk_end = c->range_end[dt];
+      if (a.chunk_end <= a.chunk_begin) continue;
+      Timed t(c, 2, stream);
+      const cudaError_t e = launch_direct(a, dt, c->cfg.noise, c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT, c->rounds,
+                                          c->any_inplace, stream);
+      t.done();
+      if (e != cudaSuccess) return cuda_fail(e, "forward launch");
+    }
+    c->scalars_step = step;
+    c->scalars_sigma = true;
+    c->sim_step = step;
+    return SMAT_OK;
+  }
   if (c->fused) {
-    // a1 (alpha, c; sigma of fixed-sigma tensors; counter reset), then a3 (with a2
-    // for sigma_rel tensors) in one work-list launch
+    // a1 (alpha, c; sigma of fixed-sigma tensors; counter reset), then a2 and a3 in
+    // one work-list launch
     smat_status st = run_scalars(c, step, false, stream);
     if (st != SMAT_OK) return st;
     c->scalars_sigma = true;

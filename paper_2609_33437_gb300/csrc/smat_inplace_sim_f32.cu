@@ -14,4 +14,10 @@ cudaError_t SMAT_FAMILY(launch_simulate_inplace_f32)(const KArgs& a, int grid, i
                               : sim_run<10 | kFamily, DT_F32, true>(a, grid, noise, per_elem_alpha, s);
 }
 
+cudaError_t SMAT_FAMILY(launch_direct_inplace_f32)(const KArgs& a, int noise, bool per_elem_alpha, int rounds, cudaStream_t s) {
+  if (a.chunk_end <= a.chunk_begin) return cudaSuccess;
+  return (rounds & 0xFF) == 7 ? direct_run<7 | kFamily, DT_F32, true>(a, noise, per_elem_alpha, s)
+                              : direct_run<10 | kFamily, DT_F32, true>(a, noise, per_elem_alpha, s);
+}
+
 }  // namespace smat

@@ -154,6 +154,9 @@ cudaError_t launch_delta_stats(const KArgs& a, int grid, int dtype, cudaStream_t
 cudaError_t launch_scalars(const KArgs& a, int noise, int rounds, cudaStream_t s);
 cudaError_t launch_simulate(const KArgs& a, int grid, int dtype, int noise, bool per_elem_alpha,
                             int rounds, bool inplace, cudaStream_t s);
+// The forward of a list without statistics, scalars included, one CTA per chunk.
+cudaError_t launch_direct(const KArgs& a, int dtype, int noise, bool per_elem_alpha, int rounds, bool inplace,
+                          cudaStream_t s);
 cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise, bool per_elem_alpha,
                                   int rounds, bool inplace, cudaStream_t s);
 // The forward launchers below exist twice: as declared (the packed draw
@@ -191,6 +194,14 @@ cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise
                                                int rounds, cudaStream_t s);                                   \
   cudaError_t launch_simulate_inplace_bf16##sfx(const KArgs& a, int grid, int noise, bool per_elem_alpha,     \
                                                 int rounds, cudaStream_t s);                                  \
+  cudaError_t launch_direct_f32##sfx(const KArgs& a, int noise, bool per_elem_alpha, int rounds, cudaStream_t s);\
+  cudaError_t launch_direct_bf16##sfx(const KArgs& a, int noise, bool per_elem_alpha, int rounds, cudaStream_t s);\
+  cudaError_t launch_direct_inplace_f32##sfx(const KArgs& a, int noise, bool per_elem_alpha, int rounds,       \
+                                             cudaStream_t s);                                                  \
+  cudaError_t launch_direct_inplace_bf16##sfx(const KArgs& a, int noise, bool per_elem_alpha, int rounds,      \
+                                              cudaStream_t s);                                                 \
+  cudaError_t launch_direct_laplace_f32##sfx(const KArgs& a, bool per_elem_alpha, bool inplace, cudaStream_t s);\
+  cudaError_t launch_direct_laplace_bf16##sfx(const KArgs& a, bool per_elem_alpha, bool inplace, cudaStream_t s);\
   cudaError_t launch_gradmap##sfx(const KArgs& a, int grid, int gdtype, bool per_elem_alpha, bool accumulate, \
                                   int rounds, cudaStream_t s);                                                \
   int gradmap_ctas_per_sm##sfx(int gdtype, bool per_elem_alpha, bool accumulate, int rounds);                 \

@@ -32,4 +32,13 @@ int SMAT_FAMILY(laplace_ctas_per_sm_bf16)(bool per_elem_alpha) {
                         : FusedVariant<10 | kFamily, DT_BF16, NOISE_LAPLACE, false, false>::occ();
 }
 
+cudaError_t SMAT_FAMILY(launch_direct_laplace_bf16)(const KArgs& a, bool per_elem_alpha, bool inplace, cudaStream_t s) {
+  if (a.chunk_end <= a.chunk_begin) return cudaSuccess;
+  if (per_elem_alpha)
+    return inplace ? direct_run_one<10 | kFamily, DT_BF16, NOISE_LAPLACE, true, true>(a, s)
+                   : direct_run_one<10 | kFamily, DT_BF16, NOISE_LAPLACE, true, false>(a, s);
+  return inplace ? direct_run_one<10 | kFamily, DT_BF16, NOISE_LAPLACE, false, true>(a, s)
+                 : direct_run_one<10 | kFamily, DT_BF16, NOISE_LAPLACE, false, false>(a, s);
+}
+
 }  // namespace smat

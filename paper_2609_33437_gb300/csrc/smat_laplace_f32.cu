@@ -27,4 +27,13 @@ cudaError_t SMAT_FAMILY(launch_laplace_f32)(const KArgs& a, int grid, bool fused
   return inplace ? laplace_run<false, true>(a, grid, fused, s) : laplace_run<false, false>(a, grid, fused, s);
 }
 
+cudaError_t SMAT_FAMILY(launch_direct_laplace_f32)(const KArgs& a, bool per_elem_alpha, bool inplace, cudaStream_t s) {
+  if (a.chunk_end <= a.chunk_begin) return cudaSuccess;
+  if (per_elem_alpha)
+    return inplace ? direct_run_one<10 | kFamily, DT_F32, NOISE_LAPLACE, true, true>(a, s)
+                   : direct_run_one<10 | kFamily, DT_F32, NOISE_LAPLACE, true, false>(a, s);
+  return inplace ? direct_run_one<10 | kFamily, DT_F32, NOISE_LAPLACE, false, true>(a, s)
+                 : direct_run_one<10 | kFamily, DT_F32, NOISE_LAPLACE, false, false>(a, s);
+}
+
 }  // namespace smat

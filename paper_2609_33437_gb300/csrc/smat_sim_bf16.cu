@@ -17,4 +17,10 @@ int SMAT_FAMILY(simulate_ctas_per_sm_bf16)(int noise, bool per_elem_alpha, int r
                               : sim_occ<10 | kFamily, DT_BF16>(noise, per_elem_alpha);
 }
 
+cudaError_t SMAT_FAMILY(launch_direct_bf16)(const KArgs& a, int noise, bool per_elem_alpha, int rounds, cudaStream_t s) {
+  if (a.chunk_end <= a.chunk_begin) return cudaSuccess;
+  return (rounds & 0xFF) == 7 ? direct_run<7 | kFamily, DT_BF16, false>(a, noise, per_elem_alpha, s)
+                              : direct_run<10 | kFamily, DT_BF16, false>(a, noise, per_elem_alpha, s);
+}
+
 }  // namespace smat

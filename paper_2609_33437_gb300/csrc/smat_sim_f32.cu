@@ -17,4 +17,10 @@ int SMAT_FAMILY(simulate_ctas_per_sm_f32)(int noise, bool per_elem_alpha, int ro
                               : sim_occ<10 | kFamily, DT_F32>(noise, per_elem_alpha);
 }
 
+cudaError_t SMAT_FAMILY(launch_direct_f32)(const KArgs& a, int noise, bool per_elem_alpha, int rounds, cudaStream_t s) {
+  if (a.chunk_end <= a.chunk_begin) return cudaSuccess;
+  return (rounds & 0xFF) == 7 ? direct_run<7 | kFamily, DT_F32, false>(a, noise, per_elem_alpha, s)
+                              : direct_run<10 | kFamily, DT_F32, false>(a, noise, per_elem_alpha, s);
+}
+
 }  // namespace smat

@@ -79,3 +79,41 @@ def test_bounded_wait_runs_out_and_reports():
     sess2.simulate_multi(2)
     torch.cuda.synchronize()
     assert all(torch.equal(x.view(torch.int16), y.view(torch.int16)) for x, y in zip(sim, sess2._keep[2]))
+
+
+@pytest.mark.parametrize("noise", [S.SMAT_NOISE_UNIFORM, S.SMAT_NOISE_GAUSSIAN, S.SMAT_NOISE_LAPLACE])
+@pytest.mark.parametrize("alpha_mode", [S.SMAT_ALPHA_GLOBAL, S.SMAT_ALPHA_PER_TENSOR, S.SMAT_ALPHA_PER_ELEMENT])
+@pytest.mark.parametrize("draw_bits", [32, 16])
+def test_list_without_statistics_equals_the_grid_stride_forward(noise, alpha_mode, draw_bits):
+    """A list without sigma_rel tensors runs one launch per dtype that draws the
+    scalars itself; theta~ and the mapped gradients equal, bit for bit, those of
+    the separate scalars launch and grid-stride forward, over both dtypes in one
+    list, empty tensors, sizes around a group and a chunk, an offset, sigma 0, and
+    in place."""
+    sizes = [0, 1, 15, 16, 4097, 70_001, 16, 0, 131_072 + 5]
+    dts = [torch.bfloat16, torch.float32]
+    th = [(torch.randn(n, device="cuda") * 0.02).to(dts[k % 2]) for k, n in enumerate(sizes)]
+    t0 = [(t.float() + torch.randn(t.numel(), device="cuda") * 1e-3).to(t.dtype) for t in th]
+    gs = [torch.randn(n, device="cuda") for n in sizes]
+    keep = [0.5, 0.7, 1.0, 0.3, 0.9, 0.7, 0.0, 0.5, 0.3]
+    sigma = [1e-3, 1e-3, 0.0, 2e-3, 1e-3, 1e-4, 1e-3, 0.0, 1e-3]
+    got = []
+    for flags, inplace in ((0, False), (S.SMAT_FLAG_UNFUSED_STATS, False), (0, True), (S.SMAT_FLAG_CHUNK_LOG2(16), False)):
+        base = [t.clone() for t in t0]
+        sim = base if inplace else [torch.empty_like(t) for t in th]
+        sess = S.SmatSession(th, base, sim, keep, sigma, seed=21, alpha_min=0.2, alpha_mode=alpha_mode, noise=noise,
+                             flags=flags, draw_bits=draw_bits, elem_offsets=[16 * k for k in range(len(sizes))])
+        for step in (1, 4):
+            if inplace and step > 1:
+                for s, t in zip(sim, t0):
+                    s.copy_(t)
+                sess.mark_theta0_resident()
+            sess.simulate_multi(step)
+        out = [torch.empty_like(g) for g in gs]
+        sess.grad_map_multi(4, gs, out)
+        torch.cuda.synchronize()
+        got.append([x.view(torch.int16 if x.dtype == torch.bfloat16 else torch.int32) for x in sim + out])
+        sess.close()
+    for other in got[1:]:
+        for k, (a, b) in enumerate(zip(got[0], other)):
+            assert torch.equal(a, b), k

@@ -342,12 +342,11 @@ __device__ __forceinline__ void adam_chunk(const KArgs& a, const TView& v, const
   }
 }
 
-// The work of a launch: units of at most kMaxGradUnitElems in grid-stride
-// order, the last ones (fewer than the grid) in pieces, so that the CTAs end
-// together: 5.02 units per CTA took six units' time (1e8 bf16 elements 391 -> 352
-// us). The gradient map alone keeps whole units: its three CTAs per SM share the
-// bandwidth that an early one leaves, and the pieces cost more than they give
-// (bf16 75.5 -> 79.9 us).
+// The claims of a launch, one CTA each: units of at most kMaxGradUnitElems, the
+// last ones (fewer than the resident CTAs) in pieces. With two persistent CTAs per
+// SM and whole units, 5.02 units per CTA took six units' time (1e8 bf16 elements
+// 391 us; 354 with the pieces); a CTA per claim leaves the order to the hardware
+// (vision tower in fp32 1440 -> 1316 us, 1e8 fp32 elements 439 -> 427, bf16 358).
 __device__ __forceinline__ int64_t unit_claims(const KArgs& a) {
   const int64_t n = a.grad_units * (a.chunk_end - a.chunk_begin);
   return a.grad_whole + ((n - a.grad_whole) << a.grad_split);

@@ -330,6 +330,12 @@ struct Timed {
   }
 };
 
+// Gradient-map units of at most `most` elements (a power of two).
+void set_grad_unit(const smat_ctx* c, KArgs& a, int64_t most) {
+  a.grad_unit = std::min(c->chunk_elems, most);
+  a.grad_units = (int32_t)(c->chunk_elems / a.grad_unit);
+}
+
 KArgs base_args(const smat_ctx* c, uint32_t step) {
   KArgs a;
   std::memset(&a, 0, sizeof(a));
@@ -345,8 +351,7 @@ KArgs base_args(const smat_ctx* c, uint32_t step) {
   a.alpha_min = c->cfg.alpha_min;
   a.alpha_width = c->cfg.alpha_max - c->cfg.alpha_min;
   a.alpha_mode = c->cfg.alpha_mode;
-  a.grad_unit = std::min(c->chunk_elems, kMaxGradUnitElems);
-  a.grad_units = (int32_t)(c->chunk_elems / a.grad_unit);
+  set_grad_unit(c, a, kMaxGradUnitElems);
   if (c->d_sync) {
     a.work_counter = c->d_sync;
     a.error = c->d_sync + 2;
@@ -386,23 +391,16 @@ int grid_for(const smat_ctx* c, int64_t chunks, int dtype) {
   return (int)(chunks < resident ? chunks : resident);
 }
 
-// Grid of the work-list launch of one dtype range.
-int fused_grid(const smat_ctx* c, int dt) {
-  const int64_t chunks = c->range_end[dt] - c->range_begin[dt];
-  if (c->any_inplace || dt != SMAT_BF16) return grid_for(c, chunks, dt);
-  const int per_sm = fused_wide_occ(c->cfg.noise, c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT, c->rounds);
-  return (int)std::min(chunks, (int64_t)c->sm_count * per_sm);
-}
-
-// Grid of the fused AdamW launch over a's chunk range, and the split of its last
-// units (KArgs): up to eight pieces of at least 2^13 elements.
+// Grid of the fused AdamW launch over a's chunk range, one CTA per claim, and the
+// split of its last units (KArgs): whole units for as many full rounds of the
+// resident CTAs as there are, then up to eight pieces of at least 2^13 elements
+// per unit, so that the CTAs end together.
 int split_units(KArgs& a, int64_t resident) {
   const int64_t units = (a.chunk_end - a.chunk_begin) * (int64_t)a.grad_units;
   a.grad_split = 0;
   while (a.grad_split < 3 && (a.grad_unit >> (a.grad_split + 1)) >= 2 * kMinChunkElems) a.grad_split += 1;
   a.grad_whole = units / resident * resident;
-  const int64_t claims = a.grad_whole + ((units - a.grad_whole) << a.grad_split);
-  return (int)std::min(claims, resident);
+  return (int)std::min(a.grad_whole + ((units - a.grad_whole) << a.grad_split), int64_t(INT32_MAX));
 }
 
 // Rows a2 + a1: delta statistics (if needed) then the per-call scalars.
@@ -617,7 +615,7 @@ smat_status smat_simulate_multi(smat_ctx* c, uint32_t step, smat_stream_t stream
       a.items = c->d_items + c->item_begin[dt];
       a.n_items = c->item_count[dt];
       a.work_counter = c->d_sync + dt;
-      const int grid = fused_grid(c, dt);
+      const int grid = c->item_count[dt];  // one CTA per item
       Timed t(c, 2, stream);
       const cudaError_t e = launch_stats_simulate(a, grid, dt, c->cfg.noise, c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT,
                                                   c->rounds, c->any_inplace, stream);
@@ -696,13 +694,22 @@ smat_status smat_grad_map_multi(smat_ctx* c, uint32_t step, const void* const* g
   KArgs a = base_args(c, step);
   a.chunk_begin = 0;
   a.chunk_end = (int64_t)c->h_chunks.size();
-  const int64_t resident = (int64_t)c->sm_count *
-                           grad_map_occ(gdtype, c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT, accumulate != 0, c->rounds);
-  const int grid = (int)(a.chunk_end < resident ? a.chunk_end : resident);
+  const bool pe = c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT;
+  // One CTA per unit. fp32 gradients and per-element alpha take units of 2^15; the
+  // other bf16 maps, whose threads keep four groups in flight, lose on short units:
+  // they take 2^17, or where the list's chunks are smaller walk them in grid-stride
+  // order (1e8 elements: 75.5 us against 78.2 with a CTA per 2^16; 3.5e9 in chunks of
+  // 2^18: 2330 us against 2163 with a CTA per 2^17; fp32 accumulation on 4.9e8: 921
+  // us grid-stride, 847 per 2^17, 829 per 2^15).
+  const bool small = gdtype == SMAT_F32 || pe;
+  if (small) set_grad_unit(c, a, kSmallGradUnitElems);
+  const int64_t units = a.chunk_end * (int64_t)a.grad_units;
+  const int64_t resident = (int64_t)c->sm_count * grad_map_occ(gdtype, pe, accumulate != 0, c->rounds);
+  const int64_t most = small || a.grad_unit == kMaxGradUnitElems ? INT32_MAX : resident;
+  const int grid = (int)std::min(units, most);
   if (a.chunk_end <= 0) return SMAT_OK;
   Timed t(c, 3, stream);
-  const cudaError_t e = launch_grad_map(a, grid, gdtype, c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT,
-                                       accumulate != 0, c->rounds, stream);
+  const cudaError_t e = launch_grad_map(a, grid, gdtype, pe, accumulate != 0, c->rounds, stream);
   t.done();
   if (e != cudaSuccess) return cuda_fail(e, "gradient map launch");
   return SMAT_OK;
@@ -906,7 +913,7 @@ smat_status smat_debug_fused(smat_ctx* c, uint32_t step, const int32_t* d_items,
   a.items = d_items;
   a.n_items = n_items;
   a.work_counter = c->d_sync + SMAT_BF16;
-  e = launch_stats_simulate_bf16(a, fused_grid(c, SMAT_BF16), c->cfg.noise,
+  e = launch_stats_simulate_bf16(a, n_items, c->cfg.noise,
                                  c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT, c->rounds, stream);
   if (e != cudaSuccess) return cuda_fail(e, "fused launch");
   c->scalars_step = -1;  // sigma_t of this call may be incomplete

@@ -22,9 +22,8 @@ constexpr uint32_t kGlobalAlphaTensor = 0x0FFFFFFFu;
 // the first loads' latency) less often, many chunks keep every CTA busy to
 // the end; measured best from 2^22 to 2^32 elements. Always a multiple of 16, so a chunk never
 // splits a 16-element mask draw group of an aligned tensor. Statistics and
-// forward work items are whole chunks; the gradient map, whose CTAs take
-// its units in a fixed grid-stride order, walks units of at most
-// kMaxGradUnitElems so its CTAs end closer together.
+// forward work items are whole chunks; the gradient map takes units of at most
+// kMaxGradUnitElems, or kSmallGradUnitElems where a thread has one group in flight.
 // Stream variant code passed as `rounds` to the launchers below (and the `R`
 // template parameter of the kernels): the Philox rounds (10 or 7) in the low
 // byte, kDraw16 set for the 16-bit draw option (see smat_device.cuh).
@@ -33,6 +32,7 @@ constexpr int kDraw16 = 0x100;
 constexpr int64_t kMinChunkElems = int64_t(1) << 12;
 constexpr int64_t kMaxChunkElems = int64_t(1) << 18;
 constexpr int64_t kMaxGradUnitElems = int64_t(1) << 17;
+constexpr int64_t kSmallGradUnitElems = int64_t(1) << 15;
 constexpr int kMaxRounds = 10;
 
 enum : uint32_t {

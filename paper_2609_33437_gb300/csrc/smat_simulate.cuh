@@ -240,20 +240,20 @@ __device__ __forceinline__ void sim_chunk_noise(const KArgs& a, const TView& v, 
 }
 
 // ------------------------------------------- a2 + a3 fused (sigma_rel lists) ---
-// A persistent kernel that takes work items in list order from a counter:
-// statistics items (a2, one chunk each) and forward items (a3). Every
-// statistics item of a tensor precedes its forward items in the list (with a
-// lead of about one grid width), so the bandwidth-bound statistics of later
-// tensors run beside the compute-bound forward of earlier ones. The CTA that
-// finishes a tensor's last statistics chunk sums the chunk partials in chunk
-// order, publishes sigma_t and releases the tensor's ready flag; forward items
-// of that tensor wait for the flag.
+// Each CTA takes one work item, in list order by a ticket from a counter:
+// statistics items (a2, one chunk each) and forward items (a3). Every statistics
+// item of a tensor precedes its forward items in the list (with a lead of about
+// one grid width), so the bandwidth-bound statistics of later tensors run beside
+// the compute-bound forward of earlier ones. The CTA that finishes a tensor's last
+// statistics chunk sums the chunk partials in chunk order, publishes sigma_t and
+// releases the tensor's ready flag; forward items of that tensor wait for the
+// flag. (Persistent CTAs that took items until the list ended: 7B list 11.04 ms,
+// this 10.88 ms.)
 //
-// Progress: items are taken in list order and a statistics item never waits,
-// so every item a waiting forward item depends on is already held by a
-// running CTA. The wait is bounded all the same: after kWaitLimit polls
-// (about one second) it sets bit 0 of *a.error, skips the item and returns to
-// the queue.
+// Progress: a CTA takes its ticket when it runs, and a statistics item never
+// waits, so every item a waiting forward item depends on is already held by a
+// running CTA. The wait is bounded all the same: after kWaitLimit polls (about one
+// second) it sets bit 0 of *a.error and skips the item.
 __device__ __forceinline__ bool wait_ready(const KArgs& a, int t) { return wait_value(a.ready + t, a.epoch, a.error); }
 
 // All threads of the CTA call this for the same chunk (it has a barrier).
@@ -290,75 +290,72 @@ __global__ void __launch_bounds__(kBlock, kFusedCtas<DT, NOISE, PE, IP>)
   __shared__ int s_item;
   __shared__ int s_flag;
   __shared__ ChunkQueue s_cq;
-  for (;;) {
+  if (threadIdx.x == 0) {
+    s_item = atomicAdd(a.work_counter, 1);
+    s_cq.n_tie = 0;
+    s_cq.n_tail = 0;
+  }
+  __syncthreads();
+  const int it = s_item;
+  if (it >= a.n_items) return;  // same value in every thread
+  const uint32_t code = (uint32_t)a.items[it];
+  const int64_t ci = (int64_t)(code & ~kItemForward);
+  const Chunk ch = a.chunks[ci];
+  const DevTensor& T = a.tensors[ch.tensor];
+  if (!(code & kItemForward)) {
+    double ds, dq;
+    chunk_delta_sums<DT>(T, ch, sh_s, sh_q, ds, dq);
     if (threadIdx.x == 0) {
-      s_item = atomicAdd(a.work_counter, 1);
-      s_cq.n_tie = 0;
-      s_cq.n_tail = 0;
+      a.partials[ci].sum = ds;
+      a.partials[ci].sumsq = dq;
+      __threadfence();
+      s_flag = (atomicAdd(a.tensor_done + ch.tensor, 1) == T.n_chunks - 1) ? 1 : 0;
     }
     __syncthreads();
-    const int it = s_item;
-    if (it >= a.n_items) break;  // same value in every thread
-    const uint32_t code = (uint32_t)a.items[it];
-    const int64_t ci = (int64_t)(code & ~kItemForward);
-    const Chunk ch = a.chunks[ci];
-    const DevTensor& T = a.tensors[ch.tensor];
-    if (!(code & kItemForward)) {
-      double ds, dq;
-      chunk_delta_sums<DT>(T, ch, sh_s, sh_q, ds, dq);
+    if (s_flag) {
+      // last statistics chunk of this tensor: sum the partials in chunk order
+      __threadfence();
+      double s = 0.0, q = 0.0;
+      for (int k = threadIdx.x; k < T.n_chunks; k += kBlock) {
+        s += __ldcg(&a.partials[T.chunk_first + k].sum);
+        q += __ldcg(&a.partials[T.chunk_first + k].sumsq);
+      }
+      s = warp_sum(s);
+      q = warp_sum(q);
+      if ((threadIdx.x & 31) == 0) {
+        sh_s[threadIdx.x >> 5] = s;
+        sh_q[threadIdx.x >> 5] = q;
+      }
+      __syncthreads();
       if (threadIdx.x == 0) {
-        a.partials[ci].sum = ds;
-        a.partials[ci].sumsq = dq;
+        double ts = 0.0, tq = 0.0;
+        for (int w = 0; w < kBlock / 32; ++w) {
+          ts += sh_s[w];
+          tq += sh_q[w];
+        }
+        const float sigma = sigma_from_sums(ts, tq, T.numel, T.sigma_rel);
+        a.scal[ch.tensor].sigma = sigma;
+        a.scal[ch.tensor].noise_scale = noise_scale_of<NOISE>(sigma);
         __threadfence();
-        s_flag = (atomicAdd(a.tensor_done + ch.tensor, 1) == T.n_chunks - 1) ? 1 : 0;
-      }
-      __syncthreads();
-      if (s_flag) {
-        // last statistics chunk of this tensor: sum the partials in chunk order
-        __threadfence();
-        double s = 0.0, q = 0.0;
-        for (int k = threadIdx.x; k < T.n_chunks; k += kBlock) {
-          s += __ldcg(&a.partials[T.chunk_first + k].sum);
-          q += __ldcg(&a.partials[T.chunk_first + k].sumsq);
-        }
-        s = warp_sum(s);
-        q = warp_sum(q);
-        if ((threadIdx.x & 31) == 0) {
-          sh_s[threadIdx.x >> 5] = s;
-          sh_q[threadIdx.x >> 5] = q;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-          double ts = 0.0, tq = 0.0;
-          for (int w = 0; w < kBlock / 32; ++w) {
-            ts += sh_s[w];
-            tq += sh_q[w];
-          }
-          const float sigma = sigma_from_sums(ts, tq, T.numel, T.sigma_rel);
-          a.scal[ch.tensor].sigma = sigma;
-          a.scal[ch.tensor].noise_scale = noise_scale_of<NOISE>(sigma);
-          __threadfence();
-          st_release(a.ready + ch.tensor, a.epoch);
-        }
-      }
-    } else {
-      if (T.flags & TF_SIGMA_REL) {
-        if (threadIdx.x == 0) s_flag = wait_ready(a, ch.tensor) ? 1 : 0;
-        __syncthreads();
-      } else if (threadIdx.x == 0) {
-        s_flag = 1;
-      }
-      __syncthreads();
-      if (s_flag) {
-        DevScalars S;
-        S.alpha = __ldcg(&a.scal[ch.tensor].alpha);
-        S.c = __ldcg(&a.scal[ch.tensor].c);
-        S.sigma = __ldcg(&a.scal[ch.tensor].sigma);
-        S.noise_scale = __ldcg(&a.scal[ch.tensor].noise_scale);
-        forward_chunk<R, DT, NOISE, PE, IP>(a, make_view(T, S), T, ch, s_cq);
+        st_release(a.ready + ch.tensor, a.epoch);
       }
     }
-    __syncthreads();  // s_item, s_flag and the shared sums are reused by the next item
+  } else {
+    if (T.flags & TF_SIGMA_REL) {
+      if (threadIdx.x == 0) s_flag = wait_ready(a, ch.tensor) ? 1 : 0;
+      __syncthreads();
+    } else if (threadIdx.x == 0) {
+      s_flag = 1;
+    }
+    __syncthreads();
+    if (s_flag) {
+      DevScalars S;
+      S.alpha = __ldcg(&a.scal[ch.tensor].alpha);
+      S.c = __ldcg(&a.scal[ch.tensor].c);
+      S.sigma = __ldcg(&a.scal[ch.tensor].sigma);
+      S.noise_scale = __ldcg(&a.scal[ch.tensor].noise_scale);
+      forward_chunk<R, DT, NOISE, PE, IP>(a, make_view(T, S), T, ch, s_cq);
+    }
   }
 }
 

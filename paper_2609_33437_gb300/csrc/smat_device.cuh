@@ -13,10 +13,11 @@
 // All of them are multi-tensor launches over a chunk table (chunks of one
 // tensor, 2^12 to 2^18 elements, the size chosen per list). The forward of a
 // list without statistics has one CTA per chunk, which draws the chunk's scalars
-// itself; with statistics fused for sigma_rel tensors it is a persistent launch
-// whose CTAs take whole chunks from an ordered work list; the unfused statistics,
-// the forward beside them and the gradient map walk the table in grid-stride
-// order. Each thread owns 16 consecutive elements at a time (one 256-bit load
+// itself; with statistics fused for sigma_rel tensors one CTA per item of an
+// ordered work list (by ticket); the gradient map one CTA per unit, a part of a
+// chunk; the unfused statistics, the forward beside them and the bf16 gradient map
+// of short chunks walk the table in grid-stride order. Each thread owns 16
+// consecutive elements at a time (one 256-bit load
 // per bf16 input, two per fp32 input), which is exactly one Philox block of
 // the mask stream (16 high bytes) and three blocks of the noise stream (24
 // bits per element); with the 16-bit draw option, two blocks of each. The
@@ -562,6 +563,14 @@ __device__ __forceinline__ void load16(const void* base, int64_t i, Raw16<DT>& v
     ld32B(p, *reinterpret_cast<uint32_t(*)[8]>(v.r));
     ld32B(p + 8, *reinterpret_cast<uint32_t(*)[8]>(v.r + 8));
   }
+}
+
+// Ask for the 32-byte pieces of the same elements in L2 (no register waits for them).
+template <int DT>
+__device__ __forceinline__ void prefetch16(const void* base, int64_t i) {
+  const char* p = static_cast<const char*>(base) + i * (DT == DT_BF16 ? 2 : 4);
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+  if (DT != DT_BF16) asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 32));
 }
 
 template <int DT>

@@ -24,15 +24,15 @@ constexpr uint32_t kGlobalAlphaTensor = 0x0FFFFFFFu;
 // splits a 16-element mask draw group of an aligned tensor. Statistics and
 // forward work items are whole chunks; the gradient map takes units of at most
 // kMaxGradUnitElems, or kSmallGradUnitElems where a thread has one group in flight.
-// Stream variant code passed as `rounds` to the launchers below (and the `R`
-// template parameter of the kernels): the Philox rounds (10 or 7) in the low
-// byte, kDraw16 set for the 16-bit draw option (see smat_device.cuh).
-constexpr int kDraw16 = 0x100;
-
 constexpr int64_t kMinChunkElems = int64_t(1) << 12;
 constexpr int64_t kMaxChunkElems = int64_t(1) << 18;
 constexpr int64_t kMaxGradUnitElems = int64_t(1) << 17;
 constexpr int64_t kSmallGradUnitElems = int64_t(1) << 15;
+
+// Stream variant code passed as `rounds` to the launchers below (and the `R`
+// template parameter of the kernels): the Philox rounds (10 or 7) in the low
+// byte, kDraw16 set for the 16-bit draw option (see smat_device.cuh).
+constexpr int kDraw16 = 0x100;
 constexpr int kMaxRounds = 10;
 
 enum : uint32_t {
@@ -122,7 +122,7 @@ struct KArgs {
   int64_t chunk_end;
   int64_t grad_unit;     // gradient map: elements per unit (divides the chunk size)
   int32_t grad_units;    // gradient map: units per chunk
-  int64_t grad_whole;    // fused AdamW: units taken whole, a multiple of the grid; the rest in 2^grad_split pieces each
+  int64_t grad_whole;    // fused AdamW: units taken whole, a multiple of the resident CTAs; the rest in 2^grad_split pieces each
   int32_t grad_split;
   RoundKeys key;
   uint32_t step;

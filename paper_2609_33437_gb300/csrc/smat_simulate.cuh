@@ -182,6 +182,22 @@ struct ChunkQueue {
   int n_tail;
 };
 
+// Whether a pass asks for the next pass's inputs in L2 before its own draws, in
+// chunks of four passes or more (kAheadElems; 4e6 fp32 elements in two-pass chunks:
+// 14.5 us without, 14.8 with). fp32 groups at two CTAs per SM, and uniform and
+// noise-free bf16 groups, which do little arithmetic, wait for DRAM (long scoreboard
+// the largest stall, 5.5 per issue with bf16 and uniform noise). 1e8 fp32 elements:
+// uniform 188 -> 178 us (99% of the copy bandwidth), Gaussian 224 -> 213, Laplace
+// 225 -> 212, per-element alpha with uniform noise 200 -> 184, with Gaussian 246 ->
+// 241; bf16 vision tower with uniform noise 603 -> 593 us for the step, 7B layers with
+// statistics 1630 -> 1570; the next group held in registers at three CTAs per SM made
+// the step 623. The other bf16 laws are bound by their
+// arithmetic, where the two instructions cost more than they give (0.5B decoder,
+// Gaussian: 634 -> 642 us).
+template <int DT, int NOISE, bool PE>
+constexpr bool kAhead = DT == DT_F32 || (!PE && (NOISE == NOISE_UNIFORM || NOISE == NOISE_NONE));
+constexpr int64_t kAheadElems = 4 * 16 * (int64_t)kBlock;
+
 // IP: the launch may hold in-place tensors (a separate instantiation, so the
 // launches without any carry none of the in-place code).
 template <int R, int DT, int NOISE, bool PE, bool IDENT, bool J0, bool IP>
@@ -189,11 +205,17 @@ __device__ __forceinline__ void sim_chunk(const KArgs& a, const TView& v, const 
                                           const Chunk& ch, ChunkQueue& cq) {
   const bool vec = (v.flags & TF_VEC) != 0u;
   const bool masked = (v.flags & TF_MASK) != 0u;
+  const bool ahead = kAhead<DT, NOISE, PE> && ch.end - ch.begin >= kAheadElems;
   for (int64_t i = ch.begin + 16 * (int64_t)threadIdx.x; i < ch.end; i += 16 * (int64_t)kBlock) {
     if (vec && i + 16 <= ch.end) {
       Raw16<DT> th, t0;
       load16<DT>(T.theta, i, th);
       load16<DT>(T.theta0, i, t0);
+      const int64_t next = i + 16 * (int64_t)kBlock;
+      if (ahead && next + 16 <= ch.end) {
+        prefetch16<DT>(T.theta, next);
+        prefetch16<DT>(T.theta0, next);
+      }
       const uint32_t f = sim_group16<R, DT, NOISE, PE, IDENT, J0, false, IP>(a, v, th, t0, T.sim, i);
       if (f) {
         const uint32_t entry = (((uint32_t)(i - ch.begin) >> 4) << 2) | f;

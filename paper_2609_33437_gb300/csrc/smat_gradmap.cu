@@ -342,11 +342,10 @@ __device__ __forceinline__ void adam_chunk(const KArgs& a, const TView& v, const
   }
 }
 
-// The claims of a launch, one CTA each: units of at most kMaxGradUnitElems, the
-// last ones (fewer than the resident CTAs) in pieces. With two persistent CTAs per
-// SM and whole units, 5.02 units per CTA took six units' time (1e8 bf16 elements
-// 391 us; 354 with the pieces); a CTA per claim leaves the order to the hardware
-// (vision tower in fp32 1440 -> 1316 us, 1e8 fp32 elements 439 -> 427, bf16 358).
+// The claims of a launch, each one CTA's or shared out over the resident CTAs (the
+// host's rule): units of at most kMaxGradUnitElems, the last ones (fewer than the
+// resident CTAs) in pieces. With two persistent CTAs per SM and whole units, 5.02
+// units per CTA took six units' time (1e8 bf16 elements 391 us; 354 with the pieces).
 __device__ __forceinline__ int64_t unit_claims(const KArgs& a) {
   const int64_t n = a.grad_units * (a.chunk_end - a.chunk_begin);
   return a.grad_whole + ((n - a.grad_whole) << a.grad_split);

@@ -391,16 +391,16 @@ int grid_for(const smat_ctx* c, int64_t chunks, int dtype) {
   return (int)(chunks < resident ? chunks : resident);
 }
 
-// Grid of the fused AdamW launch over a's chunk range, one CTA per claim, and the
-// split of its last units (KArgs): whole units for as many full rounds of the
-// resident CTAs as there are, then up to eight pieces of at least 2^13 elements
-// per unit, so that the CTAs end together.
-int split_units(KArgs& a, int64_t resident) {
+// Claims of the fused AdamW launch over a's chunk range, and the split of its last
+// units (KArgs): whole units for as many full rounds of the resident CTAs as there
+// are, then up to eight pieces of at least 2^13 elements per unit, so that the CTAs
+// end together.
+int64_t split_units(KArgs& a, int64_t resident) {
   const int64_t units = (a.chunk_end - a.chunk_begin) * (int64_t)a.grad_units;
   a.grad_split = 0;
   while (a.grad_split < 3 && (a.grad_unit >> (a.grad_split + 1)) >= 2 * kMinChunkElems) a.grad_split += 1;
   a.grad_whole = units / resident * resident;
-  return (int)std::min(a.grad_whole + ((units - a.grad_whole) << a.grad_split), int64_t(INT32_MAX));
+  return std::min(a.grad_whole + ((units - a.grad_whole) << a.grad_split), int64_t(INT32_MAX));
 }
 
 // Rows a2 + a1: delta statistics (if needed) then the per-call scalars.
@@ -803,7 +803,15 @@ smat_status smat_grad_map_adamw_multi(smat_ctx* c, uint32_t step, const void* co
     a.chunk_end = c->range_end[dt];
     if (a.chunk_end <= a.chunk_begin) continue;
     const int pdt = dt == 0 ? SMAT_F32 : SMAT_BF16;
-    const int grid = split_units(a, (int64_t)c->sm_count * grad_map_adamw_occ(gdtype, pdt, pe, c->rounds));
+    // fp32 parameters take a CTA per claim (vision tower 1440 -> 1316 us, 3e8 elements
+    // 1285 -> 1214), and so do fp32 gradients of bf16 ones in units of 2^17 (0.5B decoder
+    // 1810 -> 1786); the other bf16 calls stay with the resident CTAs (2.35e8 elements
+    // with fp32 gradients in units of 2^16: 875 us with a CTA per claim, 856 resident;
+    // bf16 gradients: 1e8 359 and 354, 5.4e8 2298 and 2281).
+    const int64_t resident = (int64_t)c->sm_count * grad_map_adamw_occ(gdtype, pdt, pe, c->rounds);
+    const bool per_claim = pdt == SMAT_F32 || (gdtype == SMAT_F32 && a.grad_unit == kMaxGradUnitElems);
+    const int64_t claims = split_units(a, resident);
+    const int grid = (int)(per_claim ? claims : std::min(claims, resident));
     Timed tm(c, 3, stream);
     const cudaError_t e = launch_grad_map_adamw(a, grid, gdtype, pdt, pe, c->rounds, stream);
     tm.done();

@@ -56,10 +56,13 @@ int64_t merge_chunk_for(int64_t total) {
 constexpr int kHistBins = 2048;  // an interval's 2046 bins, one below it and one above it
 constexpr int kInner = kHistBins - 2;
 // Passes over the inputs: one or two when the sample's interval holds the
-// threshold; a miss costs one pass and leaves fewer than 2046 2^20 keys, which
-// three more decide (bins of at most 2^20, 2^10 and 1 keys).
+// threshold. An interval never reaches past kInfKey (NaN keys count in the bin
+// above it), so it is at most kInfKey + 1 <= 2046 2^20 keys wide and three passes
+// decide it (bins of at most 2^20, 2^10 and 1 keys); a miss costs one pass more.
 constexpr int kPasses = 4;
 constexpr uint32_t kInfKey = 0x7F800000u;
+static_assert((uint64_t(kInner) << 20) >= uint64_t(kInfKey) + 1 && (uint64_t(kInner) << 10) >= (1u << 20) && kInner >= 1 << 10,
+              "kPasses passes decide every slot");
 constexpr size_t kMergeAlign = 256;
 
 struct MTensor {
@@ -689,8 +692,10 @@ __global__ void __launch_bounds__(kSampleThreads) ties_sample_kernel(const __gri
     TiesSlot S;
     S.done = all ? 1u : 0u;
     S.pad = 0u;
-    const uint32_t lo = open_bottom ? 0u : prefix[1];
-    const uint32_t hi = open_top ? 0x7FFFFFFFu : prefix[0];
+    // NaN samples end the interval at kInfKey: from a NaN's key a miss below
+    // would span more than the passes can decide
+    const uint32_t lo = open_bottom ? 0u : min(prefix[1], kInfKey);
+    const uint32_t hi = open_top ? kInfKey : min(prefix[0], kInfKey);
     set_interval(S, lo, (uint64_t)hi - lo + 1);
     m.slots[slot] = S;
     if (all) {
@@ -904,10 +909,9 @@ __global__ void __launch_bounds__(kBlock) ties_select_kernel(const __grid_consta
       }
     }
     m.slots[slot] = S;
-    if (S.done) {
-      m.thr[slot] = thr;
-      atomicAdd(m.n_done, 1u);
-    }
+    // an undecided slot holds its interval's lower end: never a threshold that trims nothing
+    m.thr[slot] = S.done ? thr : S.lo;
+    if (S.done) atomicAdd(m.n_done, 1u);
   }
   __syncthreads();  // the bins have been read
   for (int b = threadIdx.x; b < kHistBins; b += kBlock) gh[b] = 0ull;

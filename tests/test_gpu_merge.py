@@ -53,7 +53,9 @@ def _check(t0s, exs, outs, dtype, method, kw, elem_offsets=None, thr=None):
         view = np.uint16 if dtype == O.BF16 else np.uint32
         assert np.array_equal(got.view(view), ref.view(view)), f"tensor {k}"
         if thr is not None:
-            assert np.array_equal(thr[k].cpu().numpy().view(np.uint32), rthr), f"tensor {k} thresholds"
+            nan = np.uint32(0x7F800001)  # the first of the NaN keys, which all stand for one threshold
+            got_thr = np.minimum(thr[k].cpu().numpy().view(np.uint32), nan)
+            assert np.array_equal(got_thr, np.minimum(rthr, nan)), f"tensor {k} thresholds"
 
 
 SIZES = [1, 15, 16, 17, 4096, 65_536 + 33, 131_073]
@@ -185,14 +187,16 @@ def test_merge_special_values(method, dtype):
 
 
 @pytest.mark.parametrize("dtype", [O.F32, O.BF16])
-@pytest.mark.parametrize("shape", ["normal", "mostly_zero", "sample_low", "sample_high", "infinities", "two_values"])
-@pytest.mark.parametrize("retention", [1e-4, 0.5, 1.0])
+@pytest.mark.parametrize("shape", ["normal", "mostly_zero", "sample_low", "sample_high", "infinities", "two_values",
+                                   "sample_nan", "sample_half_nan", "half_nan", "all_nan_but_sample"])
+@pytest.mark.parametrize("retention", [1e-4, 0.25, 0.5, 1.0])
 def test_merge_ties_threshold_selection(dtype, shape, retention):
     """Thresholds of tensors larger than the selection's sample (65,536
     elements, in 16-element groups at 16 floor(g (n / 16) / 4096)) equal the
     oracle's, also where the sample shows other magnitudes than the rest (its
     interval misses, and the next passes start from the whole range), where
-    most keys are equal, and with infinities."""
+    most keys are equal, with infinities, and with NaN in all or half of the
+    sample, all over the tensor, or everywhere else (a NaN threshold is any NaN)."""
     n, K = 200_000 + 37, 2
     g = torch.Generator().manual_seed(31)
     t0 = torch.randn(n, generator=g) * 0.02
@@ -211,6 +215,14 @@ def test_merge_ties_threshold_selection(dtype, shape, retention):
     elif shape == "two_values":
         d = torch.where(d > 0, 0.25, 0.5)
         t0 = torch.zeros(n)
+    elif shape == "sample_nan":
+        d[:, seen] = float("nan")
+    elif shape == "sample_half_nan":
+        d[(torch.rand(K, n, generator=g) < 0.5) & seen] = float("nan")
+    elif shape == "half_nan":
+        d[torch.rand(K, n, generator=g) < 0.5] = float("nan")
+    elif shape == "all_nan_but_sample":
+        d[:, ~seen] = float("nan")
     tdt = torch.bfloat16 if dtype == O.BF16 else torch.float32
     t0d = t0.to(tdt).cuda()
     exd = [(t0 + d[e]).to(tdt).cuda() for e in range(K)]

@@ -42,16 +42,25 @@ namespace smat {
 namespace {
 
 constexpr int kMergeMaxExperts = SMAT_MERGE_MAX_EXPERTS;
-// Elements per chunk of a merge: 2^16, or for lists of fewer than 2432 such
-// chunks (16 per SM) a smaller power of two down to 2^13, so that a small
-// merge is spread over the chip (61 chunks of 2^16 left most SMs idle: TIES of 4
-// experts of 4e6 fp32 elements spent 55 us in the merge pass, 14 at HBM speed).
+// Elements per chunk of a merge: 2^16, or for lists of fewer than kFewChunks
+// such chunks (16 per SM of a GB300's 152; a tuning value, any other count works)
+// a smaller power of two down to 2^13, so that a small merge is spread over the
+// chip (61 chunks of 2^16 left most SMs idle: TIES of 4 experts of 4e6 fp32
+// elements spent 55 us in the merge pass, 14 at HBM speed).
 constexpr int64_t kMergeChunkMax = int64_t(1) << 16;
 constexpr int64_t kMergeChunkMin = int64_t(1) << 13;
+constexpr int64_t kFewChunks = 16 * 152;
 int64_t merge_chunk_for(int64_t total) {
   int64_t c = kMergeChunkMax;
-  while (c > kMergeChunkMin && total / c < 2432) c /= 2;
+  while (c > kMergeChunkMin && total / c < kFewChunks) c /= 2;
   return c;
+}
+// Chunk records a workspace has room for: at least the chunks of n tensors of
+// total elements (n more than total / chunk at most, and total / chunk below
+// 2 kFewChunks where the chunk is not the largest), and no fewer for a list that
+// has grown, so that a workspace sized for a caller's largest list serves the others.
+int64_t merge_chunk_room(int64_t total, int32_t n) {
+  return n + std::min(total / kMergeChunkMin, 2 * kFewChunks + total / kMergeChunkMax);
 }
 constexpr int kHistBins = 2048;  // an interval's 2046 bins, one below it and one above it
 constexpr int kInner = kHistBins - 2;
@@ -944,12 +953,19 @@ struct MLayout {
 
 size_t align_m(size_t x) { return (x + kMergeAlign - 1) / kMergeAlign * kMergeAlign; }
 
-MLayout merge_layout(int32_t n, int64_t n_chunks, int K, bool ties) {
+// What merge_check finds of a list: its elements, chunk size, chunks and dtype
+// (one dtype per call).
+struct MPlan {
+  int64_t total, chunk, n_chunks;
+  int32_t dtype;
+};
+
+MLayout merge_layout(int32_t n, const MPlan& p, int K, bool ties) {
   MLayout L;
   size_t off = 0;
   const size_t slots = (size_t)n * (size_t)K;
   L.tensors = off; off = align_m(off + sizeof(MTensor) * (size_t)n);
-  L.chunks = off;  off = align_m(off + sizeof(Chunk) * (size_t)n_chunks);
+  L.chunks = off;  off = align_m(off + sizeof(Chunk) * (size_t)merge_chunk_room(p.total, n));
   L.experts = off; off = align_m(off + sizeof(void*) * slots);
   L.thr = off;     off = align_m(off + sizeof(uint32_t) * slots);
   L.slots = off;   off = align_m(off + sizeof(TiesSlot) * slots);
@@ -974,10 +990,8 @@ bool m_overlaps(const void* a, size_t na, const void* b, size_t nb) {
   return x < y + nb && y < x + na;
 }
 
-// Host-side validation (no device access); returns the chunk count and the
-// list's dtype (one dtype per call).
-smat_status merge_check(const smat_merge_tensor* t, int32_t n, const smat_merge_config* cfg, int64_t* n_chunks,
-                        int32_t* dtype_out) {
+// Host-side validation (no device access).
+smat_status merge_check(const smat_merge_tensor* t, int32_t n, const smat_merge_config* cfg, MPlan* plan) {
   if (!cfg) return mfail(SMAT_ERR_INVALID_ARG, "cfg is NULL");
   if (cfg->method < SMAT_MERGE_WA || cfg->method > SMAT_MERGE_TIES)
     return mfail(SMAT_ERR_UNSUPPORTED, "merge method %d not supported", cfg->method);
@@ -1024,8 +1038,7 @@ smat_status merge_check(const smat_merge_tensor* t, int32_t n, const smat_merge_
   const int64_t chunk = merge_chunk_for(total);
   for (int32_t k = 0; k < n; ++k) nc += (t[k].numel + chunk - 1) / chunk;
   if (nc >= (int64_t(1) << 31)) return mfail(SMAT_ERR_INVALID_ARG, "too many chunks");
-  *n_chunks = nc;
-  *dtype_out = n > 0 ? t[0].dtype : SMAT_F32;
+  *plan = {total, chunk, nc, n > 0 ? t[0].dtype : SMAT_F32};
   return SMAT_OK;
 }
 
@@ -1067,24 +1080,20 @@ using namespace smat;
 
 extern "C" size_t smat_merge_workspace_bytes(const smat_merge_tensor* tensors, int32_t n_tensors,
                                              const smat_merge_config* cfg) {
-  int64_t nc = 0;
-  int32_t dt = 0;
-  if (merge_check(tensors, n_tensors, cfg, &nc, &dt) != SMAT_OK) return 0;
-  return merge_layout(n_tensors, nc, cfg->n_experts, cfg->method == SMAT_MERGE_TIES).total;
+  MPlan plan;
+  if (merge_check(tensors, n_tensors, cfg, &plan) != SMAT_OK) return 0;
+  return merge_layout(n_tensors, plan, cfg->n_experts, cfg->method == SMAT_MERGE_TIES).total;
 }
 
 extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_tensors, const smat_merge_config* cfg,
                                   void* d_workspace, size_t workspace_bytes, smat_stream_t stream) {
-  int64_t nc = 0;
-  int32_t dtype = 0;
-  smat_status st = merge_check(tensors, n_tensors, cfg, &nc, &dtype);
+  MPlan plan;
+  smat_status st = merge_check(tensors, n_tensors, cfg, &plan);
   if (st != SMAT_OK) return st;
   const int K = cfg->n_experts;
   const bool ties = cfg->method == SMAT_MERGE_TIES;
-  int64_t total = 0;
-  for (int32_t k = 0; k < n_tensors; ++k) total = std::min(total + tensors[k].numel, int64_t(1) << 62);
-  const int64_t chunk = merge_chunk_for(total);
-  const MLayout L = merge_layout(n_tensors, nc, K, ties);
+  const int64_t chunk = plan.chunk, nc = plan.n_chunks;
+  const MLayout L = merge_layout(n_tensors, plan, K, ties);
   if (!d_workspace || (uintptr_t)d_workspace % kMergeAlign)
     return mfail(SMAT_ERR_WORKSPACE, "workspace NULL or not 256-byte aligned");
   if (workspace_bytes < L.total) return mfail(SMAT_ERR_WORKSPACE, "workspace %zu < %zu bytes", workspace_bytes, L.total);
@@ -1179,7 +1188,7 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
   const int64_t slots64 = (int64_t)slots;
   int64_t largest = 0;
   for (int32_t k = 0; k < n_tensors; ++k) largest = tensors[k].numel > largest ? tensors[k].numel : largest;
-  if (dtype == SMAT_BF16)
+  if (plan.dtype == SMAT_BF16)
     e = rounds == 7 ? merge_launch<7, DT_BF16>(m, slots64, largest, ties, sms, stream)
                     : merge_launch<10, DT_BF16>(m, slots64, largest, ties, sms, stream);
   else
@@ -1192,13 +1201,12 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
 extern "C" smat_status smat_merge_ties_thresholds(const smat_merge_tensor* tensors, int32_t n_tensors,
                                                   const smat_merge_config* cfg, const void* d_workspace,
                                                   uint32_t* d_out, smat_stream_t stream) {
-  int64_t nc = 0;
-  int32_t dtype = 0;
-  smat_status st = merge_check(tensors, n_tensors, cfg, &nc, &dtype);
+  MPlan plan;
+  smat_status st = merge_check(tensors, n_tensors, cfg, &plan);
   if (st != SMAT_OK) return st;
   if (cfg->method != SMAT_MERGE_TIES) return mfail(SMAT_ERR_STATE, "not a TIES configuration");
   if (!d_workspace || !d_out) return mfail(SMAT_ERR_INVALID_ARG, "NULL pointer");
-  const MLayout L = merge_layout(n_tensors, nc, cfg->n_experts, true);
+  const MLayout L = merge_layout(n_tensors, plan, cfg->n_experts, true);
   const size_t bytes = sizeof(uint32_t) * (size_t)n_tensors * (size_t)cfg->n_experts;
   if (bytes && cudaMemcpyAsync(d_out, static_cast<const char*>(d_workspace) + L.thr, bytes,
                                cudaMemcpyDeviceToDevice, stream) != cudaSuccess)

@@ -231,6 +231,37 @@ def test_merge_host_validation(L):
     assert ws([tens(), b]) == 0  # one dtype per call
 
 
+def test_merge_workspace_grows_with_the_list(L):
+    """A workspace sized for a list serves every list whose tensors are no
+    larger (the chunk size, which follows the list's size, does not show in the
+    bytes), and has room for the list's chunks of 2^13 to 2^16 elements."""
+    K = 2
+    exps = (ctypes.c_void_p * K)(3 << 50, 4 << 50)
+
+    def ws(numels, method):
+        arr = (S.MergeTensor * len(numels))()
+        for k, n in enumerate(numels):
+            t = arr[k]
+            t.theta0, t.out, t.numel, t.dtype, t.tensor_id = 1 << 50, 2 << 50, n, S.SMAT_BF16, k
+            t.experts = ctypes.cast(exps, ctypes.c_void_p)
+        c = S.MergeConfig(method, K, 0.5, 0.0, 0.5, 0, 10, 0)
+        return L.smat_merge_workspace_bytes(ctypes.byref(arr), len(numels), ctypes.byref(c))
+
+    edges = sorted({max(m + d, 0) for e in range(12, 37) for m in (1 << e, 2432 << min(e, 20)) for d in (-1, 0, 1)})
+    for method in (S.SMAT_MERGE_TA, S.SMAT_MERGE_TIES):
+        for make in (lambda n: [n], lambda n: [n // 3, n - n // 3], lambda n: [n, 5, 0, 65_537]):
+            last = 0
+            for n in edges:
+                numels = make(n)
+                chunk = 1 << 16
+                while chunk > 1 << 13 and sum(numels) // chunk < 2432:
+                    chunk //= 2
+                got = ws(numels, method)
+                assert got >= max(last, 24 * sum(-(-x // chunk) for x in numels)), (n, method)
+                last = got
+            assert ws(numels + [0], method) >= last
+
+
 def test_binding_matches_header_layout(tmp_path):
     """The ctypes binding agrees with include/smat.h as a C compiler reads it:
     the size and every field offset of each struct, the value of each constant

@@ -266,27 +266,53 @@ def test_fused_adamw_special_moments(dtype):
     sess.close()
 
 
-@pytest.mark.parametrize("pdt,gdt", [(torch.float32, torch.float32), (torch.bfloat16, torch.bfloat16)])
+@pytest.mark.parametrize("pdt,gdt", [(torch.float32, torch.float32), (torch.bfloat16, torch.bfloat16),
+                                     (torch.bfloat16, torch.float32)])
 def test_adamw_units_and_pieces_equal(pdt, gdt):
-    """The launch takes whole units and, past the last full round of the grid,
-    pieces of units: theta and the moments do not depend on the chunk size,
-    with fewer units than CTAs, a remainder of one unit, units too small to cut
-    and tensors that end inside a piece."""
-    sizes = [305 * (1 << 14) - 5, 4096, 70_001, 16]
-    t0 = [(torch.randn(n, device="cuda") * 0.02).to(pdt) for n in sizes]
-    gs = [torch.randn(n, device="cuda").to(gdt) for n in sizes]
+    """The launch takes whole units for as many full rounds of the resident CTAs
+    (two per SM, R) as there are, then pieces of units. One CTA takes each claim,
+    or the resident CTAs share them, by dtypes and unit length. theta and the
+    moments depend on none of it and equal the oracle's: one remaining unit in
+    eight pieces, ending inside one (chunks of 2^17: R + 1 units; 2^16: 2 R + 1),
+    two (2^18: R + 2, one of the whole ones empty), R - 2 in two pieces each (2^14),
+    none (2^15: 4 R units), and units too short to cut (2^12)."""
+    dev = torch.device("cuda")
+    R = 2 * torch.cuda.get_device_properties(dev).multi_processor_count
+    sizes = [((R - 2) << 17) - 5, 16, (1 << 17) + 80_003]
+    keeps = [0.7, 1.0, 0.3]
+    gen = torch.Generator(device=dev).manual_seed(23)
+    th0 = [(torch.randn(n, generator=gen, device=dev) * 0.02).to(pdt) for n in sizes]
+    gs = [torch.randn(n, generator=gen, device=dev).to(gdt) for n in sizes]
+    sim = [torch.empty_like(t) for t in th0]
     ref = None
-    for log2 in (12, 14, 15, 18):
-        th = [t.clone() for t in t0]
-        m1 = [torch.full((n,), 0.01, device="cuda") for n in sizes]
-        m2 = [torch.full((n,), 0.02, device="cuda") for n in sizes]
-        sess = S.SmatSession(th, t0, [torch.empty_like(t) for t in t0], [0.7, 1.0, 0.3, 0.5], [1e-3] * 4, seed=5,
-                             alpha_min=0.3, flags=S.SMAT_FLAG_CHUNK_LOG2(log2))
+    for log2 in (17, 18, 16, 15, 14, 12):
+        th = [t.clone() for t in th0]
+        m1 = [torch.full((n,), 0.01, device=dev) for n in sizes]
+        m2 = [torch.full((n,), 0.02, device=dev) for n in sizes]
+        sess = S.SmatSession(th, th0, sim, keeps, [1e-3] * 3, seed=5, alpha_min=0.3,
+                             flags=S.SMAT_FLAG_CHUNK_LOG2(log2))
         sess.simulate_multi(3)
-        sess.grad_map_adamw_multi(3, gs, m1, m2, lr=1e-3, weight_decay=0.01, adam_step=4)
+        sess.grad_map_adamw_multi(3, gs, m1, m2, adam_step=4, **HP)
         torch.cuda.synchronize()
-        got = [x.view(torch.int16 if x.dtype == torch.bfloat16 else torch.int32) for x in th + m1 + m2]
-        ref = got if ref is None else ref
-        for k, (a, b) in enumerate(zip(ref, got)):
-            assert torch.equal(a, b), (log2, k)
         sess.close()
+        got = [x.view(torch.int16 if x.dtype == torch.bfloat16 else torch.int32) for x in th + m1 + m2]
+        if ref is not None:
+            for k, (a, b) in enumerate(zip(ref, got)):
+                assert torch.equal(a, b), (log2, k)
+            continue
+        ref = got
+        cfg = O.config(seed=5, step=3, alpha_min=0.3, alpha_mode=O.ALPHA_GLOBAL, noise=O.NOISE_UNIFORM)
+        odt, ogt = (O.F32 if d == torch.float32 else O.BF16 for d in (pdt, gdt))
+        for k, n in enumerate(sizes):
+            rng = np.random.default_rng(k)
+            edges = (np.arange(0, n, 1 << 17)[:, None] + np.array([-1, 0])).reshape(-1)
+            idx = np.unique(np.concatenate([edges[edges >= 0], [n - 1], rng.integers(0, n, 20_000)]))
+            at = torch.from_numpy(idx).to(dev)
+            bits, a, b = O.gradmap_adamw_at(cfg, O.tensor(k, n, odt, keep_prob=keeps[k], sigma=1e-3), idx,
+                                            to_host(gs[k][at].float()), to_host(th0[k][at].float()),
+                                            np.full(idx.size, 0.01), np.full(idx.size, 0.02), adam_step=4, gdtype=ogt,
+                                            **HP)
+            stored = to_host(th[k][at])
+            assert np.array_equal(stored.astype(np.uint32) if odt == O.BF16 else stored.view(np.uint32), bits), k
+            assert np.array_equal(to_host(m1[k][at]).view(np.uint32), a.view(np.uint32)), k
+            assert np.array_equal(to_host(m2[k][at]).view(np.uint32), b.view(np.uint32)), k

@@ -110,19 +110,12 @@ struct MArgs {
 
 __device__ __forceinline__ uint32_t abs_key(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
 
-// Expert e's contribution to a 16-element group: acc += c Delta on the
-// elements whose bit is set in keep (bit k: element k).
+// An expert's contribution to a 16-element group: acc += c Delta.
 template <int DT>
-__device__ __forceinline__ void merge_acc16(float c, uint32_t keep, const Raw16<DT>& x, const Raw16<DT>& t0,
-                                            float2 (&acc)[8]) {
+__device__ __forceinline__ void merge_acc16(float c, const Raw16<DT>& x, const Raw16<DT>& t0, float2 (&acc)[8]) {
   const float2 c2 = splat(c);
 #pragma unroll
-  for (int h = 0; h < 8; ++h) {
-    const float2 b = t0.pair(h);
-    const float2 d = sub2_rn(x.pair(h), b);
-    const float2 f = fma2_rn(c2, d, acc[h]);
-    acc[h] = make_float2(((keep >> (2 * h)) & 1u) ? f.x : acc[h].x, ((keep >> (2 * h + 1)) & 1u) ? f.y : acc[h].y);
-  }
+  for (int h = 0; h < 8; ++h) acc[h] = fma2_rn(c2, sub2_rn(x.pair(h), t0.pair(h)), acc[h]);
 }
 
 template <int DT>
@@ -158,13 +151,13 @@ __device__ __forceinline__ void merge_linear16(const MArgs& m, const MTensor& T,
 #pragma unroll
     for (int b = 0; b < kExpertBatch; ++b) load16<DT>(xp[e + b], i, x[b]);
 #pragma unroll
-    for (int b = 0; b < kExpertBatch; ++b) merge_acc16<DT>(m.c, 0xFFFFu, x[b], t0, acc);
+    for (int b = 0; b < kExpertBatch; ++b) merge_acc16<DT>(m.c, x[b], t0, acc);
   }
 #pragma unroll 1
   for (; e < m.K; ++e) {
     Raw16<DT> x;
     load16<DT>(xp[e], i, x);
-    merge_acc16<DT>(m.c, 0xFFFFu, x, t0, acc);
+    merge_acc16<DT>(m.c, x, t0, acc);
   }
   store_merged16<DT>(T, i, t0, acc);
 }
@@ -468,52 +461,47 @@ __device__ __forceinline__ void merge_elem(const MArgs& m, const MTensor& T, int
   store1<DT>(T.out, i, __fadd_rn(t0, acc));
 }
 
-// TIES merge pass (no draws: one build for all stream variants).
+// TIES merge pass, one CTA per chunk (no draws: one build for all stream variants).
 template <int DT, int BATCH, bool FULL>
 __global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 3 : 2) ties_merge_kernel(const __grid_constant__ MArgs m) {
   __shared__ const void* s_x[kMergeMaxExperts];
   __shared__ float s_lo[kMergeMaxExperts];
-  for (int64_t ci = blockIdx.x; ci < m.n_chunks; ci += gridDim.x) {
-    const Chunk ch = m.chunks[ci];
-    const MTensor& T = m.tensors[ch.tensor];
-    const void* const t0_p = T.theta0;
-    void* const out_p = T.out;
-    const bool vec = (T.flags & TF_VEC) != 0u;
-    __syncthreads();
-    if (threadIdx.x < m.K) {
-      s_x[threadIdx.x] = m.experts[ch.tensor * m.K + threadIdx.x];
-      const uint32_t thr = m.thr[ch.tensor * m.K + threadIdx.x];
-      s_lo[threadIdx.x] = __uint_as_float(thr > 1u ? thr : 1u);
-    }
-    __syncthreads();
-    for (int64_t i = ch.begin + 8 * (int64_t)threadIdx.x; i < ch.end; i += 8 * (int64_t)kBlock) {
-      if (vec && i + 8 <= ch.end && merge_ties8<DT, BATCH, FULL>(m, t0_p, out_p, s_x, s_lo, i)) continue;
-      const int64_t e_end = (i + 8 < ch.end) ? i + 8 : ch.end;
+  const Chunk ch = m.chunks[blockIdx.x];
+  const MTensor& T = m.tensors[ch.tensor];
+  const void* const t0_p = T.theta0;
+  void* const out_p = T.out;
+  const bool vec = (T.flags & TF_VEC) != 0u;
+  if (threadIdx.x < m.K) {
+    s_x[threadIdx.x] = m.experts[ch.tensor * m.K + threadIdx.x];
+    const uint32_t thr = m.thr[ch.tensor * m.K + threadIdx.x];
+    s_lo[threadIdx.x] = __uint_as_float(thr > 1u ? thr : 1u);
+  }
+  __syncthreads();
+  for (int64_t i = ch.begin + 8 * (int64_t)threadIdx.x; i < ch.end; i += 8 * (int64_t)kBlock) {
+    if (vec && i + 8 <= ch.end && merge_ties8<DT, BATCH, FULL>(m, t0_p, out_p, s_x, s_lo, i)) continue;
+    const int64_t e_end = (i + 8 < ch.end) ? i + 8 : ch.end;
 #pragma unroll 1
-      for (int64_t e = i; e < e_end; ++e) merge_elem<10, DT, SMAT_MERGE_TIES>(m, T, ch.tensor, e);
-    }
+    for (int64_t e = i; e < e_end; ++e) merge_elem<10, DT, SMAT_MERGE_TIES>(m, T, ch.tensor, e);
   }
 }
 
-// WA and TA. bf16 at three CTAs per SM (76 registers): two left 7% of the copy
+// WA and TA (they differ in m.c alone), one CTA per chunk. bf16 at three CTAs per SM (76 registers): two left 7% of the copy
 // bandwidth unused, four spill (8 experts of 1e8 elements: 332, 309 and 357 us,
 // 16 experts 572, 541 and 636 us).
 template <int DT>
 constexpr int kLinearCtas = DT == DT_BF16 ? 3 : 2;
 
-template <int R, int DT, int METHOD>
+template <int DT>
 __global__ void __launch_bounds__(kBlock, kLinearCtas<DT>) merge_kernel(const __grid_constant__ MArgs m) {
-  for (int64_t ci = blockIdx.x; ci < m.n_chunks; ci += gridDim.x) {
-    const Chunk ch = m.chunks[ci];
-    const MTensor& T = m.tensors[ch.tensor];
-    const bool vec = (T.flags & TF_VEC) != 0u;
-    for (int64_t i = ch.begin + 16 * (int64_t)threadIdx.x; i < ch.end; i += 16 * (int64_t)kBlock) {
-      if (vec && i + 16 <= ch.end) {
-        merge_linear16<DT>(m, T, ch.tensor, i);
-      } else {
-        const int64_t e_end = (i + 16 < ch.end) ? i + 16 : ch.end;
-        for (int64_t e = i; e < e_end; ++e) merge_elem<R, DT, METHOD>(m, T, ch.tensor, e);
-      }
+  const Chunk ch = m.chunks[blockIdx.x];
+  const MTensor& T = m.tensors[ch.tensor];
+  const bool vec = (T.flags & TF_VEC) != 0u;
+  for (int64_t i = ch.begin + 16 * (int64_t)threadIdx.x; i < ch.end; i += 16 * (int64_t)kBlock) {
+    if (vec && i + 16 <= ch.end) {
+      merge_linear16<DT>(m, T, ch.tensor, i);
+    } else {
+      const int64_t e_end = (i + 16 < ch.end) ? i + 16 : ch.end;
+      for (int64_t e = i; e < e_end; ++e) merge_elem<10, DT, SMAT_MERGE_TA>(m, T, ch.tensor, e);
     }
   }
 }
@@ -927,22 +915,14 @@ __global__ void __launch_bounds__(kBlock) ties_select_kernel(const __grid_consta
 }
 
 template <int R, int DT>
-cudaError_t merge_method(const MArgs& m, int grid, cudaStream_t s) {
-  switch (m.method) {
-    case SMAT_MERGE_WA: merge_kernel<R, DT, SMAT_MERGE_WA><<<grid, kBlock, 0, s>>>(m); break;
-    case SMAT_MERGE_TA: merge_kernel<R, DT, SMAT_MERGE_TA><<<grid, kBlock, 0, s>>>(m); break;
-    case SMAT_MERGE_DARE_TA: {
-      const size_t smem = dare_smem_bytes(m.K);
-      if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(dare_kernel<R, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem);
-        if (e != cudaSuccess) return e;
-      }
-      dare_kernel<R, DT><<<grid, kBlock, smem, s>>>(m);
-      break;
-    }
-    default: return cudaErrorInvalidValue;  // TIES: ties_merge_run
+cudaError_t dare_run(const MArgs& m, int grid, cudaStream_t s) {
+  const size_t smem = dare_smem_bytes(m.K);
+  if (smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(dare_kernel<R, DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)smem);
+    if (e != cudaSuccess) return e;
   }
+  dare_kernel<R, DT><<<grid, kBlock, smem, s>>>(m);
   return cudaGetLastError();
 }
 
@@ -1048,9 +1028,9 @@ cudaError_t ties_merge_run(const MArgs& m, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <int R, int DT>
-cudaError_t merge_launch(MArgs m, int64_t slots, int64_t largest, bool ties, int sms, cudaStream_t s) {
-  if (ties) {
+template <int DT>
+cudaError_t merge_launch(MArgs m, int64_t slots, int64_t largest, int rounds, int sms, cudaStream_t s) {
+  if (m.method == SMAT_MERGE_TIES) {
     const int64_t items = m.n_chunks * ((m.K + kHistExperts - 1) / kHistExperts);  // one CTA each
     m.n_slots = (int32_t)slots;
     ties_sample_kernel<DT><<<(int)slots, kSampleThreads, 0, s>>>(m);
@@ -1059,8 +1039,6 @@ cudaError_t merge_launch(MArgs m, int64_t slots, int64_t largest, bool ties, int
       ties_hist_kernel<DT><<<(int)std::min(items, int64_t(INT32_MAX)), kBlock, 0, s>>>(m);
       ties_select_kernel<DT><<<(int)slots, kBlock, 0, s>>>(m);
     }
-  }
-  if (ties) {
     if constexpr (DT == DT_BF16)
       if (m.K % 8 == 0) return ties_merge_run<DT, 8, true>(m, s);
     if (m.K % 4 == 0) return ties_merge_run<DT, 4, true>(m, s);
@@ -1069,8 +1047,12 @@ cudaError_t merge_launch(MArgs m, int64_t slots, int64_t largest, bool ties, int
   // one CTA per chunk, started by the hardware as others end (8 experts of 1e8 bf16
   // elements 309 -> 306 us, 16 experts 542 -> 534 us); DARE's CTAs, with their
   // shared memory, are worth keeping (4e7 elements: 175 against 187 us)
-  const int64_t grid = m.method == SMAT_MERGE_DARE_TA && m.n_chunks > 2 * (int64_t)sms ? 2 * (int64_t)sms : m.n_chunks;
-  return merge_method<R, DT>(m, (int)grid, s);
+  if (m.method == SMAT_MERGE_DARE_TA) {
+    const int grid = (int)std::min(m.n_chunks, 2 * (int64_t)sms);
+    return rounds == 7 ? dare_run<7, DT>(m, grid, s) : dare_run<10, DT>(m, grid, s);
+  }
+  merge_kernel<DT><<<(int)m.n_chunks, kBlock, 0, s>>>(m);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -1189,11 +1171,9 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
   int64_t largest = 0;
   for (int32_t k = 0; k < n_tensors; ++k) largest = tensors[k].numel > largest ? tensors[k].numel : largest;
   if (plan.dtype == SMAT_BF16)
-    e = rounds == 7 ? merge_launch<7, DT_BF16>(m, slots64, largest, ties, sms, stream)
-                    : merge_launch<10, DT_BF16>(m, slots64, largest, ties, sms, stream);
+    e = merge_launch<DT_BF16>(m, slots64, largest, rounds, sms, stream);
   else
-    e = rounds == 7 ? merge_launch<7, DT_F32>(m, slots64, largest, ties, sms, stream)
-                    : merge_launch<10, DT_F32>(m, slots64, largest, ties, sms, stream);
+    e = merge_launch<DT_F32>(m, slots64, largest, rounds, sms, stream);
   if (e != cudaSuccess) return mfail(SMAT_ERR_CUDA, "merge launch failed");
   return SMAT_OK;
 }

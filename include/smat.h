@@ -398,8 +398,8 @@ typedef struct {
 } smat_merge_config;
 
 /* Bytes of device workspace smat_merge needs (0 on invalid arguments). They
- * never fall as tensors grow or are added: a workspace sized for a program's
- * largest list serves its smaller ones (same method, no more experts). */
+ * grow with the tensors and experts, not with the tensors' sizes: a workspace
+ * serves any list of no more of either (same method). */
 size_t smat_merge_workspace_bytes(const smat_merge_tensor* tensors, int32_t n_tensors,
                                   const smat_merge_config* cfg);
 

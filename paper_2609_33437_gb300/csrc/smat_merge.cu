@@ -55,13 +55,6 @@ int64_t merge_chunk_for(int64_t total) {
   while (c > kMergeChunkMin && total / c < kFewChunks) c /= 2;
   return c;
 }
-// Chunk records a workspace has room for: at least the chunks of n tensors of
-// total elements (n more than total / chunk at most, and total / chunk below
-// 2 kFewChunks where the chunk is not the largest), and no fewer for a list that
-// has grown, so that a workspace sized for a caller's largest list serves the others.
-int64_t merge_chunk_room(int64_t total, int32_t n) {
-  return n + std::min(total / kMergeChunkMin, 2 * kFewChunks + total / kMergeChunkMax);
-}
 constexpr int kHistBins = 2048;  // an interval's 2046 bins, one below it and one above it
 constexpr int kInner = kHistBins - 2;
 // Passes over the inputs: one or two when the sample's interval holds the
@@ -91,22 +84,51 @@ struct TiesSlot {  // 16 bytes
   uint32_t pad;
 };
 
+// A list cut into chunks of `elems` elements, one tensor after the other: first[t]
+// is tensor t's first chunk, first[n_tensors] == n the number of chunks.
+struct ChunkSplit {
+  const int32_t* first;
+  int64_t elems;
+  int64_t n;
+};
+
 struct MArgs {
   const MTensor* tensors;
-  const Chunk* chunks;
+  ChunkSplit chunks;
   const void* const* experts;  // [tensor * K + e]
   uint32_t* thr;               // [tensor * K + e] TIES threshold keys
   TiesSlot* slots;             // [tensor * K + e]
   int64_t* rank;               // r of each slot (1 = the largest key)
   uint32_t* n_done;            // slots decided so far
   unsigned long long* hist;    // [(tensor * K + e) * kHistBins], see ties_hist_kernel
-  int64_t n_chunks;
   RoundKeys key;
   int32_t K, method;
+  int32_t n_tensors;
   float gamma, c;              // c: per-expert coefficient (WA 1/K, TA gamma, DARE gamma / p_keep)
   int32_t n_slots;
-  int64_t chunk;               // elements per chunk
 };
+
+// Chunk c of the split, by a binary search of the tensors' first chunks (they stay in
+// L1: the streaming loads allocate no lines there). A table with a record per chunk took
+// one load, but beyond 64 KB its upload from pageable memory waits for the stream,
+// and a merge call then does not return before the work ahead of it is done (two
+// experts of 3.5e7 fp32 elements, called in a row: 111 us each with 102 KB of records,
+// 93 now). Without a barrier: finding it together, with one load per thread, made the
+// DARE kernel's warps wait for each other at every chunk (0.5B decoder 2366 -> 2407 us).
+__device__ __forceinline__ Chunk chunk_of(const MArgs& m, const ChunkSplit& split, int64_t c) {
+  int lo = 0, hi = m.n_tensors;  // first[lo] <= c < first[hi]
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (split.first[mid] <= c) lo = mid;
+    else hi = mid;
+  }
+  Chunk ch;
+  ch.tensor = lo;
+  ch.pad = 0;
+  ch.begin = (c - split.first[lo]) * split.elems;
+  ch.end = min(ch.begin + split.elems, m.tensors[lo].numel);
+  return ch;
+}
 
 __device__ __forceinline__ uint32_t abs_key(float x) { return __float_as_uint(x) & 0x7FFFFFFFu; }
 
@@ -466,7 +488,7 @@ template <int DT, int BATCH, bool FULL>
 __global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 3 : 2) ties_merge_kernel(const __grid_constant__ MArgs m) {
   __shared__ const void* s_x[kMergeMaxExperts];
   __shared__ float s_lo[kMergeMaxExperts];
-  const Chunk ch = m.chunks[blockIdx.x];
+  const Chunk ch = chunk_of(m, m.chunks, blockIdx.x);
   const MTensor& T = m.tensors[ch.tensor];
   const void* const t0_p = T.theta0;
   void* const out_p = T.out;
@@ -493,7 +515,7 @@ constexpr int kLinearCtas = DT == DT_BF16 ? 3 : 2;
 
 template <int DT>
 __global__ void __launch_bounds__(kBlock, kLinearCtas<DT>) merge_kernel(const __grid_constant__ MArgs m) {
-  const Chunk ch = m.chunks[blockIdx.x];
+  const Chunk ch = chunk_of(m, m.chunks, blockIdx.x);
   const MTensor& T = m.tensors[ch.tensor];
   const bool vec = (T.flags & TF_VEC) != 0u;
   for (int64_t i = ch.begin + 16 * (int64_t)threadIdx.x; i < ch.end; i += 16 * (int64_t)kBlock) {
@@ -517,8 +539,8 @@ __global__ void __launch_bounds__(kBlock, 2) dare_kernel(const __grid_constant__
   DareShared s;
   s.keep = reinterpret_cast<uint4*>(dare_smem);
   s.queue = reinterpret_cast<uint16_t*>(s.keep + m.K * kBlock) + 32 * m.K * warp;
-  for (int64_t ci = blockIdx.x; ci < m.n_chunks; ci += gridDim.x) {
-    const Chunk ch = m.chunks[ci];
+  for (int64_t ci = blockIdx.x; ci < m.chunks.n; ci += gridDim.x) {
+    const Chunk ch = chunk_of(m, m.chunks, ci);
     const MTensor& T = m.tensors[ch.tensor];
     const bool vec = (T.flags & TF_VEC) != 0u;
     const bool masked = (T.flags & TF_MASK) != 0u;
@@ -752,12 +774,11 @@ __global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 3) ties_hist_kerne
   __shared__ int n_list;
   if (*m.n_done == (uint32_t)m.n_slots) return;
   const int nbat = (m.K + kHistExperts - 1) / kHistExperts;
-  const int64_t items = m.n_chunks * nbat;
+  const int64_t items = m.chunks.n * nbat;
   for (int64_t w = blockIdx.x; w < items; w += gridDim.x) {
-    const int64_t ci = w / nbat;
     const int e0 = (int)(w % nbat) * kHistExperts;
     const int ne = m.K - e0 < kHistExperts ? m.K - e0 : kHistExperts;
-    const Chunk ch = m.chunks[ci];
+    const Chunk ch = chunk_of(m, m.chunks, w / nbat);
     const MTensor& T = m.tensors[ch.tensor];
     const int slot0 = ch.tensor * m.K + e0;
     uint32_t lo[kHistExperts];
@@ -855,7 +876,7 @@ __global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 3) ties_hist_kerne
     }
     // the ne histograms are consecutive slots' bins in the global array
     unsigned long long* gh = m.hist + (size_t)slot0 * kHistBins;
-    const uint32_t most = T.numel <= kOffChunks * m.chunk ? kOffMost : 1u;
+    const uint32_t most = T.numel <= kOffChunks * m.chunks.elems ? kOffMost : 1u;
     for (int b = threadIdx.x; b < ne * kHistBins; b += kBlock) {
       const uint32_t c = h[b];
       if (c) {
@@ -928,7 +949,7 @@ cudaError_t dare_run(const MArgs& m, int grid, cudaStream_t s) {
 
 // ------------------------------------------------------------------- host ---
 struct MLayout {
-  size_t tensors, chunks, experts, thr, slots, n_done, rank, hist, total;
+  size_t tensors, first, experts, thr, slots, n_done, rank, hist, total;
 };
 
 size_t align_m(size_t x) { return (x + kMergeAlign - 1) / kMergeAlign * kMergeAlign; }
@@ -940,12 +961,13 @@ struct MPlan {
   int32_t dtype;
 };
 
-MLayout merge_layout(int32_t n, const MPlan& p, int K, bool ties) {
+// A workspace's bytes grow with the tensors and experts alone.
+MLayout merge_layout(int32_t n, int K, bool ties) {
   MLayout L;
   size_t off = 0;
   const size_t slots = (size_t)n * (size_t)K;
   L.tensors = off; off = align_m(off + sizeof(MTensor) * (size_t)n);
-  L.chunks = off;  off = align_m(off + sizeof(Chunk) * (size_t)merge_chunk_room(p.total, n));
+  L.first = off;   off = align_m(off + sizeof(int32_t) * ((size_t)n + 1));
   L.experts = off; off = align_m(off + sizeof(void*) * slots);
   L.thr = off;     off = align_m(off + sizeof(uint32_t) * slots);
   L.slots = off;   off = align_m(off + sizeof(TiesSlot) * slots);
@@ -1024,14 +1046,14 @@ smat_status merge_check(const smat_merge_tensor* t, int32_t n, const smat_merge_
 
 template <int DT, int BATCH, bool FULL>
 cudaError_t ties_merge_run(const MArgs& m, cudaStream_t s) {
-  ties_merge_kernel<DT, BATCH, FULL><<<(int)m.n_chunks, kBlock, 0, s>>>(m);
+  ties_merge_kernel<DT, BATCH, FULL><<<(int)m.chunks.n, kBlock, 0, s>>>(m);
   return cudaGetLastError();
 }
 
 template <int DT>
 cudaError_t merge_launch(MArgs m, int64_t slots, int64_t largest, int rounds, int sms, cudaStream_t s) {
   if (m.method == SMAT_MERGE_TIES) {
-    const int64_t items = m.n_chunks * ((m.K + kHistExperts - 1) / kHistExperts);  // one CTA each
+    const int64_t items = m.chunks.n * ((m.K + kHistExperts - 1) / kHistExperts);  // one CTA each
     m.n_slots = (int32_t)slots;
     ties_sample_kernel<DT><<<(int)slots, kSampleThreads, 0, s>>>(m);
     // no pass where every tensor is small enough for the sample to decide
@@ -1048,10 +1070,10 @@ cudaError_t merge_launch(MArgs m, int64_t slots, int64_t largest, int rounds, in
   // elements 309 -> 306 us, 16 experts 542 -> 534 us); DARE's CTAs, with their
   // shared memory, are worth keeping (4e7 elements: 175 against 187 us)
   if (m.method == SMAT_MERGE_DARE_TA) {
-    const int grid = (int)std::min(m.n_chunks, 2 * (int64_t)sms);
+    const int grid = (int)std::min(m.chunks.n, 2 * (int64_t)sms);
     return rounds == 7 ? dare_run<7, DT>(m, grid, s) : dare_run<10, DT>(m, grid, s);
   }
-  merge_kernel<DT><<<(int)m.n_chunks, kBlock, 0, s>>>(m);
+  merge_kernel<DT><<<(int)m.chunks.n, kBlock, 0, s>>>(m);
   return cudaGetLastError();
 }
 
@@ -1064,7 +1086,7 @@ extern "C" size_t smat_merge_workspace_bytes(const smat_merge_tensor* tensors, i
                                              const smat_merge_config* cfg) {
   MPlan plan;
   if (merge_check(tensors, n_tensors, cfg, &plan) != SMAT_OK) return 0;
-  return merge_layout(n_tensors, plan, cfg->n_experts, cfg->method == SMAT_MERGE_TIES).total;
+  return merge_layout(n_tensors, cfg->n_experts, cfg->method == SMAT_MERGE_TIES).total;
 }
 
 extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_tensors, const smat_merge_config* cfg,
@@ -1074,8 +1096,7 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
   if (st != SMAT_OK) return st;
   const int K = cfg->n_experts;
   const bool ties = cfg->method == SMAT_MERGE_TIES;
-  const int64_t chunk = plan.chunk, nc = plan.n_chunks;
-  const MLayout L = merge_layout(n_tensors, plan, K, ties);
+  const MLayout L = merge_layout(n_tensors, K, ties);
   if (!d_workspace || (uintptr_t)d_workspace % kMergeAlign)
     return mfail(SMAT_ERR_WORKSPACE, "workspace NULL or not 256-byte aligned");
   if (workspace_bytes < L.total) return mfail(SMAT_ERR_WORKSPACE, "workspace %zu < %zu bytes", workspace_bytes, L.total);
@@ -1086,14 +1107,13 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
     for (int e = 0; ok && e < K; ++e) ok = access.check(tensors[k].experts[e]) == 1;
     if (!ok) return mfail(SMAT_ERR_INVALID_ARG, "tensor %d: a pointer is not accessible from the GPU", k);
   }
-  if (n_tensors == 0 || nc == 0) return SMAT_OK;
+  if (n_tensors == 0 || plan.n_chunks == 0) return SMAT_OK;
 
   // tables (host), then one upload each
   const float keep = 1.0f - cfg->p_drop;
   const uint64_t T = (uint64_t)std::floor((double)keep * 4294967296.0);
   std::vector<MTensor> ht((size_t)n_tensors);
-  std::vector<Chunk> hc;
-  hc.reserve((size_t)nc);
+  std::vector<int32_t> first((size_t)n_tensors + 1, 0);
   std::vector<const void*> hx((size_t)n_tensors * (size_t)K, nullptr);
   std::vector<int64_t> hrank((size_t)n_tensors * (size_t)K, 0);
   for (int32_t k = 0; k < n_tensors; ++k) {
@@ -1122,28 +1142,20 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
       r = r < 1 ? 1 : (r > d.numel ? d.numel : r);
       for (int e = 0; e < K; ++e) hrank[(size_t)k * K + e] = r;
     }
-    for (int64_t j = 0; j * chunk < d.numel; ++j) {
-      Chunk ch;
-      ch.tensor = k;
-      ch.pad = 0;
-      ch.begin = j * chunk;
-      ch.end = (j + 1) * chunk < d.numel ? (j + 1) * chunk : d.numel;
-      hc.push_back(ch);
-    }
+    first[(size_t)k + 1] = first[(size_t)k] + (int32_t)((d.numel + plan.chunk - 1) / plan.chunk);
   }
   char* ws = static_cast<char*>(d_workspace);
   MArgs m;
   std::memset(&m, 0, sizeof(m));
   m.tensors = reinterpret_cast<const MTensor*>(ws + L.tensors);
-  m.chunks = reinterpret_cast<const Chunk*>(ws + L.chunks);
+  m.chunks = {reinterpret_cast<const int32_t*>(ws + L.first), plan.chunk, plan.n_chunks};
   m.experts = reinterpret_cast<const void* const*>(ws + L.experts);
   m.thr = reinterpret_cast<uint32_t*>(ws + L.thr);
   m.slots = reinterpret_cast<TiesSlot*>(ws + L.slots);
   m.n_done = reinterpret_cast<uint32_t*>(ws + L.n_done);
   m.rank = reinterpret_cast<int64_t*>(ws + L.rank);
   m.hist = ties ? reinterpret_cast<unsigned long long*>(ws + L.hist) : nullptr;
-  m.n_chunks = nc;
-  m.chunk = chunk;
+  m.n_tensors = n_tensors;
   m.key = make_round_keys(cfg->seed);
   m.K = K;
   m.method = cfg->method;
@@ -1153,7 +1165,7 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
         : cfg->method == SMAT_MERGE_DARE_TA ? cfg->gamma * inv_keep : cfg->gamma;
   const size_t slots = (size_t)n_tensors * (size_t)K;
   cudaError_t e = cudaMemcpyAsync(ws + L.tensors, ht.data(), sizeof(MTensor) * ht.size(), cudaMemcpyHostToDevice, stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.chunks, hc.data(), sizeof(Chunk) * hc.size(), cudaMemcpyHostToDevice, stream);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.first, first.data(), sizeof(int32_t) * first.size(), cudaMemcpyHostToDevice, stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.experts, hx.data(), sizeof(void*) * slots, cudaMemcpyHostToDevice, stream);
   if (e != cudaSuccess) return mfail(SMAT_ERR_CUDA, "merge table upload failed");
   int dev = 0, sms = 1;
@@ -1186,7 +1198,7 @@ extern "C" smat_status smat_merge_ties_thresholds(const smat_merge_tensor* tenso
   if (st != SMAT_OK) return st;
   if (cfg->method != SMAT_MERGE_TIES) return mfail(SMAT_ERR_STATE, "not a TIES configuration");
   if (!d_workspace || !d_out) return mfail(SMAT_ERR_INVALID_ARG, "NULL pointer");
-  const MLayout L = merge_layout(n_tensors, plan, cfg->n_experts, true);
+  const MLayout L = merge_layout(n_tensors, cfg->n_experts, true);
   const size_t bytes = sizeof(uint32_t) * (size_t)n_tensors * (size_t)cfg->n_experts;
   if (bytes && cudaMemcpyAsync(d_out, static_cast<const char*>(d_workspace) + L.thr, bytes,
                                cudaMemcpyDeviceToDevice, stream) != cudaSuccess)

@@ -94,7 +94,8 @@ struct ChunkSplit {
 
 struct MArgs {
   const MTensor* tensors;
-  ChunkSplit chunks;
+  ChunkSplit chunks;           // of the merge kernels
+  ChunkSplit hist_chunks;      // of the TIES threshold passes
   const void* const* experts;  // [tensor * K + e]
   uint32_t* thr;               // [tensor * K + e] TIES threshold keys
   TiesSlot* slots;             // [tensor * K + e]
@@ -569,9 +570,26 @@ __global__ void __launch_bounds__(kBlock, 2) dare_kernel(const __grid_constant__
 }
 
 // --------------------------------------------------- TIES threshold selection ---
+template <int DT>
+__device__ __forceinline__ void load_lane(const void* base, int64_t i, Raw16<DT>& v) {
+  load16<DT>(base, i, v);
+}
+template <int DT>
+__device__ __forceinline__ void load_lane(const void* base, int64_t i, Raw8<DT>& v) {
+  load8<DT>(base, i, v);
+}
+
+// A thread's 32 bytes of one array: 16 bf16 or 8 fp32 elements. (16 fp32
+// elements of theta0 and four experts took 147 registers, one CTA per SM.)
+template <int DT>
+using RawLane = std::conditional_t<DT == DT_BF16, Raw16<DT>, Raw8<DT>>;
+template <int DT>
+constexpr int kLaneElems = DT == DT_BF16 ? 16 : 8;
+
 // Elements sampled per slot, as 16-element groups spread evenly over the
-// tensor; a tensor of at most this many elements is read whole.
-constexpr int kSampleElems = 1 << 16;
+// tensor; a tensor of at most kWholeElems elements is read whole.
+constexpr int kSampleElems = 1 << 15;
+constexpr int kWholeElems = 1 << 16;
 
 // The interval [lo, lo + width) as the slot's next one: the smallest shift
 // whose 2046 bins cover it from a multiple of 2^shift.
@@ -634,9 +652,11 @@ __device__ __forceinline__ void select_from_top(const Count* hist, int nb, long 
 }
 
 // The first interval of each slot, one CTA per slot: two order statistics of
-// the sample, eight standard deviations of the sampled rank to either side of
+// the sample, six standard deviations of the sampled rank to either side of
 // r's share, each by a radix select of three digits (11, 11 and 10 bits). The
-// three readings of the sample (2 x 128 KB for bf16) come from L2 after the first.
+// sample's keys stay in registers, 32 per thread (65,536 keys read anew for each digit
+// took 50 us for an fp32 slot, these take 33); a tensor that is read whole comes from L2
+// after the first digit.
 constexpr int kSampleThreads = 1024;
 
 template <int DT>
@@ -654,58 +674,89 @@ __global__ void __launch_bounds__(kSampleThreads) ties_sample_kernel(const __gri
     }
     return;
   }
-  const bool all = n <= kSampleElems, vec = (T.flags & TF_VEC) != 0u;
-  const int groups = all ? (int)((n + 15) / 16) : kSampleElems / 16;
+  const bool all = n <= kWholeElems, vec = (T.flags & TF_VEC) != 0u;
   const int64_t seen = all ? n : kSampleElems;
   // ranks in the sample, counted from the largest key: the upper end of the
   // interval and the lower one
   long long rank[2] = {r, r};
   if (!all) {
     const double p = (double)r / (double)n, at = p * (double)seen;
-    const double d = 8.0 * sqrt(at * (1.0 - p)) + 32.0;
+    const double d = 6.0 * sqrt(at * (1.0 - p)) + 16.0;
     rank[0] = (long long)ceil(at - d);
     rank[1] = (long long)floor(at + d);
   }
   const bool open_top = rank[0] < 1, open_bottom = rank[1] > seen;
   if (open_top) rank[0] = 1;
   if (open_bottom) rank[1] = seen;
+  constexpr int kMine = kSampleElems / kSampleThreads, kLane = kLaneElems<DT>;
   uint32_t prefix[2] = {0u, 0u};
   const int shifts[3] = {21, 10, 0}, widths[3] = {11, 11, 10};
+  // each(count) calls count for every key of the sample
+  auto select = [&](auto&& each) {
 #pragma unroll 1
-  for (int pass = 0; pass < 3; ++pass) {
-    const int shift = shifts[pass], nb = 1 << widths[pass];
-    const uint32_t decided = pass == 0 ? 0u : ~0u << shifts[pass - 1];
-    const bool same = prefix[0] == prefix[1];
-    for (int b = threadIdx.x; b < 2 * kHistBins; b += kSampleThreads) (&h[0][0])[b] = 0u;
-    __syncthreads();
-    auto count = [&](uint32_t key) {
-      const uint32_t digit = (key >> shift) & (uint32_t)(nb - 1);
-      if ((key & decided) == prefix[0]) atomicAdd(&h[0][digit], 1u);
-      if (!same && (key & decided) == prefix[1]) atomicAdd(&h[1][digit], 1u);
-    };
-    for (int g = threadIdx.x; g < groups; g += kSampleThreads) {
-      const int64_t i = 16 * (all ? (int64_t)g : (int64_t)g * (n / 16) / groups);
-      if (vec && i + 16 <= n) {
-        Raw16<DT> t0, y;
-        load16<DT>(T.theta0, i, t0);
-        load16<DT>(x, i, y);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const float2 d = sub2_rn(y.pair(q), t0.pair(q));
-          count(abs_key(d.x));
-          count(abs_key(d.y));
-        }
-      } else {
-        for (int64_t k = i; k < n && k < i + 16; ++k) count(abs_key(__fsub_rn(load1<DT>(x, k), load1<DT>(T.theta0, k))));
+    for (int pass = 0; pass < 3; ++pass) {
+      const int shift = shifts[pass], nb = 1 << widths[pass];
+      const uint32_t decided = pass == 0 ? 0u : ~0u << shifts[pass - 1];
+      const bool same = prefix[0] == prefix[1];
+      for (int b = threadIdx.x; b < 2 * kHistBins; b += kSampleThreads) (&h[0][0])[b] = 0u;
+      __syncthreads();
+      each([&](uint32_t key) {
+        const uint32_t digit = (key >> shift) & (uint32_t)(nb - 1);
+        if ((key & decided) == prefix[0]) atomicAdd(&h[0][digit], 1u);
+        if (!same && (key & decided) == prefix[1]) atomicAdd(&h[1][digit], 1u);
+      });
+      __syncthreads();
+      for (int q = 0; q < 2; ++q) {
+        select_from_top(h[same ? 0 : q], nb, rank[q], sh);
+        prefix[q] |= (uint32_t)sh.digit << shift;
+        rank[q] -= sh.above;
+        __syncthreads();
       }
     }
-    __syncthreads();
-    for (int q = 0; q < 2; ++q) {
-      select_from_top(h[same ? 0 : q], nb, rank[q], sh);
-      prefix[q] |= (uint32_t)sh.digit << shift;
-      rank[q] -= sh.above;
-      __syncthreads();
+  };
+  // the keys of the lane of kLane elements at i
+  auto lane_keys = [&](int64_t i, uint32_t* keys) {
+    RawLane<DT> t0, y;
+    load_lane<DT>(T.theta0, i, t0);
+    load_lane<DT>(x, i, y);
+#pragma unroll
+    for (int q = 0; q < kLane / 2; ++q) {
+      const float2 d = sub2_rn(y.pair(q), t0.pair(q));
+      keys[2 * q] = abs_key(d.x);
+      keys[2 * q + 1] = abs_key(d.y);
     }
+  };
+  auto key_at = [&](int64_t i) { return abs_key(__fsub_rn(load1<DT>(x, i), load1<DT>(T.theta0, i))); };
+  if (all) {
+    select([&](auto&& count) {
+      for (int i = kLane * (int)threadIdx.x; i < (int)n; i += kLane * kSampleThreads) {
+        if (vec && i + kLane <= (int)n) {
+          uint32_t keys[kLane];
+          lane_keys(i, keys);
+#pragma unroll
+          for (int k = 0; k < kLane; ++k) count(keys[k]);
+        } else {
+          for (int k = i; k < (int)n && k < i + kLane; ++k) count(key_at(k));
+        }
+      }
+    });
+  } else {
+    uint32_t mine[kMine];
+#pragma unroll
+    for (int l = 0; l < kMine / kLane; ++l) {
+      const int at = kLane * ((int)threadIdx.x + l * kSampleThreads);  // place in the sample
+      const int64_t i = 16 * ((int64_t)(at / 16) * (n / 16) / (kSampleElems / 16)) + at % 16;
+      if (vec) {
+        lane_keys(i, mine + l * kLane);
+      } else {
+#pragma unroll
+        for (int k = 0; k < kLane; ++k) mine[l * kLane + k] = key_at(i + k);
+      }
+    }
+    select([&](auto&& count) {
+#pragma unroll
+      for (int k = 0; k < kMine; ++k) count(mine[k]);
+    });
   }
   if (threadIdx.x == 0) {
     TiesSlot S;
@@ -752,33 +803,20 @@ constexpr uint32_t kOffMost = 256u;  // sums of 2^14 chunks stay below 2^22
 constexpr int64_t kOffChunks = 1 << 14;
 constexpr int kOffList = 512;
 
-template <int DT>
-__device__ __forceinline__ void load_lane(const void* base, int64_t i, Raw16<DT>& v) {
-  load16<DT>(base, i, v);
-}
-template <int DT>
-__device__ __forceinline__ void load_lane(const void* base, int64_t i, Raw8<DT>& v) {
-  load8<DT>(base, i, v);
-}
-
-// A thread's 32 bytes of one array: 16 bf16 or 8 fp32 elements. (16 fp32
-// elements of theta0 and four experts took 147 registers, one CTA per SM.)
-template <int DT>
-using RawLane = std::conditional_t<DT == DT_BF16, Raw16<DT>, Raw8<DT>>;
+constexpr int kHistCtas(int dtype) { return dtype == DT_BF16 ? 4 : 3; }  // per SM
 
 template <int DT>
-__global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 3) ties_hist_kernel(const __grid_constant__ MArgs m) {
-  constexpr int kLane = DT == DT_BF16 ? 16 : 8;
+__global__ void __launch_bounds__(kBlock, kHistCtas(DT)) ties_hist_kernel(const __grid_constant__ MArgs m) {
   __shared__ uint32_t h[kHistExperts * kHistBins];
   __shared__ uint16_t list[kOffList];  // (group << 2) | expert of the batch
   __shared__ int n_list;
   if (*m.n_done == (uint32_t)m.n_slots) return;
   const int nbat = (m.K + kHistExperts - 1) / kHistExperts;
-  const int64_t items = m.chunks.n * nbat;
+  const int64_t items = m.hist_chunks.n * nbat;
   for (int64_t w = blockIdx.x; w < items; w += gridDim.x) {
     const int e0 = (int)(w % nbat) * kHistExperts;
     const int ne = m.K - e0 < kHistExperts ? m.K - e0 : kHistExperts;
-    const Chunk ch = chunk_of(m, m.chunks, w / nbat);
+    const Chunk ch = chunk_of(m, m.hist_chunks, w / nbat);
     const MTensor& T = m.tensors[ch.tensor];
     const int slot0 = ch.tensor * m.K + e0;
     uint32_t lo[kHistExperts];
@@ -810,8 +848,8 @@ __global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 3) ties_hist_kerne
     };
     const bool vec = (T.flags & TF_VEC) != 0u;
     const void* t0p = T.theta0;
-    for (int64_t i = ch.begin + kLane * (int64_t)threadIdx.x; i < ch.end; i += kLane * (int64_t)kBlock) {
-      if (vec && i + kLane <= ch.end) {
+    for (int64_t i = ch.begin + kLaneElems<DT> * (int64_t)threadIdx.x; i < ch.end; i += kLaneElems<DT> * (int64_t)kBlock) {
+      if (vec && i + kLaneElems<DT> <= ch.end) {
         RawLane<DT> t0, x[kHistExperts];
         load_lane<DT>(t0p, i, t0);
 #pragma unroll
@@ -822,7 +860,7 @@ __global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 3) ties_hist_kerne
           if (xp[b]) {
             uint32_t bits = 0u;
 #pragma unroll
-            for (int q = 0; q < kLane / 2; ++q) {
+            for (int q = 0; q < kLaneElems<DT> / 2; ++q) {
               const float2 d = sub2_rn(x[b].pair(q), t0.pair(q));
               const uint32_t k0 = abs_key(d.x), k1 = abs_key(d.y);
               bits |= k0 | k1;
@@ -836,7 +874,7 @@ __global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 3) ties_hist_kerne
           }
         }
       } else {
-        const int64_t e_end = (i + kLane < ch.end) ? i + kLane : ch.end;
+        const int64_t e_end = (i + kLaneElems<DT> < ch.end) ? i + kLaneElems<DT> : ch.end;
         for (int64_t k = i; k < e_end; ++k) {
           const float t0 = load1<DT>(t0p, k);
 #pragma unroll
@@ -876,7 +914,7 @@ __global__ void __launch_bounds__(kBlock, DT == DT_BF16 ? 4 : 3) ties_hist_kerne
     }
     // the ne histograms are consecutive slots' bins in the global array
     unsigned long long* gh = m.hist + (size_t)slot0 * kHistBins;
-    const uint32_t most = T.numel <= kOffChunks * m.chunks.elems ? kOffMost : 1u;
+    const uint32_t most = T.numel <= kOffChunks * m.hist_chunks.elems ? kOffMost : 1u;
     for (int b = threadIdx.x; b < ne * kHistBins; b += kBlock) {
       const uint32_t c = h[b];
       if (c) {
@@ -967,7 +1005,7 @@ MLayout merge_layout(int32_t n, int K, bool ties) {
   size_t off = 0;
   const size_t slots = (size_t)n * (size_t)K;
   L.tensors = off; off = align_m(off + sizeof(MTensor) * (size_t)n);
-  L.first = off;   off = align_m(off + sizeof(int32_t) * ((size_t)n + 1));
+  L.first = off;   off = align_m(off + sizeof(int32_t) * ((size_t)n + 1) * (ties ? 2 : 1));  // chunks, hist_chunks
   L.experts = off; off = align_m(off + sizeof(void*) * slots);
   L.thr = off;     off = align_m(off + sizeof(uint32_t) * slots);
   L.slots = off;   off = align_m(off + sizeof(TiesSlot) * slots);
@@ -1044,6 +1082,23 @@ smat_status merge_check(const smat_merge_tensor* t, int32_t n, const smat_merge_
   return SMAT_OK;
 }
 
+// Chunk of the threshold passes: their CTAs clear and flush up to 32 KB of bins per
+// item, so items are as long as they can be (2^16 elements) while they fill whole
+// rounds of the resident CTAs, of which the tensors' short last chunks take at most
+// half. Two experts of 1.8e7 fp32 elements: 52 and 48 us for the two passes that
+// count in the merge kernels' chunks of 2^13, 44 and 41 in one round.
+int64_t hist_chunk_for(const MPlan& p, int32_t n, int K, int sms) {
+  const int64_t nbat = (K + kHistExperts - 1) / kHistExperts;
+  const int64_t resident = std::max<int64_t>(kHistCtas(p.dtype) * (int64_t)sms / nbat, 1);
+  int64_t chunk = kMergeChunkMax + 1;
+  for (int64_t rounds = 1; chunk > kMergeChunkMax; ++rounds) {
+    const int64_t items = resident * rounds - n;
+    if (2 * items >= resident * rounds) chunk = (p.total + items - 1) / items;
+  }
+  const int64_t step = 16 * (int64_t)kBlock;
+  return std::min(std::max((chunk + step - 1) / step * step, kMergeChunkMin), kMergeChunkMax);
+}
+
 template <int DT, int BATCH, bool FULL>
 cudaError_t ties_merge_run(const MArgs& m, cudaStream_t s) {
   ties_merge_kernel<DT, BATCH, FULL><<<(int)m.chunks.n, kBlock, 0, s>>>(m);
@@ -1053,17 +1108,18 @@ cudaError_t ties_merge_run(const MArgs& m, cudaStream_t s) {
 template <int DT>
 cudaError_t merge_launch(MArgs m, int64_t slots, int64_t largest, int rounds, int sms, cudaStream_t s) {
   if (m.method == SMAT_MERGE_TIES) {
-    const int64_t items = m.chunks.n * ((m.K + kHistExperts - 1) / kHistExperts);  // one CTA each
+    const int64_t items = m.hist_chunks.n * ((m.K + kHistExperts - 1) / kHistExperts);  // one CTA each
     m.n_slots = (int32_t)slots;
     ties_sample_kernel<DT><<<(int)slots, kSampleThreads, 0, s>>>(m);
     // no pass where every tensor is small enough for the sample to decide
-    for (int p = 0; p < (largest > kSampleElems ? kPasses : 0); ++p) {
+    for (int p = 0; p < (largest > kWholeElems ? kPasses : 0); ++p) {
       ties_hist_kernel<DT><<<(int)std::min(items, int64_t(INT32_MAX)), kBlock, 0, s>>>(m);
       ties_select_kernel<DT><<<(int)slots, kBlock, 0, s>>>(m);
     }
     if constexpr (DT == DT_BF16)
       if (m.K % 8 == 0) return ties_merge_run<DT, 8, true>(m, s);
     if (m.K % 4 == 0) return ties_merge_run<DT, 4, true>(m, s);
+    if (m.K == 2) return ties_merge_run<DT, 2, true>(m, s);
     return ties_merge_run<DT, 4, false>(m, s);
   }
   // one CTA per chunk, started by the hardware as others end (8 experts of 1e8 bf16
@@ -1108,12 +1164,16 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
     if (!ok) return mfail(SMAT_ERR_INVALID_ARG, "tensor %d: a pointer is not accessible from the GPU", k);
   }
   if (n_tensors == 0 || plan.n_chunks == 0) return SMAT_OK;
+  int dev = 0, sms = 1;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return mfail(SMAT_ERR_CUDA, "device query failed");
 
   // tables (host), then one upload each
   const float keep = 1.0f - cfg->p_drop;
   const uint64_t T = (uint64_t)std::floor((double)keep * 4294967296.0);
   std::vector<MTensor> ht((size_t)n_tensors);
-  std::vector<int32_t> first((size_t)n_tensors + 1, 0);
+  const int64_t hist_chunk = hist_chunk_for(plan, n_tensors, K, sms);
+  std::vector<int32_t> first(((size_t)n_tensors + 1) * (ties ? 2 : 1), 0);
   std::vector<const void*> hx((size_t)n_tensors * (size_t)K, nullptr);
   std::vector<int64_t> hrank((size_t)n_tensors * (size_t)K, 0);
   for (int32_t k = 0; k < n_tensors; ++k) {
@@ -1143,12 +1203,17 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
       for (int e = 0; e < K; ++e) hrank[(size_t)k * K + e] = r;
     }
     first[(size_t)k + 1] = first[(size_t)k] + (int32_t)((d.numel + plan.chunk - 1) / plan.chunk);
+    if (ties) {
+      int32_t* f = first.data() + n_tensors + 1 + k;
+      f[1] = f[0] + (int32_t)((d.numel + hist_chunk - 1) / hist_chunk);
+    }
   }
   char* ws = static_cast<char*>(d_workspace);
   MArgs m;
   std::memset(&m, 0, sizeof(m));
   m.tensors = reinterpret_cast<const MTensor*>(ws + L.tensors);
   m.chunks = {reinterpret_cast<const int32_t*>(ws + L.first), plan.chunk, plan.n_chunks};
+  if (ties) m.hist_chunks = {m.chunks.first + n_tensors + 1, hist_chunk, first.back()};
   m.experts = reinterpret_cast<const void* const*>(ws + L.experts);
   m.thr = reinterpret_cast<uint32_t*>(ws + L.thr);
   m.slots = reinterpret_cast<TiesSlot*>(ws + L.slots);
@@ -1168,9 +1233,6 @@ extern "C" smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_te
   if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.first, first.data(), sizeof(int32_t) * first.size(), cudaMemcpyHostToDevice, stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(ws + L.experts, hx.data(), sizeof(void*) * slots, cudaMemcpyHostToDevice, stream);
   if (e != cudaSuccess) return mfail(SMAT_ERR_CUDA, "merge table upload failed");
-  int dev = 0, sms = 1;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return mfail(SMAT_ERR_CUDA, "device query failed");
   const int rounds = cfg->philox_rounds == 7 ? 7 : 10;
   if (ties) {
     e = cudaMemsetAsync(ws + L.n_done, 0, sizeof(uint32_t), stream);

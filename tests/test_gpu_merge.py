@@ -191,8 +191,8 @@ def test_merge_special_values(method, dtype):
                                    "sample_nan", "sample_half_nan", "half_nan", "all_nan_but_sample"])
 @pytest.mark.parametrize("retention", [1e-4, 0.25, 0.5, 1.0])
 def test_merge_ties_threshold_selection(dtype, shape, retention):
-    """Thresholds of tensors larger than the selection's sample (65,536
-    elements, in 16-element groups at 16 floor(g (n / 16) / 4096)) equal the
+    """Thresholds of tensors larger than the selection's sample (32,768
+    elements, in 16-element groups at 16 floor(g (n / 16) / 2048)) equal the
     oracle's, also where the sample shows other magnitudes than the rest (its
     interval misses, and the next passes start from the whole range), where
     most keys are equal, with infinities, and with NaN in all or half of the
@@ -202,7 +202,7 @@ def test_merge_ties_threshold_selection(dtype, shape, retention):
     t0 = torch.randn(n, generator=g) * 0.02
     d = torch.randn(K, n, generator=g) * 1e-3
     seen = torch.zeros(n, dtype=torch.bool)
-    first = 16 * (torch.arange(4096) * (n // 16) // 4096)
+    first = 16 * (torch.arange(2048) * (n // 16) // 2048)
     seen[(first[:, None] + torch.arange(16)).reshape(-1)] = True
     if shape == "mostly_zero":
         d[torch.rand(K, n, generator=g) < 0.8] = 0.0
@@ -304,6 +304,21 @@ def test_merge_refuses_mismatched_tensors():
     S.merge(views, exs, views, S.SMAT_MERGE_TA, gamma=0.5)
     for a, b in zip(outs, views):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dtype", [O.F32, O.BF16])
+@pytest.mark.parametrize("K", [2, 5])
+def test_merge_ties_long_threshold_items(dtype, K):
+    """The threshold passes' items are as long as fill whole rounds of the CTAs
+    (here no power of two), the merge pass's chunks are not: the thresholds and
+    the merge equal the oracle's on several tensors, one of them unaligned."""
+    t0s, exs = _experts([3_000_017, 40_000, 2_500_003 + 1], K, dtype, seed=90 + K)
+    t0s[2], exs[2] = t0s[2][1:], [x[1:] for x in exs[2]]
+    outs = [torch.empty_like(t) for t in t0s]
+    kw = dict(gamma=0.4, retention=0.2)
+    thr = S.merge(t0s, exs, outs, S.SMAT_MERGE_TIES, return_thresholds=True, **kw)
+    torch.cuda.synchronize()
+    _check(t0s, exs, outs, dtype, S.SMAT_MERGE_TIES, kw, thr=thr)
 
 
 @pytest.mark.parametrize("method", list(METHODS))

@@ -150,17 +150,17 @@ cudaError_t launch_direct(const KArgs& a, int dtype, int noise, bool per_elem_al
                           : SMAT_BY_FAMILY(launch_direct_f32)(a, noise, per_elem_alpha, rounds, s);
 }
 
-cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise, bool per_elem_alpha,
+cudaError_t launch_stats_simulate(const KArgs& a, int sms, int dtype, int noise, bool per_elem_alpha,
                                   int rounds, bool inplace, cudaStream_t s) {
   if (noise == NOISE_LAPLACE)
-    return dtype == DT_BF16 ? SMAT_BY_FAMILY(launch_laplace_bf16)(a, grid, true, per_elem_alpha, inplace, s)
-                            : SMAT_BY_FAMILY(launch_laplace_f32)(a, grid, true, per_elem_alpha, inplace, s);
+    return dtype == DT_BF16 ? SMAT_BY_FAMILY(launch_laplace_bf16)(a, sms, true, per_elem_alpha, inplace, s)
+                            : SMAT_BY_FAMILY(launch_laplace_f32)(a, sms, true, per_elem_alpha, inplace, s);
   if (inplace)
     return dtype == DT_BF16
-               ? SMAT_BY_FAMILY(launch_stats_simulate_inplace_bf16)(a, grid, noise, per_elem_alpha, rounds, s)
-               : SMAT_BY_FAMILY(launch_stats_simulate_inplace_f32)(a, grid, noise, per_elem_alpha, rounds, s);
-  return dtype == DT_BF16 ? SMAT_BY_FAMILY(launch_stats_simulate_bf16)(a, grid, noise, per_elem_alpha, rounds, s)
-                          : SMAT_BY_FAMILY(launch_stats_simulate_f32)(a, grid, noise, per_elem_alpha, rounds, s);
+               ? SMAT_BY_FAMILY(launch_stats_simulate_inplace_bf16)(a, sms, noise, per_elem_alpha, rounds, s)
+               : SMAT_BY_FAMILY(launch_stats_simulate_inplace_f32)(a, sms, noise, per_elem_alpha, rounds, s);
+  return dtype == DT_BF16 ? SMAT_BY_FAMILY(launch_stats_simulate_bf16)(a, sms, noise, per_elem_alpha, rounds, s)
+                          : SMAT_BY_FAMILY(launch_stats_simulate_f32)(a, sms, noise, per_elem_alpha, rounds, s);
 }
 
 int streaming_ctas_per_sm(int dtype, int noise, bool pe, int rounds) {

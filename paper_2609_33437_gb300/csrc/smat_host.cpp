@@ -615,9 +615,10 @@ smat_status smat_simulate_multi(smat_ctx* c, uint32_t step, smat_stream_t stream
       a.items = c->d_items + c->item_begin[dt];
       a.n_items = c->item_count[dt];
       a.work_counter = c->d_sync + dt;
-      const int grid = c->item_count[dt];  // one CTA per item
+      a.chunk_begin = c->range_begin[dt];
+      a.chunk_end = c->range_end[dt];
       Timed t(c, 2, stream);
-      const cudaError_t e = launch_stats_simulate(a, grid, dt, c->cfg.noise, c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT,
+      const cudaError_t e = launch_stats_simulate(a, c->sm_count, dt, c->cfg.noise, c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT,
                                                   c->rounds, c->any_inplace, stream);
       t.done();
       if (e != cudaSuccess) return cuda_fail(e, "fused statistics + forward launch");
@@ -921,7 +922,7 @@ smat_status smat_debug_fused(smat_ctx* c, uint32_t step, const int32_t* d_items,
   a.items = d_items;
   a.n_items = n_items;
   a.work_counter = c->d_sync + SMAT_BF16;
-  e = launch_stats_simulate_bf16(a, n_items, c->cfg.noise,
+  e = launch_stats_simulate_bf16(a, c->sm_count, c->cfg.noise,
                                  c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT, c->rounds, stream);
   if (e != cudaSuccess) return cuda_fail(e, "fused launch");
   c->scalars_step = -1;  // sigma_t of this call may be incomplete

@@ -9,11 +9,11 @@
 
 namespace smat {
 
-cudaError_t SMAT_FAMILY(launch_stats_simulate_inplace_bf16)(const KArgs& a, int grid, int noise,
+cudaError_t SMAT_FAMILY(launch_stats_simulate_inplace_bf16)(const KArgs& a, int sms, int noise,
                                                             bool per_elem_alpha, int rounds, cudaStream_t s) {
   if (a.n_items <= 0) return cudaSuccess;
-  return (rounds & 0xFF) == 7 ? fused_run<7 | kFamily, DT_BF16, true>(a, grid, noise, per_elem_alpha, s)
-                              : fused_run<10 | kFamily, DT_BF16, true>(a, grid, noise, per_elem_alpha, s);
+  return (rounds & 0xFF) == 7 ? fused_run<7 | kFamily, DT_BF16, true>(a, sms, noise, per_elem_alpha, s)
+                              : fused_run<10 | kFamily, DT_BF16, true>(a, sms, noise, per_elem_alpha, s);
 }
 
 }  // namespace smat

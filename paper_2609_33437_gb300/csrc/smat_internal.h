@@ -157,7 +157,9 @@ cudaError_t launch_simulate(const KArgs& a, int grid, int dtype, int noise, bool
 // The forward of a list without statistics, scalars included, one CTA per chunk.
 cudaError_t launch_direct(const KArgs& a, int dtype, int noise, bool per_elem_alpha, int rounds, bool inplace,
                           cudaStream_t s);
-cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise, bool per_elem_alpha,
+// The work-list launch of a.n_items items over the chunks a.chunk_begin .. a.chunk_end;
+// sms: the device's SM count.
+cudaError_t launch_stats_simulate(const KArgs& a, int sms, int dtype, int noise, bool per_elem_alpha,
                                   int rounds, bool inplace, cudaStream_t s);
 // The forward launchers below exist twice: as declared (the packed draw
 // layout) and with the suffix _d16 (the 16-bit draw option). Each forward
@@ -171,14 +173,14 @@ cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise
                                         cudaStream_t s);                                                      \
   int simulate_ctas_per_sm_f32##sfx(int noise, bool per_elem_alpha, int rounds);                              \
   int simulate_ctas_per_sm_bf16##sfx(int noise, bool per_elem_alpha, int rounds);                             \
-  cudaError_t launch_stats_simulate_f32##sfx(const KArgs& a, int grid, int noise, bool per_elem_alpha,        \
+  cudaError_t launch_stats_simulate_f32##sfx(const KArgs& a, int sms, int noise, bool per_elem_alpha,        \
                                              int rounds, cudaStream_t s);                                     \
-  cudaError_t launch_stats_simulate_bf16##sfx(const KArgs& a, int grid, int noise, bool per_elem_alpha,       \
+  cudaError_t launch_stats_simulate_bf16##sfx(const KArgs& a, int sms, int noise, bool per_elem_alpha,       \
                                               int rounds, cudaStream_t s);                                    \
   /* Resident CTAs per SM of launch_stats_simulate_bf16 (uniform or Gaussian). */                             \
   int fused_wide_ctas_per_sm##sfx(int noise, bool per_elem_alpha, int rounds);                                \
-  /* Laplace noise (10 rounds; smat_laplace_*.cu): the work-list launch when `fused`, else the grid-stride    \
-     one; in-place instantiations when `inplace`. */                                                          \
+  /* Laplace noise (10 rounds; smat_laplace_*.cu): the work-list launch when `fused` (grid: the SM count),   \
+     else the grid-stride one; in-place instantiations when `inplace`. */                                     \
   cudaError_t launch_laplace_f32##sfx(const KArgs& a, int grid, bool fused, bool per_elem_alpha, bool inplace, \
                                       cudaStream_t s);                                                        \
   cudaError_t launch_laplace_bf16##sfx(const KArgs& a, int grid, bool fused, bool per_elem_alpha,             \
@@ -186,9 +188,9 @@ cudaError_t launch_stats_simulate(const KArgs& a, int grid, int dtype, int noise
   /* Resident CTAs per SM of launch_laplace_bf16's work-list launch without in-place tensors. */               \
   int laplace_ctas_per_sm_bf16##sfx(bool per_elem_alpha);                                                      \
   /* the same launches for lists with in-place tensors (smat_inplace_*.cu) */                                \
-  cudaError_t launch_stats_simulate_inplace_f32##sfx(const KArgs& a, int grid, int noise, bool per_elem_alpha, \
+  cudaError_t launch_stats_simulate_inplace_f32##sfx(const KArgs& a, int sms, int noise, bool per_elem_alpha, \
                                                      int rounds, cudaStream_t s);                             \
-  cudaError_t launch_stats_simulate_inplace_bf16##sfx(const KArgs& a, int grid, int noise,                    \
+  cudaError_t launch_stats_simulate_inplace_bf16##sfx(const KArgs& a, int sms, int noise,                    \
                                                       bool per_elem_alpha, int rounds, cudaStream_t s);       \
   cudaError_t launch_simulate_inplace_f32##sfx(const KArgs& a, int grid, int noise, bool per_elem_alpha,      \
                                                int rounds, cudaStream_t s);                                   \

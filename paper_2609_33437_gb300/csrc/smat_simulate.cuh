@@ -272,6 +272,12 @@ __device__ __forceinline__ void sim_chunk_noise(const KArgs& a, const TView& v, 
 // flag. (Persistent CTAs that took items until the list ended: 7B list 11.04 ms,
 // this 10.88 ms.)
 //
+// WALK: CTAs that go on to further items, as many as there are chunks, for lists
+// whose items all run at once or nearly (fused_walks). With a CTA per item the
+// tickets, and so the forward items, then fall unevenly over the SMs, while a CTA
+// that walks takes its forward item where its statistics item ran: 2e6 bf16
+// elements, Gaussian noise, 32.8 us with a CTA per item and 26.8 walking; 1e6 28 and 24.
+//
 // Progress: a CTA takes its ticket when it runs, and a statistics item never
 // waits, so every item a waiting forward item depends on is already held by a
 // running CTA. The wait is bounded all the same: after kWaitLimit polls (about one
@@ -304,7 +310,7 @@ __device__ __forceinline__ void forward_chunk(const KArgs& a, const TView& v, co
 template <int DT, int NOISE, bool PE, bool IP>
 constexpr int kFusedCtas = DT != DT_BF16 ? 2 : IP ? (PE ? 2 : 3) : (PE || NOISE == NOISE_LAPLACE ? 3 : 4);
 
-template <int R, int DT, int NOISE, bool PE, bool IP>
+template <int R, int DT, int NOISE, bool PE, bool IP, bool WALK>
 __global__ void __launch_bounds__(kBlock, kFusedCtas<DT, NOISE, PE, IP>)
     stats_simulate_kernel(const __grid_constant__ KArgs a) {
   __shared__ double sh_s[kBlock / 32];
@@ -312,73 +318,76 @@ __global__ void __launch_bounds__(kBlock, kFusedCtas<DT, NOISE, PE, IP>)
   __shared__ int s_item;
   __shared__ int s_flag;
   __shared__ ChunkQueue s_cq;
-  if (threadIdx.x == 0) {
-    s_item = atomicAdd(a.work_counter, 1);
-    s_cq.n_tie = 0;
-    s_cq.n_tail = 0;
-  }
-  __syncthreads();
-  const int it = s_item;
-  if (it >= a.n_items) return;  // same value in every thread
-  const uint32_t code = (uint32_t)a.items[it];
-  const int64_t ci = (int64_t)(code & ~kItemForward);
-  const Chunk ch = a.chunks[ci];
-  const DevTensor& T = a.tensors[ch.tensor];
-  if (!(code & kItemForward)) {
-    double ds, dq;
-    chunk_delta_sums<DT>(T, ch, sh_s, sh_q, ds, dq);
+  do {
     if (threadIdx.x == 0) {
-      a.partials[ci].sum = ds;
-      a.partials[ci].sumsq = dq;
-      __threadfence();
-      s_flag = (atomicAdd(a.tensor_done + ch.tensor, 1) == T.n_chunks - 1) ? 1 : 0;
+      s_item = atomicAdd(a.work_counter, 1);
+      s_cq.n_tie = 0;
+      s_cq.n_tail = 0;
     }
     __syncthreads();
-    if (s_flag) {
-      // last statistics chunk of this tensor: sum the partials in chunk order
-      __threadfence();
-      double s = 0.0, q = 0.0;
-      for (int k = threadIdx.x; k < T.n_chunks; k += kBlock) {
-        s += __ldcg(&a.partials[T.chunk_first + k].sum);
-        q += __ldcg(&a.partials[T.chunk_first + k].sumsq);
-      }
-      s = warp_sum(s);
-      q = warp_sum(q);
-      if ((threadIdx.x & 31) == 0) {
-        sh_s[threadIdx.x >> 5] = s;
-        sh_q[threadIdx.x >> 5] = q;
-      }
-      __syncthreads();
+    const int it = s_item;
+    if (it >= a.n_items) return;  // same value in every thread
+    const uint32_t code = (uint32_t)a.items[it];
+    const int64_t ci = (int64_t)(code & ~kItemForward);
+    const Chunk ch = a.chunks[ci];
+    const DevTensor& T = a.tensors[ch.tensor];
+    if (!(code & kItemForward)) {
+      double ds, dq;
+      chunk_delta_sums<DT>(T, ch, sh_s, sh_q, ds, dq);
       if (threadIdx.x == 0) {
-        double ts = 0.0, tq = 0.0;
-        for (int w = 0; w < kBlock / 32; ++w) {
-          ts += sh_s[w];
-          tq += sh_q[w];
-        }
-        const float sigma = sigma_from_sums(ts, tq, T.numel, T.sigma_rel);
-        a.scal[ch.tensor].sigma = sigma;
-        a.scal[ch.tensor].noise_scale = noise_scale_of<NOISE>(sigma);
+        a.partials[ci].sum = ds;
+        a.partials[ci].sumsq = dq;
         __threadfence();
-        st_release(a.ready + ch.tensor, a.epoch);
+        s_flag = (atomicAdd(a.tensor_done + ch.tensor, 1) == T.n_chunks - 1) ? 1 : 0;
+      }
+      __syncthreads();
+      if (s_flag) {
+        // last statistics chunk of this tensor: sum the partials in chunk order
+        __threadfence();
+        double s = 0.0, q = 0.0;
+        for (int k = threadIdx.x; k < T.n_chunks; k += kBlock) {
+          s += __ldcg(&a.partials[T.chunk_first + k].sum);
+          q += __ldcg(&a.partials[T.chunk_first + k].sumsq);
+        }
+        s = warp_sum(s);
+        q = warp_sum(q);
+        if ((threadIdx.x & 31) == 0) {
+          sh_s[threadIdx.x >> 5] = s;
+          sh_q[threadIdx.x >> 5] = q;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          double ts = 0.0, tq = 0.0;
+          for (int w = 0; w < kBlock / 32; ++w) {
+            ts += sh_s[w];
+            tq += sh_q[w];
+          }
+          const float sigma = sigma_from_sums(ts, tq, T.numel, T.sigma_rel);
+          a.scal[ch.tensor].sigma = sigma;
+          a.scal[ch.tensor].noise_scale = noise_scale_of<NOISE>(sigma);
+          __threadfence();
+          st_release(a.ready + ch.tensor, a.epoch);
+        }
+      }
+    } else {
+      if (T.flags & TF_SIGMA_REL) {
+        if (threadIdx.x == 0) s_flag = wait_ready(a, ch.tensor) ? 1 : 0;
+        __syncthreads();
+      } else if (threadIdx.x == 0) {
+        s_flag = 1;
+      }
+      __syncthreads();
+      if (s_flag) {
+        DevScalars S;
+        S.alpha = __ldcg(&a.scal[ch.tensor].alpha);
+        S.c = __ldcg(&a.scal[ch.tensor].c);
+        S.sigma = __ldcg(&a.scal[ch.tensor].sigma);
+        S.noise_scale = __ldcg(&a.scal[ch.tensor].noise_scale);
+        forward_chunk<R, DT, NOISE, PE, IP>(a, make_view(T, S), T, ch, s_cq);
       }
     }
-  } else {
-    if (T.flags & TF_SIGMA_REL) {
-      if (threadIdx.x == 0) s_flag = wait_ready(a, ch.tensor) ? 1 : 0;
-      __syncthreads();
-    } else if (threadIdx.x == 0) {
-      s_flag = 1;
-    }
-    __syncthreads();
-    if (s_flag) {
-      DevScalars S;
-      S.alpha = __ldcg(&a.scal[ch.tensor].alpha);
-      S.c = __ldcg(&a.scal[ch.tensor].c);
-      S.sigma = __ldcg(&a.scal[ch.tensor].sigma);
-      S.noise_scale = __ldcg(&a.scal[ch.tensor].noise_scale);
-      forward_chunk<R, DT, NOISE, PE, IP>(a, make_view(T, S), T, ch, s_cq);
-    }
-  }
+    if (WALK) __syncthreads();  // the next item reuses the shared words
+  } while (WALK);
 }
 
 template <int R, int DT, int NOISE, bool PE, bool IP>
@@ -436,14 +445,29 @@ int occupancy_of(Kernel k) {
   return v;
 }
 
+// Whether the CTAs of a work-list launch walk: from 3/8 of a round of the resident
+// CTAs (below it the forward items have SMs of their own: 2e5 elements 5-9% faster with
+// a CTA per item) to 1, 5/4 and 3/2 rounds at two, three and four CTAs per SM (next
+// sizes measured on either side: 0.81 and 1.21, 1.07 and 1.34, 1.41 and 2.0; beyond
+// it the two are within 2%, and from 1e8 elements a CTA per item is 0.5-2% faster).
+inline bool fused_walks(int64_t items, int64_t resident, int ctas) {
+  return 8 * items >= 3 * resident && 4 * items <= (ctas + 2) * resident;
+}
+
 template <int R, int DT, int NOISE, bool PE, bool IP>
 struct FusedVariant {
   static int occ() {
-    static int v = occupancy_of(stats_simulate_kernel<R, DT, NOISE, PE, IP>);
+    static int v = occupancy_of(stats_simulate_kernel<R, DT, NOISE, PE, IP, false>);
     return v;
   }
-  static cudaError_t run(const KArgs& a, int grid, cudaStream_t s) {
-    stats_simulate_kernel<R, DT, NOISE, PE, IP><<<grid, kBlock, 0, s>>>(a);
+  static cudaError_t run(const KArgs& a, int sms, cudaStream_t s) {
+    const int64_t chunks = a.chunk_end - a.chunk_begin;  // 0: a list of the caller's (test hook)
+    const int64_t resident = (int64_t)sms * occ();
+    if (chunks > 0 && fused_walks(a.n_items, resident, occ()))
+      stats_simulate_kernel<R, DT, NOISE, PE, IP, true>
+          <<<(unsigned)(chunks < resident ? chunks : resident), kBlock, 0, s>>>(a);
+    else
+      stats_simulate_kernel<R, DT, NOISE, PE, IP, false><<<a.n_items, kBlock, 0, s>>>(a);
     return cudaGetLastError();
   }
 };
@@ -462,10 +486,10 @@ cudaError_t direct_run(const KArgs& a, int noise, bool pe, cudaStream_t s) {
 }
 
 template <int R, int DT, bool IP>
-cudaError_t fused_run(const KArgs& a, int grid, int noise, bool pe, cudaStream_t s) {
+cudaError_t fused_run(const KArgs& a, int sms, int noise, bool pe, cudaStream_t s) {
   if (noise == NOISE_GAUSSIAN)
-    return pe ? FusedVariant<R, DT, NOISE_GAUSSIAN, true, IP>::run(a, grid, s) : FusedVariant<R, DT, NOISE_GAUSSIAN, false, IP>::run(a, grid, s);
-  return pe ? FusedVariant<R, DT, NOISE_UNIFORM, true, IP>::run(a, grid, s) : FusedVariant<R, DT, NOISE_UNIFORM, false, IP>::run(a, grid, s);
+    return pe ? FusedVariant<R, DT, NOISE_GAUSSIAN, true, IP>::run(a, sms, s) : FusedVariant<R, DT, NOISE_GAUSSIAN, false, IP>::run(a, sms, s);
+  return pe ? FusedVariant<R, DT, NOISE_UNIFORM, true, IP>::run(a, sms, s) : FusedVariant<R, DT, NOISE_UNIFORM, false, IP>::run(a, sms, s);
 }
 
 template <int R, int DT, int NOISE, bool PE, bool IP>

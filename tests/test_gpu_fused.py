@@ -51,6 +51,36 @@ def test_fused_and_unfused_give_identical_outputs(chunk_log2):
     assert a.poll_errors() == 0 and b.poll_errors() == 0
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("noise,alpha_mode", [(S.SMAT_NOISE_GAUSSIAN, S.SMAT_ALPHA_PER_TENSOR),
+                                              (S.SMAT_NOISE_UNIFORM, S.SMAT_ALPHA_PER_ELEMENT),
+                                              (S.SMAT_NOISE_LAPLACE, S.SMAT_ALPHA_GLOBAL)])
+def test_work_list_walked_and_one_cta_per_item_equal(dtype, noise, alpha_mode):
+    """The work list is walked by CTAs that take several items, or has a CTA per
+    item, by its length against the resident CTAs (a round at two, three or four
+    per SM): lists of 0.1 to 2.4 rounds, on both sides of each line, some with
+    a tensor of fixed sigma and in place, equal the separate passes bit for bit."""
+    bits = torch.int16 if dtype == torch.bfloat16 else torch.int32
+    for sizes, inplace in (([100_003], False), ([500_009], False), ([2_000_003, 33], False), ([2_000_003], True),
+                           ([3_000_017], False), ([5_000_011], False), ([9_000_011, 17, 70_001], False)):
+        th = [(torch.randn(n, device="cuda") * 0.02).to(dtype) for n in sizes]
+        t0 = [(t.float() + torch.randn(t.numel(), device="cuda") * 1e-3).to(dtype) for t in th]
+        rel = [0.1 if n != 70_001 else 0.0 for n in sizes]
+        got = []
+        for flags in (0, S.SMAT_FLAG_UNFUSED_STATS):
+            base = [t.clone() for t in t0]
+            sim = base if inplace else [torch.empty_like(t) for t in th]
+            sess = S.SmatSession(th, base, sim, [0.7] * len(sizes), [1e-3] * len(sizes), rel, seed=9, alpha_min=0.2,
+                                 alpha_mode=alpha_mode, noise=noise, flags=flags)
+            sess.simulate_multi(2)
+            torch.cuda.synchronize()
+            assert sess.poll_errors() == 0
+            got.append(sim)
+            sess.close()
+        for a, b in zip(*got):
+            assert torch.equal(a.view(bits), b.view(bits)), sizes
+
+
 @pytest.mark.parametrize("chunk_log2", [0, 18])
 def test_fused_list_matches_oracle_and_reports_no_errors(chunk_log2):
     run_and_check_full(_rel_list(), steps=(0, 1, 5), flags=S.SMAT_FLAG_CHUNK_LOG2(chunk_log2) if chunk_log2 else 0)

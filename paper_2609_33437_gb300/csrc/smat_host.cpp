@@ -330,6 +330,10 @@ struct Timed {
   }
 };
 
+// Units per SM from which a CTA per unit of the gradient map beats the resident CTAs that
+// share them: with fewer, the launch of a second and third CTA costs more than an uneven end.
+constexpr int64_t kUnitsPerSm = 7;
+
 // Gradient-map units of at most `most` elements (a power of two).
 void set_grad_unit(const smat_ctx* c, KArgs& a, int64_t most) {
   a.grad_unit = std::min(c->chunk_elems, most);
@@ -696,17 +700,20 @@ smat_status smat_grad_map_multi(smat_ctx* c, uint32_t step, const void* const* g
   a.chunk_begin = 0;
   a.chunk_end = (int64_t)c->h_chunks.size();
   const bool pe = c->cfg.alpha_mode == SMAT_ALPHA_PER_ELEMENT;
-  // One CTA per unit. fp32 gradients and per-element alpha take units of 2^15; the
-  // other bf16 maps, whose threads keep four groups in flight, lose on short units:
-  // they take 2^17, or where the list's chunks are smaller walk them in grid-stride
-  // order (1e8 elements: 75.5 us against 78.2 with a CTA per 2^16; 3.5e9 in chunks of
-  // 2^18: 2330 us against 2163 with a CTA per 2^17; fp32 accumulation on 4.9e8: 921
-  // us grid-stride, 847 per 2^17, 829 per 2^15).
+  // One CTA per unit from kUnitsPerSm units per SM; fewer are walked in grid-stride
+  // order (fp32 gradients: 7e6 elements 12.4 us walked and 14.4 with a CTA per unit,
+  // 2.5e7 31 and 36, 3e7 43 and 45, 3.5e7 50.7 and 49.9, 1e8 134 and 123). fp32
+  // gradients and per-element alpha take units of 2^15; the other bf16 maps, whose
+  // threads keep four groups in flight, lose on short units: they take 2^17, or where
+  // the list's chunks are smaller walk them (1e8 elements: 75.5 us against 78.2 with a
+  // CTA per 2^16; 3.5e9 in chunks of 2^18: 2330 us against 2163 with a CTA per 2^17;
+  // fp32 accumulation on 4.9e8: 921 us walked, 847 per 2^17, 829 per 2^15).
   const bool small = gdtype == SMAT_F32 || pe;
   if (small) set_grad_unit(c, a, kSmallGradUnitElems);
   const int64_t units = a.chunk_end * (int64_t)a.grad_units;
   const int64_t resident = (int64_t)c->sm_count * grad_map_occ(gdtype, pe, accumulate != 0, c->rounds);
-  const int64_t most = small || a.grad_unit == kMaxGradUnitElems ? INT32_MAX : resident;
+  const bool per_unit = (small || a.grad_unit == kMaxGradUnitElems) && units >= kUnitsPerSm * c->sm_count;
+  const int64_t most = per_unit ? INT32_MAX : resident;
   const int grid = (int)std::min(units, most);
   if (a.chunk_end <= 0) return SMAT_OK;
   Timed t(c, 3, stream);

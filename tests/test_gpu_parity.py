@@ -287,6 +287,52 @@ def test_inplace_gradient_map_equals_out_of_place(gdt, alpha_mode, keep):
         sess.close()
 
 
+@pytest.mark.parametrize("gdt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("alpha_mode", [S.SMAT_ALPHA_PER_TENSOR, S.SMAT_ALPHA_PER_ELEMENT])
+@pytest.mark.parametrize("accumulate", [False, True])
+def test_gradient_map_units_equal(gdt, alpha_mode, accumulate):
+    """The map's launch has a CTA per unit from seven units per SM, else the
+    resident CTAs share the units out: on a list with more than that of 2^12 and
+    2^15 elements and fewer of 2^17, and a tensor that ends inside a unit, the
+    gradients do not depend on the chunk size, and equal the oracle's at every
+    unit's edge and random elements."""
+    dev = torch.device("cuda")
+    sms = torch.cuda.get_device_properties(dev).multi_processor_count
+    sizes = [(7 * sms + 3) * (1 << 15) + 21, 70_001]
+    gen = torch.Generator(device=dev).manual_seed(4)
+    th = [torch.randn(n, generator=gen, device=dev) * 0.02 for n in sizes]
+    sim = [torch.empty_like(t) for t in th]
+    gs = [torch.randn(n, generator=gen, device=dev).to(gdt) for n in sizes]
+    acc = [torch.randn(n, generator=gen, device=dev).to(gdt) for n in sizes]
+    bits = torch.int32 if gdt == torch.float32 else torch.int16
+    ref = None
+    for log2 in (0, 12, 15, 18):
+        sess = S.SmatSession(th, th, sim, [0.7, 0.3], [1e-3] * 2, seed=3, alpha_min=0.3, alpha_mode=alpha_mode,
+                             flags=S.SMAT_FLAG_CHUNK_LOG2(log2) if log2 else 0)
+        sess.simulate_multi(2)
+        out = [a.clone() for a in acc]
+        sess.grad_map_multi(2, gs, out, accumulate=accumulate)
+        torch.cuda.synchronize()
+        sess.close()
+        if ref is not None:
+            assert all(torch.equal(a.view(bits), b.view(bits)) for a, b in zip(ref, out)), log2
+            continue
+        ref = out
+        ogt = O.F32 if gdt == torch.float32 else O.BF16
+        cfg = O.config(seed=3, step=2, alpha_min=0.3, noise=O.NOISE_UNIFORM,
+                       alpha_mode=O.ALPHA_PER_TENSOR if alpha_mode == S.SMAT_ALPHA_PER_TENSOR else O.ALPHA_PER_ELEMENT)
+        for k, n in enumerate(sizes):
+            edges = (np.arange(0, n, 1 << 15)[:, None] + np.array([-1, 0])).reshape(-1)
+            idx = np.unique(np.concatenate([edges[edges >= 0], [n - 1],
+                                            np.random.default_rng(k).integers(0, n, 20_000)]))
+            at = torch.from_numpy(idx).to(dev)
+            want = O.gradmap_at(cfg, O.tensor(k, n, O.F32, keep_prob=[0.7, 0.3][k], sigma=1e-3), idx,
+                                to_host(gs[k][at].float()), gdtype=ogt, accumulate=accumulate,
+                                gold_vals=to_host(acc[k][at].float()))
+            got = to_host(out[k][at])
+            assert np.array_equal(got.astype(np.uint32) if ogt == O.BF16 else got.view(np.uint32), want), k
+
+
 def test_gradient_lists_refused_by_the_binding():
     """Gradients and moments that do not fit the list are refused, whichever
     tensor they belong to; separate output lists and the in-place forms (no

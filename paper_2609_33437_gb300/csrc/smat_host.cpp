@@ -398,13 +398,16 @@ int grid_for(const smat_ctx* c, int64_t chunks, int dtype) {
 // Claims of the fused AdamW launch over a's chunk range, and the split of its last
 // units (KArgs): whole units for as many full rounds of the resident CTAs as there
 // are, then up to eight pieces of at least 2^13 elements per unit, so that the CTAs
-// end together.
-int64_t split_units(KArgs& a, int64_t resident) {
-  const int64_t units = (a.chunk_end - a.chunk_begin) * (int64_t)a.grad_units;
+// end together. Two pieces alone are cut only if all of them run at once: they
+// save nothing else (1.4e7 bf16 elements, 247 units of 2^14 left for 304 CTAs: 61.5
+// us whole, 63.6 in halves).
+int64_t split_units(KArgs& a, int64_t units, int64_t resident) {
   a.grad_split = 0;
   while (a.grad_split < 3 && (a.grad_unit >> (a.grad_split + 1)) >= 2 * kMinChunkElems) a.grad_split += 1;
   a.grad_whole = units / resident * resident;
-  return std::min(a.grad_whole + ((units - a.grad_whole) << a.grad_split), int64_t(INT32_MAX));
+  const int64_t rest = units - a.grad_whole;
+  if (a.grad_split == 1 && 2 * rest > resident) a.grad_split = 0;
+  return std::min(a.grad_whole + (rest << a.grad_split), int64_t(INT32_MAX));
 }
 
 // Rows a2 + a1: delta statistics (if needed) then the per-call scalars.
@@ -811,14 +814,20 @@ smat_status smat_grad_map_adamw_multi(smat_ctx* c, uint32_t step, const void* co
     a.chunk_end = c->range_end[dt];
     if (a.chunk_end <= a.chunk_begin) continue;
     const int pdt = dt == 0 ? SMAT_F32 : SMAT_BF16;
-    // fp32 parameters take a CTA per claim (vision tower 1440 -> 1316 us, 3e8 elements
-    // 1285 -> 1214), and so do fp32 gradients of bf16 ones in units of 2^17 (0.5B decoder
-    // 1810 -> 1786); the other bf16 calls stay with the resident CTAs (2.35e8 elements
-    // with fp32 gradients in units of 2^16: 875 us with a CTA per claim, 856 resident;
-    // bf16 gradients: 1e8 359 and 354, 5.4e8 2298 and 2281).
+    // A CTA per claim for fp32 parameters with fp32 gradients from four units per SM
+    // (two rounds; us resident and per claim: 3e6 elements 20.6 and 22.1, 1e7 in 20
+    // tensors 58.4 and 54.4, 1.4e7 68.1 and 69.8, 2.8e7 128.0 and 128.5, 7e7 313 and 300,
+    // 3e8 1288 and 1213) and for units of 2^17 but bf16 with bf16 (fp32 with bf16: 2e8 774
+    // and 776, 3e8 1162 and 1147; bf16 with fp32: 3e8 flat 1066 and 1076, 100 tensors 1120
+    // and 1113, 0.5B decoder 1810 and 1786). The resident CTAs share out the claims of
+    // the others (per-element alpha, fp32: 6e7 254.7 and 260.3; bf16 with bf16: 1e8 351
+    // and 356, 6e8 2052 and 2065; fp32 with bf16, 20 tensors: 1e7 55 and 52, 4e7 167 and 170).
+    const bool f32s = pdt == SMAT_F32 && gdtype == SMAT_F32;
+    const int64_t units = (a.chunk_end - a.chunk_begin) * (int64_t)a.grad_units;
     const int64_t resident = (int64_t)c->sm_count * grad_map_adamw_occ(gdtype, pdt, pe, c->rounds);
-    const bool per_claim = pdt == SMAT_F32 || (gdtype == SMAT_F32 && a.grad_unit == kMaxGradUnitElems);
-    const int64_t claims = split_units(a, resident);
+    const bool long_units = a.grad_unit == kMaxGradUnitElems && (pdt == SMAT_F32 || gdtype == SMAT_F32);
+    const bool per_claim = long_units || (f32s && !pe && units >= 4 * (int64_t)c->sm_count);
+    const int64_t claims = split_units(a, units, resident);
     const int grid = (int)(per_claim ? claims : std::min(claims, resident));
     Timed tm(c, 3, stream);
     const cudaError_t e = launch_grad_map_adamw(a, grid, gdtype, pdt, pe, c->rounds, stream);

@@ -407,8 +407,9 @@ size_t smat_merge_workspace_bytes(const smat_merge_tensor* tensors, int32_t n_te
  * before return). d_workspace: device memory of at least
  * smat_merge_workspace_bytes bytes, 256-byte aligned, not in use by another
  * call until this one's work on `stream` has finished. TIES first selects
- * each tensor's per-expert threshold exactly (three passes of a radix
- * select over the magnitudes), then merges. */
+ * each tensor's per-expert threshold exactly: a sample gives an interval of
+ * magnitudes, and one or two counting passes over the inputs (up to four, where
+ * the sample shows other magnitudes than the rest) decide it. Then it merges. */
 smat_status smat_merge(const smat_merge_tensor* tensors, int32_t n_tensors, const smat_merge_config* cfg,
                        void* d_workspace, size_t workspace_bytes, smat_stream_t stream);
 

@@ -14,15 +14,14 @@
 // tensor, 2^12 to 2^18 elements, the size chosen per list). The forward of a
 // list without statistics has one CTA per chunk, which draws the chunk's scalars
 // itself; with statistics fused for sigma_rel tensors one CTA per item of an
-// ordered work list (by ticket); the gradient map one CTA per unit, a part of a
-// chunk; the unfused statistics, the forward beside them and the bf16 gradient map
-// of short chunks walk the table in grid-stride order. Each thread owns 16
-// consecutive elements at a time (one 256-bit load
-// per bf16 input, two per fp32 input), which is exactly one Philox block of
-// the mask stream (16 high bytes) and three blocks of the noise stream (24
-// bits per element); with the 16-bit draw option, two blocks of each. The
-// random words stay in registers; masks and noise are never written to
-// memory.
+// ordered work list (by ticket), or CTAs that walk a list whose items all run at
+// once; the gradient map one CTA per unit, a part of a chunk, where there are many;
+// the unfused statistics, the forward beside them and the other gradient maps walk
+// the table in grid-stride order. Each thread owns 16 consecutive elements at a
+// time (one 256-bit load per bf16 input, two per fp32 input), which is exactly one
+// Philox block of the mask stream (16 high bytes) and three blocks of the noise
+// stream (24 bits per element); with the 16-bit draw option, two blocks of each.
+// The random words stay in registers; masks and noise are never written to memory.
 //
 // The path is elementwise and bound by HBM bandwidth or by the integer
 // pipeline (Philox): there is no contraction, so no tensor-core work.
@@ -477,8 +476,8 @@ __device__ __forceinline__ void resolve_group_ties(const KArgs& a, uint32_t tid,
 
 // Groups with tie elements whose low 24 mask bits are drawn at the end of the
 // chunk, so the rare Philox calls run for the whole warp at once instead of
-// once per group. Up to four 16-bit group indices per thread (a chunk has
-// 4096 groups), two per register.
+// once per group. Up to four 16-bit group indices per thread (a unit has at most
+// 8192 groups: 2^17 elements), two per register.
 struct TieList {
   uint32_t w0 = 0u, w1 = 0u;
   int n = 0;

@@ -3,8 +3,8 @@
 // theta0, for weight averaging, Task Arithmetic, DARE followed by Task
 // Arithmetic and TIES (the merging methods of Sec. 5). Elementwise and bound
 // by HBM bandwidth: each element reads theta0 and the K experts once and
-// writes the result once (TIES first reads every expert once or twice more to
-// select its per-tensor trim thresholds exactly).
+// writes the result once (TIES first reads every expert once or twice more, at
+// most four times, to select its per-tensor trim thresholds exactly).
 //
 // Arithmetic, identical to the CPU oracle: Delta_j one fp32 subtraction;
 // experts accumulated in index order, one fused multiply-add each (WA 1/K,
@@ -784,7 +784,7 @@ __global__ void __launch_bounds__(kSampleThreads) ties_sample_kernel(const __gri
 // that no branch surrounds the shared-memory atomic: a pass that tested each
 // key against the digits decided so far and branched around the atomic took
 // 5.7 ms for 8 experts of 1.07e9 bf16 elements, bound by issue slots; this one
-// takes 3.4 (2.9 at HBM speed), bound by the shared-memory atomics (LSU data
+// takes 3.0 (2.9 at HBM speed), bound by the shared-memory atomics (LSU data
 // pipe 72% busy).
 //
 // bf16: a key that is not its bin's first (differences of bf16 values near

@@ -200,7 +200,7 @@ def test_workload_inventory():
 
 
 def test_merge_host_validation(L):
-    """smat_merge_workspace_bytes sizes valid lists (TIES adds the radix
+    """smat_merge_workspace_bytes sizes valid lists (TIES adds the threshold
     histograms) and returns 0 for invalid ones, without a GPU."""
     K, n = 3, 1 << 20
     exps = (ctypes.c_void_p * K)(*[0x40000000 + (k + 1) * 0x1000000 for k in range(K)])

@@ -325,11 +325,15 @@ def test_merge_ties_long_threshold_items(dtype, K):
 @pytest.mark.parametrize("sizes", [[35_000_011], [200_003] * 170])
 def test_merge_returns_before_the_work_ahead_of_it(method, sizes):
     """smat_merge is asynchronous: it returns while earlier work of the stream
-    still runs (no table of the call is long enough for its upload to wait)."""
+    still runs (no table of the call is long enough for its upload to wait), and
+    its tables are its own by then: the merge is the same."""
     t0s, exs = _experts(sizes, 2, O.F32, seed=3)
     outs = [torch.empty_like(t) for t in t0s]
     kw = dict(gamma=0.4, retention=0.3, p_drop=0.3 if method == S.SMAT_MERGE_DARE_TA else 0.0)
     S.merge(t0s, exs, outs, method, **kw)  # the workspace's first allocation
+    first = [x.clone() for x in outs]
+    for x in outs:
+        x.zero_()
     torch.cuda.synchronize()
     ahead = torch.cuda.Event()
     torch.cuda._sleep(200_000_000)  # about 0.1 s
@@ -337,3 +341,4 @@ def test_merge_returns_before_the_work_ahead_of_it(method, sizes):
     S.merge(t0s, exs, outs, method, **kw)
     assert not ahead.query()
     torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(first, outs))
